@@ -217,18 +217,17 @@ __device__ __forceinline__ void warp_slot(R (*red)[LW], int k, V v) {
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = x;
 }
 
-// Sums acc[k] over the warp for all k < MAXM at once (butterfly transpose
-// reduction: 31 shuffles per 32 slots instead of 5 per slot); lane l ends with
-// the warp total of slot l (+32 for the second half when MAXM = 64), which it
-// stores to red[warp][slot] for slot < L.
-template <int LMAX, int MAXM, typename T>
-__device__ __forceinline__ void warp_slots(T (*red)[LMAX], T (&acc)[MAXM], int L) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int g = 0; g < MAXM / 32; g++) {
-    T v[32];
-#pragma unroll
-    for (int i = 0; i < 32; i++) v[i] = acc[g * 32 + i];
+// Butterfly transpose over a warp: lane l enters with W values v[0..W-1] and
+// leaves with the warp sum of value l / (32 / W) in v[0].  Each halving step
+// exchanges half of what is left, then one addition per remaining step: W = 8
+// takes 9 shuffles and additions, 16 takes 16, 32 takes 31 (five per value one
+// by one).  Whatever W, a value's 32 summands are paired over lane distances
+// 16, 8, 4, 2, 1, so its sum does not depend on the W it was reduced with.
+template <int W, int OFF = 16, typename T, int A>
+__device__ __forceinline__ void warp_transpose_sum(T (&v)[A]) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (W == 32) {
+    // (as a loop: the recursion leaves v in local memory in the widest variant)
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) {
       const bool up = (lane & off) != 0;
@@ -239,32 +238,57 @@ __device__ __forceinline__ void warp_slots(T (*red)[LMAX], T (&acc)[MAXM], int L
         v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
       }
     }
-    const int slot = g * 32 + lane;
-    if (slot < L) red[warp][slot] = v[0];
+  } else if constexpr (OFF >= 1) {
+    constexpr int H = W > 1 ? W / 2 : 0;
+    const bool up = (lane & OFF) != 0;
+    if constexpr (H == 0) v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
+#pragma unroll
+    for (int i = 0; i < H; i++) {
+      const T send = up ? v[i] : v[i + H];
+      const T keep = up ? v[i + H] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+    }
+    warp_transpose_sum<(H > 0 ? H : 1), OFF / 2>(v);
   }
 }
 
-// warp_slots for an accumulator array of K <= MAXM entries (padded to 32).
+// Sums acc[k] over the warp for all k < K (a multiple of 8) and stores the sums
+// of slots k < L to red[warp][k]: groups of 32 slots, then 16 and 8, so that a
+// small bucket does not pay for 32 slots (padded to 32, every bucket took 31
+// additions: in FP64, where a warp addition occupies its SM quarter's pipe for
+// 64 cycles, two such butterflies per warp and pass).  With the gather's
+// four-slot butterfly: 32.2 -> 28.5 us per step at 256^2 FP64, GMRES(30), and
+// 7.45 -> 7.35 us in FP32.
 template <int LMAX, int K, typename T>
 __device__ __forceinline__ void warp_slots_k(T (*red)[LMAX], const T (&acc)[K], int L) {
+  static_assert(K % 8 == 0, "buckets are multiples of 8");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int g = 0; g < (K + 31) / 32; g++) {
+  for (int g = 0; g < K / 32; g++) {
     T v[32];
 #pragma unroll
-    for (int i = 0; i < 32; i++) v[i] = (g * 32 + i < K) ? acc[g * 32 + i] : T(0);
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-      const bool up = (lane & off) != 0;
-#pragma unroll
-      for (int i = 0; i < off; i++) {
-        const T send = up ? v[i] : v[i + off];
-        const T keep = up ? v[i + off] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-      }
-    }
+    for (int i = 0; i < 32; i++) v[i] = acc[g * 32 + i];
+    warp_transpose_sum<32>(v);
     const int slot = g * 32 + lane;
     if (slot < L) red[warp][slot] = v[0];
+  }
+  if constexpr (K & 16) {
+    constexpr int base = K / 32 * 32;
+    T v[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = acc[base + i];
+    warp_transpose_sum<16>(v);
+    const int slot = base + (lane >> 1);
+    if (slot < L && (lane & 1) == 0) red[warp][slot] = v[0];
+  }
+  if constexpr (K & 8) {
+    constexpr int base = K - 8;
+    T v[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = acc[base + i];
+    warp_transpose_sum<8>(v);
+    const int slot = base + (lane >> 2);
+    if (slot < L && (lane & 3) == 0) red[warp][slot] = v[0];
   }
 }
 
@@ -374,18 +398,23 @@ __device__ __forceinline__ void gather(const R* part, int L, int nb, double* tot
 #pragma unroll
       for (int q = 0; q < Q; q++) s[q] += (v[q][0] + v[q][1]) + (v[q][2] + v[q][3]);
     }
-#pragma unroll
-    for (int q = 0; q < Q; q++) s[q] = warp_sum(s[q]);
-    if (lane == 0) {
-#pragma unroll
-      for (int q = 0; q < Q; q++) {
-        const int k = k0 + q * NW;
-        if (k < L) {
-          // FP32 partials: coef only (an FP64 conversion is a long-latency
-          // operation on this GPU; consumers convert where they need FP64)
-          if constexpr (sizeof(R) == 8) tot[k] = (double)s[q];
-          coef[k] = (T)s[q];
-        }
+    // four slots by one butterfly transpose (6 shuffles and additions instead
+    // of 20), the fifth on its own; lane 8 q ends with the sum of slot q
+    warp_transpose_sum<4>(s);
+    if constexpr (Q == 5) s[4] = warp_sum(s[4]);
+    const int q = lane >> 3;
+    const int k = k0 + q * NW;
+    if ((lane & 7) == 0 && k < L) {
+      // FP32 partials: coef only (an FP64 conversion is a long-latency
+      // operation on this GPU; consumers convert where they need FP64)
+      if constexpr (sizeof(R) == 8) tot[k] = (double)s[0];
+      coef[k] = (T)s[0];
+    }
+    if constexpr (Q == 5) {
+      const int k4 = k0 + 4 * NW;
+      if (lane == 1 && k4 < L) {
+        if constexpr (sizeof(R) == 8) tot[k4] = (double)s[4];
+        coef[k4] = (T)s[4];
       }
     }
   }
