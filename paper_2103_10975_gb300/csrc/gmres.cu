@@ -29,6 +29,7 @@ int own_bytes_f2c();
 cudaError_t launch_gmres_f3c(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f2cs(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f2s32(const KParams& kp, int grid, cudaStream_t s);
+cudaError_t launch_gmres_d2s32(const KParams& kp, int grid, cudaStream_t s);
 int max_blocks_f3c(int* bs, int extra);
 int own_bytes_f3c();
 
@@ -90,7 +91,8 @@ cudaError_t launch_gmres(const KParams& kp, bool fp32, int dim, int grid, cudaSt
     return launch_gmres_f3d(kp, grid, s);
   }
   if (dim == 2) {
-    if (kp.vmode == kVShared) return launch_gmres_d2s(kp, grid, s);
+    if (kp.vmode == kVShared)
+      return kp.m <= kSmallM ? launch_gmres_d2s32(kp, grid, s) : launch_gmres_d2s(kp, grid, s);
     if (kp.vmode == kVBulk) return launch_gmres_d2b(kp, grid, s);
     return launch_gmres_d2d(kp, grid, s);
   }
@@ -123,12 +125,13 @@ int gmres_bulk_stages(bool fp32, int m) {
   return gmres_bulk_cap(fp32, m, kMaxStages) > 0 ? kMaxStages : 0;
 }
 
-int gmres_vsmem_budget(bool fp32) {
+int gmres_vsmem_budget(bool fp32, int m) {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int own = fp32 ? (int)smem_own_bytes<float, kMaxM, 256>()
-                       : (int)smem_own_bytes<double, kMaxM, 256>();
+  const int own = fp32           ? (int)smem_own_bytes<float, kMaxM, 256>()
+                  : m <= kSmallM ? (int)smem_own_bytes<double, kSmallM, 256>()
+                                 : (int)smem_own_bytes<double, kMaxM, 256>();
   const int left = optin - own - 1024;
   return left > 0 ? left : 0;
 }

@@ -396,7 +396,20 @@ __device__ __forceinline__ void gather(const R* part, int L, int nb, double* tot
         }
       }
 #pragma unroll
-      for (int q = 0; q < Q; q++) s[q] += (v[q][0] + v[q][1]) + (v[q][2] + v[q][3]);
+      for (int q = 0; q < Q; q++) {
+        if constexpr (sizeof(R) == 8) {
+          // FP64: an addition occupies the pipe for 64 cycles per warp, so the
+          // slots past L and the quarters past nb are left out (uniform tests)
+          if (k0 + q * NW < L) {
+            R a = v[q][0];
+            if (nb - g0 > 32) a += v[q][1];
+            if (nb - g0 > 64) a += v[q][2] + v[q][3];
+            s[q] = g0 == 0 ? a : s[q] + a;
+          }
+        } else {
+          s[q] += (v[q][0] + v[q][1]) + (v[q][2] + v[q][3]);
+        }
+      }
     }
     // four slots by one butterfly transpose (6 shuffles and additions instead
     // of 20), the fifth on its own; lane 8 q ends with the sum of slot q
@@ -1757,8 +1770,17 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
       // c_{j+1} = Hu(j+1,j) h2_j, the new vector's own coefficient
       auto set_norm = [&]() {
         const T h2v = sm.hn2T > T(0) ? sm.hn2T : T(0);
-        const T hnT = sqrt(h2v);
-        sm.invT = T(1) / hnT;
+        T hnT;
+        if (sizeof(T) == 8 && h2v > T(1e-290) && h2v < T(1e290)) {
+          // FP64: one reciprocal square root instead of a square root and a
+          // division (dependent chains of ~680 and ~430 cycles on this GPU)
+          const T inv = rsqrt(h2v);
+          hnT = h2v * inv;
+          sm.invT = inv;
+        } else {
+          hnT = sqrt(h2v);
+          sm.invT = T(1) / hnT;
+        }
         sm.HuT[j + 1 + j * LD] = hnT;  // (the Givens warp reads it in FP64)
         sm.cv[j + 1] = hnT * sm.coef[j];
       };
@@ -1790,14 +1812,25 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
         const int ir = min(i, j);
         const int k0 = (ir > 0 ? ir - 1 : 0) + sub;
         T c = T(0);
-        // all loads of a lane issued together (indices clamped into the column range)
+        if constexpr (sizeof(T) == 8) {
+          // FP64: only the products that exist (a warp FMA occupies its SM
+          // quarter's pipe for 64 cycles), column j's by the row's first lane.
+          // With the gather's tests, the norm's rsqrt and the m <= 32 variant:
+          // 28.5 -> 26.8 us per step at 256^2, GMRES(30)
+          if (i <= j) {
+            if (sub == 0) c = (sm.h1c[i] + sm.coef[i]) * sm.coef[j];
+            for (int k = k0; k < j; k += 8) c = fma(sm.HuT[i + k * LD], sm.coef[k], c);
+          }
+        } else {
+          // all loads of a lane issued together (indices clamped into the column range)
 #pragma unroll
-        for (int t = 0; t < (MAXM + 7) / 8; t++) {
-          const int k = k0 + 8 * t;
-          const int kk = min(k, j);
-          const T hik = kk == j ? sm.h1c[ir] + sm.coef[ir] : sm.HuT[ir + kk * LD];
-          const T prod = hik * sm.coef[kk];
-          if (i <= j && k <= j) c += prod;
+          for (int t = 0; t < (MAXM + 7) / 8; t++) {
+            const int k = k0 + 8 * t;
+            const int kk = min(k, j);
+            const T hik = kk == j ? sm.h1c[ir] + sm.coef[ir] : sm.HuT[ir + kk * LD];
+            const T prod = hik * sm.coef[kk];
+            if (i <= j && k <= j) c += prod;
+          }
         }
         c += __shfl_xor_sync(0xffffffffu, c, 4);
         c += __shfl_xor_sync(0xffffffffu, c, 2);

@@ -61,7 +61,31 @@ unsigned long long splitmix_next(unsigned long long& st) {
   return z ^ (z >> 31);
 }
 
+// Shared-memory bytes of a single solve's V slice at `blocks` CTAs (0 if the
+// slice does not fit).
+int single_vsmem(const mlgmres* h, int blocks, bool compact = false) {
+  const long long chunk = (((long long)h->N + blocks - 1) / blocks + 31) / 32 * 32;
+  const long long need = chunk * vrows_p(h->opt.m + 1) * (h->fp32 ? 4 : 8);
+  const int budget = compact ? (h->grid.dim == 2 ? gmres_compact_vsmem_budget() : 0)
+                             : gmres_vsmem_budget(h->fp32, h->opt.m);
+  return need <= budget ? (int)need : 0;
+}
+
 int auto_blocks(const mlgmres* h, int N) {
+  if (!h->fp32 && h->grid.dim == 2) {
+    // FP64: a warp FMA occupies its SM quarter's FP64 pipe for 64 cycles, so the
+    // step is bound by the tiles per SM quarter: the fewest tiles per CTA the
+    // co-resident CTAs allow, rounded up to whole tiles per quarter (32^2,
+    // GMRES(20): 8 CTAs of 4 tiles, 14.2 us per step, where 2 CTAs of 16 took
+    // 24.3; 128^2: 16.8 against 28.3; 256^2 stays at 128 CTAs of 16: 152 CTAs of
+    // 14 have as many per quarter and took 33.3 against 32.2)
+    const int tiles = (N + 31) / 32;
+    const int per = (tiles + h->max_blocks - 1) / h->max_blocks;
+    for (int t : {(per + 3) / 4 * 4, per}) {
+      const int nb = (tiles + t - 1) / t;
+      if (single_vsmem(h, nb) > 0) return nb;  // V in shared memory
+    }
+  }
   // about 512 grid points per CTA (two per thread): measured on GB300 at 256^2,
   // 128 CTAs take 18 us per Arnoldi step against 26 us with 64 and 43 us with 32;
   // never more CTAs than can be co-resident
@@ -233,16 +257,6 @@ int use_compact(const mlgmres* h) {
   if (h->opt.compact == 0) return 0;
   if (h->opt.compact == 1) return 1;
   return h->tuned_compact;
-}
-
-// Shared-memory bytes of a single solve's V slice at `blocks` CTAs (0 if the
-// slice does not fit).
-int single_vsmem(const mlgmres* h, int blocks, bool compact = false) {
-  const long long chunk = (((long long)h->N + blocks - 1) / blocks + 31) / 32 * 32;
-  const long long need = chunk * vrows_p(h->opt.m + 1) * (h->fp32 ? 4 : 8);
-  const int budget = compact ? (h->grid.dim == 2 ? gmres_compact_vsmem_budget() : 0)
-                             : gmres_vsmem_budget(h->fp32);
-  return need <= budget ? (int)need : 0;
 }
 
 // Run the persistent kernel for `count` tasks already staged in h->htasks,
@@ -901,7 +915,7 @@ mlgmres_status mlgmres_solve_batch(mlgmres_t h, int count, const mlgmres_grid* g
         const long long chunk = ((N + k - 1) / k + 31) / 32 * 32;
         need = std::max(need, chunk * vrows_p(h->opt.m + 1) * (long long)es0);
       }
-      return need <= gmres_vsmem_budget(h->fp32) ? (int)need : 0;
+      return need <= gmres_vsmem_budget(h->fp32, h->opt.m) ? (int)need : 0;
     };
     // one CTA per SM first; if the basis streams from HBM anyway, the compact
     // variant (two CTAs per SM) gets all the reserved CTAs

@@ -11,8 +11,8 @@ constexpr int kMaxM = 64;          // largest supported restart length
 // bucket limits of the compact (2 CTAs per SM) variants: m <= 47 (2D), m <= 55 (3D)
 constexpr int kCompactM2 = 48;
 constexpr int kCompactM3 = 56;
-// restart lengths up to which the FP32 2D shared-slice variant runs its m <= 32
-// instantiation (fewer buckets of j, less code)
+// restart lengths up to which the 2D shared-slice variants run their m <= 32
+// instantiations (fewer buckets of j, less code, a smaller shared state)
 constexpr int kSmallM = 32;
 // Where a launch keeps the basis V (one kernel variant each):
 constexpr int kVDirect = 0;  // HBM, loaded into registers by the passes
@@ -101,8 +101,9 @@ cudaError_t launch_gmres(const KParams& kp, bool fp32, int dim, int grid_blocks,
 int gmres_max_blocks(bool fp32, int dim, int m, int* block_threads);
 
 // Shared-memory bytes a CTA may use for its slice of V (so that slice + the
-// solver's own state fit the per-CTA limit); 0 if none.
-int gmres_vsmem_budget(bool fp32);
+// solver's own state fit the per-CTA limit); 0 if none.  The FP64 variant for
+// m <= kSmallM has a smaller state and so a larger budget.
+int gmres_vsmem_budget(bool fp32, int m = kMaxM);
 
 // Most bulk-copy stages per warp (kMaxStages) for a basis in HBM.  A pass uses
 // as many as fit in a warp's staging area for its rows.
