@@ -145,31 +145,42 @@ __global__ void apply_kernel(int n, int N, const float* kappa, const double* u, 
   out[i] = stencil<double, DIM>(u, i, n, kappa, u[i]) / (h * h);
 }
 
+// One pass per solve: about N (4 + 24 + 16) bytes, against six FP64 divisions
+// per point in every restart residual (192^3: the restart took 1.0 ms of FP64
+// pipe per cycle) and, in FP64, in every Arnoldi step.
 __global__ void kappa_faces_kernel(int n, int N, const float* __restrict__ kappa,
-                                   float* __restrict__ faces, long long fstride) {
+                                   float* __restrict__ faces, long long fstride,
+                                   double* __restrict__ faces64, long long f64stride) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const int nn = n * n;
   const int ix = i % n, iy = (i / n) % n, iz = i / nn;
   const double kc = kappa[i];
-  // the harmonic mean in FP64, rounded once to FP32
+  // the harmonic mean in FP64 (the passes' FP32 copy is rounded once)
   auto hm = [&](int j) {
     const double kn = kappa[j];
-    return (float)(2.0 * kc * kn / (kc + kn));
+    return 2.0 * kc * kn / (kc + kn);
   };
-  faces[i] = ix < n - 1 ? hm(i + 1) : 0.f;
-  faces[fstride + i] = iy < n - 1 ? hm(i + n) : 0.f;
-  faces[2 * fstride + i] = iz < n - 1 ? hm(i + nn) : 0.f;
+  const double fx = ix < n - 1 ? hm(i + 1) : 0.0;
+  const double fy = iy < n - 1 ? hm(i + n) : 0.0;
+  const double fz = iz < n - 1 ? hm(i + nn) : 0.0;
+  faces64[i] = fx;
+  faces64[f64stride + i] = fy;
+  faces64[2 * f64stride + i] = fz;
+  if (!faces) return;
+  faces[i] = (float)fx;
+  faces[fstride + i] = (float)fy;
+  faces[2 * fstride + i] = (float)fz;
   const int walls = (ix == 0) + (ix == n - 1) + (iy == 0) + (iy == n - 1) + (iz == 0) + (iz == n - 1);
   faces[3 * fstride + i] = (float)(kc * walls);
 }
 
 cudaError_t launch_kappa_faces(int n, const float* kappa, float* faces, long long fstride,
-                               cudaStream_t s) {
+                               double* faces64, long long f64stride, cudaStream_t s) {
   const int N = n * n * n;
   const int bs = 256, gr = (N + bs - 1) / bs;
   note_launches(1);
-  kappa_faces_kernel<<<gr, bs, 0, s>>>(n, N, kappa, faces, fstride);
+  kappa_faces_kernel<<<gr, bs, 0, s>>>(n, N, kappa, faces, fstride, faces64, f64stride);
   return cudaGetLastError();
 }
 

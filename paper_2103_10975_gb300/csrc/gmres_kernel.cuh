@@ -81,6 +81,39 @@ __device__ __forceinline__ T stencil3d(const T* __restrict__ u, int i, int n,
   return acc;
 }
 
+// The 3D operator from face coefficients formed once per solve: fx, fy,
+// fz at faces + a * fs hold the harmonic mean of a point's kappa and its +x, +y,
+// +z neighbour's, so the -x, -y, -z faces are the entries of i-1, i-n, i-n^2.
+// The same face values (2 kc knb / (kc + knb) rounds alike from either side),
+// faces and order as stencil3d, without its six FP64 divisions per point (~15
+// dependent FP64 instructions each): 41^3 FP64, GMRES(30), 45.0 -> 32.1 us per
+// step; 192^3 FP32, GMRES(50), 354.4 -> 329.6 us per step through the restart
+// residual alone.
+template <typename T>
+__device__ __forceinline__ T stencil3d_faces(const T* __restrict__ u, int i, int n,
+                                             const float* __restrict__ kappa,
+                                             const T* __restrict__ faces, long long fs, T uc) {
+  const int ix = i % n;
+  const int t = i / n;
+  const int iy = t % n;
+  const int iz = t / n;
+  const int nn = n * n;
+  const int off[6] = {-1, 1, -n, n, -nn, nn};
+  const bool has[6] = {ix > 0, ix < n - 1, iy > 0, iy < n - 1, iz > 0, iz < n - 1};
+  const T kc = (T)__ldg(kappa + i);
+  T acc = T(0);
+#pragma unroll
+  for (int f = 0; f < 6; f++) {
+    if (has[f]) {
+      const T kf = __ldg(faces + (f >> 1) * fs + i + ((f & 1) ? 0 : off[f]));
+      acc += kf * (uc - ldcg(u + i + off[f]));
+    } else {
+      acc += kc * uc;
+    }
+  }
+  return acc;
+}
+
 template <typename T, int DIM>
 __device__ __forceinline__ T stencil(const T* __restrict__ u, int i, int n,
                                      const float* __restrict__ kappa, T uc) {
@@ -88,6 +121,29 @@ __device__ __forceinline__ T stencil(const T* __restrict__ u, int i, int n,
     return stencil2d<T>(u, i, n, uc);
   else
     return stencil3d<T>(u, i, n, kappa, uc);
+}
+
+// The operator in FP64 at one point of a task's grid (face coefficients where
+// the task has them).
+template <int DIM>
+__device__ __forceinline__ double stencil64(const SolveTask& tk, const double* __restrict__ u,
+                                            int i, double uc) {
+  if constexpr (DIM == 3)
+    if (tk.faces64) return stencil3d_faces<double>(u, i, tk.n, tk.kappa, tk.faces64, tk.f64stride, uc);
+  return stencil<double, DIM>(u, i, tk.n, tk.kappa, uc);
+}
+
+// The same in the working precision (FP64 face coefficients serve FP64 only).
+template <typename T, int DIM>
+__device__ __forceinline__ T stencil_any(const SolveTask& tk, const T* __restrict__ u, int i,
+                                         T uc) {
+  if constexpr (sizeof(T) == 8)
+    return stencil64<DIM>(tk, u, i, uc);
+  else if constexpr (DIM == 3)
+    return tk.faces ? stencil3d_faces(u, i, tk.n, tk.kappa, tk.faces, tk.fstride, uc)
+                    : stencil<T, DIM>(u, i, tk.n, tk.kappa, uc);
+  else
+    return stencil<T, DIM>(u, i, tk.n, tk.kappa, uc);
 }
 
 // Two values side by side: two basis vectors at one point, or the coefficients
@@ -622,7 +678,7 @@ template <typename T, int DIM, int MAXM, int BS, int K>
 __device__ __forceinline__ void x_pass(Smem<T, MAXM, BS>& sm, int lo, int hi, int j, int n,
                                        const T* __restrict__ WP, T* __restrict__ Z,
                                        T* __restrict__ V, int rows, int voff,
-                                       const float* __restrict__ kappa, T s2t) {
+                                       const SolveTask& tk, T s2t) {
   constexpr int LMAX = MAXM + 2;
   constexpr int U = PointsPerTrip<T, K>::value;
   const int tid = threadIdx.x;
@@ -655,7 +711,7 @@ __device__ __forceinline__ void x_pass(Smem<T, MAXM, BS>& sm, int lo, int hi, in
     }
 #pragma unroll
     for (int u = 0; u < U; u++)
-      znum[u] = ok_[u] ? s2t * stencil<T, DIM>(WP, ii[u], n, kappa, wp[u]) : T(0);
+      znum[u] = ok_[u] ? s2t * stencil_any<T, DIM>(tk, WP, ii[u], wp[u]) : T(0);
     // sum_k h2_k v_k and sum_k c_k v_k with even and odd k apart, in the order
     // of the paired passes (x_proj), so that every placement of V rounds alike
     T sv[U][2], sz[U][2];
@@ -883,31 +939,52 @@ __device__ __forceinline__ void warp_slots_k2(T (*red)[LMAX],
 // memory twice (update, then dots) instead of being held in registers, so
 // registers only carry the accumulators; U points per trip keep the
 // stencil's global loads in flight together.
-// What a thread carries between the passes of the shared-slice 2D variant for
-// its first U = 2 points: w' at each point and its four neighbours, loaded
-// right after the Y barrier so that the loads are in flight while the CTA
-// gathers h2 and runs the scalar recurrences; and z from the X pass, which the
-// Y pass of the same step needs at the same points (no reload through L2).
-template <typename T>
+// What a thread carries between the passes of the shared-slice variants for
+// its first U = 2 points: w' at each point and its 2 DIM neighbours (0 outside
+// the grid), loaded right after the Y barrier so that the loads are in flight
+// while the CTA gathers h2 and runs the scalar recurrences, and in 3D the face
+// coefficients with them (constant: L1 hits); and z from the X pass, which the Y
+// pass of the same step needs at the same points (no reload through L2).
+template <typename T, int DIM>
 struct XCarry {
-  T c[2], l[2], r[2], d[2], t[2];
+  T c[2], nb[2][2 * DIM];
+  T kf[2][DIM == 3 ? 6 : 1];
   T z[2];
   bool pre;  // the w' values are those the next X pass needs
 };
 
-template <typename T, int BS>
-__device__ __forceinline__ void prefetch_x2d(XCarry<T>& cy, const T* __restrict__ WP, int lo,
-                                             int hi, int n) {
+template <typename T, int DIM, int BS>
+__device__ __forceinline__ void prefetch_x(XCarry<T, DIM>& cy, const SolveTask& tk,
+                                           const T* __restrict__ WP, int lo, int hi, int n) {
 #pragma unroll
   for (int u = 0; u < 2; u++) {
     const int i = lo + (int)threadIdx.x + u * BS;
     const bool ok = i < hi;
-    const int ix = i % n, iy = i / n;
     cy.c[u] = ok ? ldcg(WP + i) : T(0);
-    cy.l[u] = ok && ix > 0 ? ldcg(WP + i - 1) : T(0);
-    cy.r[u] = ok && ix < n - 1 ? ldcg(WP + i + 1) : T(0);
-    cy.d[u] = ok && iy > 0 ? ldcg(WP + i - n) : T(0);
-    cy.t[u] = ok && iy < n - 1 ? ldcg(WP + i + n) : T(0);
+    const int ix = i % n;
+    const int iy = DIM == 3 ? (i / n) % n : i / n;
+    const int iz = DIM == 3 ? i / (n * n) : 0;
+    const int off[6] = {-1, 1, -n, n, -n * n, n * n};
+    const bool has[6] = {ix > 0, ix < n - 1, iy > 0, iy < n - 1, iz > 0, iz < n - 1};
+#pragma unroll
+    for (int f = 0; f < 2 * DIM; f++) cy.nb[u][f] = ok && has[f] ? ldcg(WP + i + off[f]) : T(0);
+    if constexpr (DIM == 3) {
+      // a wall face: kappa of the point itself, against u = 0
+      if (tk.kappa && ok) {
+        const T kc = (T)__ldg(tk.kappa + i);
+#pragma unroll
+        for (int f = 0; f < 6; f++) {
+          const int at = i + ((f & 1) ? 0 : off[f]);
+          if constexpr (sizeof(T) == 8)
+            cy.kf[u][f] = has[f] ? __ldg(tk.faces64 + (f >> 1) * tk.f64stride + at) : kc;
+          else
+            cy.kf[u][f] = has[f] ? __ldg(tk.faces + (f >> 1) * tk.fstride + at) : kc;
+        }
+      } else {
+#pragma unroll
+        for (int f = 0; f < 6; f++) cy.kf[u][f] = T(1);
+      }
+    }
   }
   cy.pre = true;
 }
@@ -915,10 +992,8 @@ __device__ __forceinline__ void prefetch_x2d(XCarry<T>& cy, const T* __restrict_
 template <typename T, int DIM, int MAXM, int BS, int K>
 __device__ __forceinline__ void x_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi, int j, int n,
                                           const T* __restrict__ WP, T* __restrict__ Z,
-                                          T* __restrict__ Vs, int rows,
-                                          const float* __restrict__ kappa, T s2t,
-                                          XCarry<T>& cy) {
-  static_assert(DIM == 2, "shared-memory slices are a 2D variant");
+                                          T* __restrict__ Vs, int rows, const SolveTask& tk,
+                                          T s2t, XCarry<T, DIM>& cy) {
   constexpr int LMAX = MAXM + 2;
   using T2 = typename Vec2<T>::type;
   const int tid = threadIdx.x;
@@ -946,16 +1021,24 @@ __device__ __forceinline__ void x_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi,
   for (int i = lo + tid; i < hi; i += BS, t++) {
     T wp, znum;
     if (t < 2 && cy.pre) {
-      // the same differences, in the same order, as stencil2d
+      // the same differences, in the same order, as stencil2d / stencil3d
       const bool s1 = t == 1;
       const T uc = s1 ? cy.c[1] : cy.c[0];
-      const T l = s1 ? cy.l[1] : cy.l[0], r = s1 ? cy.r[1] : cy.r[0];
-      const T d = s1 ? cy.d[1] : cy.d[0], tp = s1 ? cy.t[1] : cy.t[0];
+      T d[2 * DIM];
+#pragma unroll
+      for (int f = 0; f < 2 * DIM; f++) d[f] = uc - (s1 ? cy.nb[1][f] : cy.nb[0][f]);
       wp = uc;
-      znum = s2t * (((uc - l) + (uc - r)) + ((uc - d) + (uc - tp)));
+      if constexpr (DIM == 2) {
+        znum = s2t * ((d[0] + d[1]) + (d[2] + d[3]));
+      } else {
+        T acc3 = T(0);
+#pragma unroll
+        for (int f = 0; f < 6; f++) acc3 += (s1 ? cy.kf[1][f] : cy.kf[0][f]) * d[f];
+        znum = s2t * acc3;
+      }
     } else {
       wp = ldcg(WP + i);
-      znum = s2t * stencil<T, DIM>(WP, i, n, kappa, wp);
+      znum = s2t * stencil_any<T, DIM>(tk, WP, i, wp);
     }
     const T* vc = Vs + vbase(i - lo, rows);
     T sv, sz;
@@ -989,11 +1072,11 @@ __device__ __forceinline__ void x_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi,
   warp_slot<LMAX>(sm.red, j + 1, accZ);
 }
 
-template <typename T, int MAXM, int BS, int K>
+template <typename T, int DIM, int MAXM, int BS, int K>
 __device__ __forceinline__ void y_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi, int j,
                                           T* __restrict__ WP, const T* __restrict__ Z,
                                           const T* __restrict__ Vs, int rows,
-                                          const XCarry<T>& cy) {
+                                          const XCarry<T, DIM>& cy) {
   constexpr int LMAX = MAXM + 2;
   using T2 = typename Vec2<T>::type;
   const int tid = threadIdx.x;
@@ -1125,6 +1208,8 @@ struct AuxSrc {  // what the X pass's stages copy besides V
   const float* kap;     // kappa (3D), or null when it is not staged
   const float* fc;      // face coefficients (3D, FP32; w' padded), or null
   long long fs;         // their array stride
+  const double* f64;    // FP64 face coefficients (3D, FP64), or null
+  long long f64s;       // their array stride
   int n;
   long long N, ldv;
 };
@@ -1278,7 +1363,8 @@ __device__ __forceinline__ T stencil_faces(const T* aw, const float* af, int i0,
 template <typename T, int DIM>
 __device__ __forceinline__ T stencil_staged(const T* aw, const float* ak,
                                             const float* __restrict__ kappa, int i, int i0,
-                                            int lane, int n, int ix, int iy, int iz) {
+                                            int lane, int n, int ix, int iy, int iz,
+                                            const AuxSrc& aux) {
   using A = Aux<T, DIM>;
   constexpr int ALN = 16 / (int)sizeof(T);
   const T uc = aw[4 + lane];
@@ -1298,7 +1384,20 @@ __device__ __forceinline__ T stencil_staged(const T* aw, const float* ak,
   } else {
     const int nn = n * n;
     T acc = T(0);
-    if (kappa) {
+    if (sizeof(T) == 8 && aux.f64) {
+      // FP64 face coefficients, formed once per solve (as stencil3d_faces)
+      const T kc = (T)__ldg(kappa + i);
+#pragma unroll
+      for (int f = 0; f < 6; f++) {
+        const bool has = f == 0 ? ix > 0 : f == 1 ? ix < n - 1 : f == 2 ? iy > 0
+                       : f == 3 ? iy < n - 1 : f == 4 ? iz > 0 : iz < n - 1;
+        const int off = f == 0 ? -1 : (f == 2 ? -n : (f == 4 ? -nn : 0));
+        if (has)
+          acc += (T)__ldg(aux.f64 + (f >> 1) * aux.f64s + i + off) * (uc - wnb(f));
+        else
+          acc += kc * uc;
+      }
+    } else if (kappa) {
       auto knbf = [&](int f) -> T {
         const int off = f == 0 ? -1 : (f == 1 ? 1 : (f == 2 ? -n : (f == 3 ? n : (f == 4 ? -nn : nn))));
         if (!ak) return (T)__ldg(kappa + i + off);
@@ -1397,9 +1496,9 @@ __device__ __forceinline__ void x_pass_bulk(Smem<T, MAXM, BS>& sm, int lo, int h
       if (af)
         znum = ok ? s2t * stencil_faces<T>(aw, af, i0, lane, n) : T(0);
       else
-        znum = ok ? s2t * stencil_staged<T, DIM>(aw, ak, kappa, i, i0, lane, n, px, py, pz) : T(0);
+        znum = ok ? s2t * stencil_staged<T, DIM>(aw, ak, kappa, i, i0, lane, n, px, py, pz, aux) : T(0);
     } else {
-      znum = ok ? s2t * stencil_staged<T, DIM>(aw, ak, kappa, i, i0, lane, n, px, py, pz) : T(0);
+      znum = ok ? s2t * stencil_staged<T, DIM>(aw, ak, kappa, i, i0, lane, n, px, py, pz, aux) : T(0);
     }
     if (DIM == 3 && !af) {
       px += NW * 32;  // the next trip's point
@@ -1563,6 +1662,9 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
   // face coefficients: the FP32 3D passes only (the FP64 ones keep FP64 faces)
   auxs.fc = (DIM == 3 && sizeof(T) == 4) ? tk.faces : nullptr;
   auxs.fs = tk.fstride;
+  auxs.f64 = (DIM == 3 && sizeof(T) == 8) ? tk.faces64 : nullptr;
+  auxs.f64s = tk.f64stride;
+  if (auxs.f64) auxs.kap = nullptr;  // kappa is then read at wall faces only
   auxs.n = n;
   auxs.N = N;
   auxs.ldv = w.ldv;
@@ -1606,9 +1708,9 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
       if (tk.zero_x) tk.x[i] = 0.0;
       if (alt) {
         const double xc = ldcg(tk.x + i);
-        const double r0 = bi - s2 * stencil<double, DIM>(tk.x, i, n, kappa, xc);
+        const double r0 = bi - s2 * stencil64<DIM>(tk, tk.x, i, xc);
         const double ac = ldcg(tk.x_alt + i);
-        const double r1 = bi - s2 * stencil<double, DIM>(tk.x_alt, i, n, kappa, ac);
+        const double r1 = bi - s2 * stencil64<DIM>(tk, tk.x_alt, i, ac);
         v1 += r0 * r0;
         v2 += r1 * r1;
       }
@@ -1654,7 +1756,7 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
           ri = tk.b[i];
         } else {
           const double xc = ldcg(tk.x + i);
-          ri = tk.b[i] - s2 * stencil<double, DIM>(tk.x, i, n, kappa, xc);
+          ri = tk.b[i] - s2 * stencil64<DIM>(tk, tk.x, i, xc);
         }
         WP[i] = (T)ri;
         v0 += ri * ri;
@@ -1693,14 +1795,14 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
     double* hist = (lb == 0) ? tk.hist : nullptr;
     int kcols = 0;
     const int jmax = arnoldi ? kp.arnoldi_steps : m;
-    XCarry<T> cy;  // shared-slice variant: values carried between its passes
+    XCarry<T, DIM> cy;  // shared-slice variants: values carried between its passes
     cy.pre = false;
     for (int j = 0;; j++) {
       // ---- X: v_j and z = A v_j, h1 = V^T z; warp 1 rotates column j-1
       // while thread 0 waits at the group barrier
       {
-#define MLG_X(KK) x_pass<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vg, rows, 0, kappa, s2t)
-#define MLG_XS(KK) x_pass_sm<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vs, rows, kappa, s2t, cy)
+#define MLG_X(KK) x_pass<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vg, rows, 0, tk, s2t)
+#define MLG_XS(KK) x_pass_sm<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vs, rows, tk, s2t, cy)
 #define MLG_XB(KK)                                                                       \
   x_pass_bulk<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vg, rows, kappa, s2t, pipe, bphase, \
                                     auxs)
@@ -1736,7 +1838,7 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
       // ---- Y: w'_{j+1} = z - V h1, h2 = V^T w'_{j+1}, ||w'_{j+1}||^2
       {
 #define MLG_Y(KK) y_pass<T, MAXM, BS, KK>(sm, lo, hi, j, WP, Z, Vg, rows, 0)
-#define MLG_YS(KK) y_pass_sm<T, MAXM, BS, KK>(sm, lo, hi, j, WP, Z, Vs, rows, cy)
+#define MLG_YS(KK) y_pass_sm<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, WP, Z, Vs, rows, cy)
 #define MLG_YB(KK) \
   y_pass_bulk<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, WP, Z, Vg, rows, pipe, bphase, w.ldv)
         if constexpr (VM == kVShared) {
@@ -1753,7 +1855,7 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
                                           &sm.flag, NoSide());
         if (!ok) goto abort;
         // w' is final everywhere: the next X pass's loads go out before the gather
-        if constexpr (VM == kVShared) prefetch_x2d<T, BS>(cy, WP, lo, hi, n);
+        if constexpr (VM == kVShared) prefetch_x<T, DIM, BS>(cy, tk, WP, lo, hi, n);
         gather<BS, T, T>((const T*)part(), j + 2, nb, sm.tot, sm.coef, ps);
         red++;
       }

@@ -32,6 +32,7 @@ struct mlgmres {
   void* W0_alloc = nullptr;  // W0's allocation (W0 may start past a zero pad)
   float* faces = nullptr;    // FP32 face coefficients (single 3D FP32 solves with kappa)
   long long fstride = 0;     // their array stride
+  double* faces64 = nullptr; // FP64 face coefficients (single 3D solves with kappa), stride ldv
   double* part = nullptr;
   double* Rg = nullptr;      // compact variants' triangles R (rg_blocks of them)
   int rg_blocks = 0;

@@ -64,6 +64,7 @@ unsigned long long splitmix_next(unsigned long long& st) {
 // Shared-memory bytes of a single solve's V slice at `blocks` CTAs (0 if the
 // slice does not fit).
 int single_vsmem(const mlgmres* h, int blocks, bool compact = false) {
+  if (h->grid.dim == 3) return 0;
   const long long chunk = (((long long)h->N + blocks - 1) / blocks + 31) / 32 * 32;
   const long long need = chunk * vrows_p(h->opt.m + 1) * (h->fp32 ? 4 : 8);
   const int budget = compact ? (h->grid.dim == 2 ? gmres_compact_vsmem_budget() : 0)
@@ -75,10 +76,8 @@ int auto_blocks(const mlgmres* h, int N) {
   if (!h->fp32 && h->grid.dim == 2) {
     // FP64: a warp FMA occupies its SM quarter's FP64 pipe for 64 cycles, so the
     // step is bound by the tiles per SM quarter: the fewest tiles per CTA the
-    // co-resident CTAs allow, rounded up to whole tiles per quarter (32^2,
-    // GMRES(20): 8 CTAs of 4 tiles, 14.2 us per step, where 2 CTAs of 16 took
-    // 24.3; 128^2: 16.8 against 28.3; 256^2 stays at 128 CTAs of 16: 152 CTAs of
-    // 14 have as many per quarter and took 33.3 against 32.2)
+    // co-resident CTAs allow, rounded up to whole tiles per quarter (32^2: 8
+    // CTAs of 4 tiles instead of 2 of 16; 256^2: 128 CTAs of 16)
     const int tiles = (N + 31) / 32;
     const int per = (tiles + h->max_blocks - 1) / h->max_blocks;
     for (int t : {(per + 3) / 4 * 4, per}) {
@@ -281,10 +280,10 @@ void run_solver(mlgmres* h, int ngroups, int ntasks, int grid, int arnoldi_steps
   kp.bulk_stages = stages >= 0 ? stages : effective_stages(h);
   kp.bulk_cap = gmres_bulk_cap(h->fp32, h->opt.m, kp.bulk_stages);
   if (kp.bulk_cap == 0) kp.bulk_stages = 0;
-  // placement of V: shared-memory slices when every task's slice fits (2D),
+  // placement of V: shared-memory slices when every task's slice fits,
   // else bulk-copy stages, else direct loads
   kp.vmode = kVDirect;
-  if (kp.vsmem > 0 && h->grid.dim == 2) kp.vmode = kVShared;
+  if (kp.vsmem > 0) kp.vmode = kVShared;
   else if (kp.bulk_stages > 0) kp.vmode = kVBulk;
   // the compact (two CTAs per SM) bulk variant, when chosen
   kp.compact = 0;
@@ -301,8 +300,9 @@ void run_solver(mlgmres* h, int ngroups, int ntasks, int grid, int arnoldi_steps
   }
   ARG(!kp.compact || (h->Rg && grid <= h->rg_blocks), "compact variant: grid exceeds its R workspace");
   // face coefficients from the current kappa (one pass over the grid)
-  if (ntasks == 1 && h->htasks[0].faces)
-    CK(launch_kappa_faces(h->grid.n, h->grid.kappa_dev, h->faces, h->fstride, s));
+  if (ntasks == 1 && h->htasks[0].faces64)
+    CK(launch_kappa_faces(h->grid.n, h->grid.kappa_dev, h->faces, h->fstride, h->faces64, h->ldv,
+                          s));
   kp.ngroups = ngroups;
   kp.group_first = h->dcfg;
   kp.task_first = h->dcfg + (ngroups + 1);
@@ -336,10 +336,12 @@ void stage_single(mlgmres* h, const SolveTask& t, int nblocks) {
   h->hcfg[3] = 1;
   h->hcfg[4] = 0;
   h->htasks[0] = t;
-  // the handle's own 3D grid: the FP32 passes use its face coefficients
-  if (h->faces && t.kappa == h->grid.kappa_dev && t.n == h->grid.n) {
+  // the handle's own 3D grid: the passes and the restarts use its face coefficients
+  if (h->faces64 && t.kappa == h->grid.kappa_dev && t.n == h->grid.n) {
     h->htasks[0].faces = h->faces;
     h->htasks[0].fstride = h->fstride;
+    h->htasks[0].faces64 = h->faces64;
+    h->htasks[0].f64stride = h->ldv;
   }
   h->hwork[0] = single_group_work(h, nblocks);
 }
@@ -646,6 +648,8 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
       CK(cudaMalloc(&h->W0_alloc, es * (size_t)h->ldv));
       h->W0 = h->W0_alloc;
     }
+    if (grid->dim == 3 && grid->kappa_dev)
+      CK(cudaMalloc(&h->faces64, sizeof(double) * 3 * (size_t)h->ldv));
     CK(cudaMalloc(&h->W1, es * (size_t)h->ldv));
     CK(cudaMalloc(&h->part, sizeof(double) * part_doubles(kPartStride)));
     if (opt->compact != 0 && gmres_compact_ok(h->fp32, grid->dim, opt->m)) {
@@ -725,6 +729,7 @@ void mlgmres_destroy(mlgmres_t h) {
   cudaFree(h->V);
   cudaFree(h->W0_alloc);
   if (h->faces) cudaFree(h->faces - (h->fstride - h->ldv) / 2);
+  cudaFree(h->faces64);
   cudaFree(h->W1);
   cudaFree(h->part);
   cudaFree(h->Rg);
@@ -908,6 +913,7 @@ mlgmres_status mlgmres_solve_batch(mlgmres_t h, int count, const mlgmres_grid* g
     const size_t es0 = h->fp32 ? sizeof(float) : sizeof(double);
     // shared-memory bytes of the largest CTA slice of V under a plan (0: does not fit)
     auto slice_need = [&](const std::vector<int>& gc, const std::vector<int>& go) {
+      if (dim == 3) return 0;  // the 3D shared-slice variants run single solves
       long long need = 0;
       for (int i = 0; i < count; i++) {
         const long long N = grid_points(dim, grids[i].n);
@@ -1092,8 +1098,8 @@ mlgmres_status mlgmres_autotune(mlgmres_t h, const double* b, int steps, int ret
     }
     for (auto [nb, compact] : shapes) {
       const int vs = single_vsmem(h, nb, compact != 0);
-      // 2D passes keep V in shared memory when the slice fits
-      const bool shared = h->grid.dim == 2 && vs > 0;
+      // the passes keep V in shared memory when the slice fits
+      const bool shared = vs > 0;
       std::vector<int> stages;
       if (shared) {
         stages.push_back(-1);

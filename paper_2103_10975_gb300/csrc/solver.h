@@ -53,6 +53,11 @@ struct SolveTask {
   // set only with a work vector W0 padded the same way (single 3D solves)
   const float* faces = nullptr;
   long long fstride = 0;
+  // FP64 face coefficients fx, fy, fz at faces64 + a * f64stride (or null:
+  // formed from kappa per point), for the FP64 evaluations of the operator: the
+  // restart residual of both precisions and the FP64 passes (single 3D solves)
+  const double* faces64 = nullptr;
+  long long f64stride = 0;
   DevResult* res;
   double* hist;          // optional |g_{j+1}|/||b|| per step (Arnoldi mode: H)
   long long hist_cap;
@@ -127,9 +132,10 @@ int gmres_compact_vsmem_budget();
 // The FP32 face coefficients of the 3D variable-coefficient operator (see
 // SolveTask::faces): fx/fy/fz(i) = harmonic mean of kappa_i and its +x/+y/+z
 // neighbour (0 on the domain's upper walls), fb(i) = kappa_i times the number
-// of the point's wall faces.
+// of the point's wall faces.  faces64 receives fx/fy/fz unrounded (SolveTask::
+// faces64).  faces may be null (FP64 handles need faces64 only).
 cudaError_t launch_kappa_faces(int n, const float* kappa, float* faces, long long fstride,
-                               cudaStream_t s);
+                               double* faces64, long long f64stride, cudaStream_t s);
 cudaError_t launch_apply(int dim, int n, const float* kappa, const double* u, double* out,
                          cudaStream_t s);
 
