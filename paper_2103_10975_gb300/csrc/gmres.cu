@@ -30,6 +30,10 @@ cudaError_t launch_gmres_f3c(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f2cs(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f2s32(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_d2s32(const KParams& kp, int grid, cudaStream_t s);
+cudaError_t launch_gmres_f3s(const KParams& kp, int grid, cudaStream_t s);
+cudaError_t launch_gmres_f3s32(const KParams& kp, int grid, cudaStream_t s);
+cudaError_t launch_gmres_d3s(const KParams& kp, int grid, cudaStream_t s);
+cudaError_t launch_gmres_d3s32(const KParams& kp, int grid, cudaStream_t s);
 int max_blocks_f3c(int* bs, int extra);
 int own_bytes_f3c();
 
@@ -72,7 +76,6 @@ int gmres_compact_max_blocks(int dim, int m) {
 }
 
 cudaError_t launch_gmres(const KParams& kp, bool fp32, int dim, int grid, cudaStream_t s) {
-  if (dim == 3 && kp.vmode == kVShared) return cudaErrorInvalidValue;
   if (kp.compact) {
     if (!gmres_compact_ok(fp32, dim, kp.m) || kp.vmode == kVDirect ||
         (dim == 3 && kp.vmode == kVShared))
@@ -87,6 +90,8 @@ cudaError_t launch_gmres(const KParams& kp, bool fp32, int dim, int grid, cudaSt
       if (kp.vmode == kVBulk) return launch_gmres_f2b(kp, grid, s);
       return launch_gmres_f2d(kp, grid, s);
     }
+    if (kp.vmode == kVShared)
+      return kp.m <= kSmallM ? launch_gmres_f3s32(kp, grid, s) : launch_gmres_f3s(kp, grid, s);
     if (kp.vmode == kVBulk) return launch_gmres_f3b(kp, grid, s);
     return launch_gmres_f3d(kp, grid, s);
   }
@@ -96,6 +101,8 @@ cudaError_t launch_gmres(const KParams& kp, bool fp32, int dim, int grid, cudaSt
     if (kp.vmode == kVBulk) return launch_gmres_d2b(kp, grid, s);
     return launch_gmres_d2d(kp, grid, s);
   }
+  if (kp.vmode == kVShared)
+    return kp.m <= kSmallM ? launch_gmres_d3s32(kp, grid, s) : launch_gmres_d3s(kp, grid, s);
   if (kp.vmode == kVBulk) return launch_gmres_d3b(kp, grid, s);
   return launch_gmres_d3d(kp, grid, s);
 }

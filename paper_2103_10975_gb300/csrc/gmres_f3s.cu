@@ -1,0 +1,12 @@
+// The 3D shared-slice variant, FP32 inner precision, for m <= 64: V slices in shared memory
+// (single solves whose slices fit; batches of 3D systems stream V).  Compiled on
+// its own so the variants build in parallel.
+#include "gmres_kernel.cuh"
+
+namespace mlg {
+
+cudaError_t launch_gmres_f3s(const KParams& kp, int grid, cudaStream_t s) {
+  return launch_t<float, 3, kMaxM, 256, kVShared>(kp, grid, s);
+}
+
+}  // namespace mlg
