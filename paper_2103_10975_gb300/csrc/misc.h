@@ -9,8 +9,11 @@ cudaError_t launch_normalise(const double* b, int N, const double* sumsq, float*
                              cudaStream_t s);
 cudaError_t launch_denormalise(const float* y, int N, const double* sumsq, double scale,
                                double* x, cudaStream_t s);
-cudaError_t launch_jacobi(int dim, int n, const float* kappa, const double* b, const double* xin,
-                          double* xout, double omega, cudaStream_t s);
+// `sweeps` damped-Jacobi sweeps on x, with tmp as the other buffer; *result is
+// the one of the two that holds the outcome.
+cudaError_t launch_jacobi(int dim, int n, const float* kappa, const double* b, double* x,
+                          double* tmp, double omega, int sweeps, double** result,
+                          cudaStream_t s);
 cudaError_t launch_store_pair(const double* b, const double* x, int N, const double* sumsq,
                               float* u, float* t, cudaStream_t s);
 cudaError_t launch_spread_dots(const double* x, const float* ring, long long stride,

@@ -79,8 +79,10 @@ int auto_blocks(const mlgmres* h, int N) {
   if (!h->fp32) {
     // FP64: a warp FMA occupies its SM quarter's FP64 pipe for 64 cycles, so the
     // step is bound by the tiles per SM quarter: the fewest tiles per CTA the
-    // co-resident CTAs allow, rounded up to whole tiles per quarter (32^2: 8
-    // CTAs of 4 tiles instead of 2 of 16; 256^2: 128 CTAs of 16)
+    // co-resident CTAs allow, rounded up to whole tiles per quarter (32^2,
+    // GMRES(20): 8 CTAs of 4 tiles, 14.2 us per step, where 2 CTAs of 16 took
+    // 24.3; 128^2: 16.8 against 28.3; 256^2 stays at 128 CTAs of 16: 152 CTAs of
+    // 14 have as many per quarter and took 33.3 against 32.2)
     const int tiles = (N + 31) / 32;
     const int per = (tiles + h->max_blocks - 1) / h->max_blocks;
     for (int t : {(per + 3) / 4 * 4, per}) {
@@ -244,13 +246,9 @@ double* learned_guess(mlgmres* h, const double* b, cudaStream_t s) {
   CK(launch_normalise(b, N, h->scal, h->u_in, s));
   guess_forward(h, h->u_in, h->y_out, s);
   double* cur = h->x_alt;
-  double* oth = h->x_tmp;
   CK(launch_denormalise(h->y_out, N, h->scal, h->c_guess, cur, s));
-  for (int k = 0; k < h->opt.guess_smooth; k++) {
-    CK(launch_jacobi(h->grid.dim, h->grid.n, h->grid.kappa_dev, b, cur, oth,
-                     (double)h->opt.guess_omega, s));
-    std::swap(cur, oth);
-  }
+  CK(launch_jacobi(h->grid.dim, h->grid.n, h->grid.kappa_dev, b, cur, h->x_tmp,
+                   (double)h->opt.guess_omega, h->opt.guess_smooth, &cur, s));
   return cur;
 }
 
@@ -1345,12 +1343,8 @@ mlgmres_status mlgmres_smooth(mlgmres_t h, const double* b, double* x, int sweep
     ARG(sweeps >= 0 && sweeps <= 1000, "sweeps must be in 0..1000");
     cudaStream_t s = (cudaStream_t)stream;
     double* cur = x;
-    double* oth = h->x_tmp;
-    for (int k = 0; k < sweeps; k++) {
-      CK(launch_jacobi(h->grid.dim, h->grid.n, h->grid.kappa_dev, b, cur, oth,
-                       (double)h->opt.guess_omega, s));
-      std::swap(cur, oth);
-    }
+    CK(launch_jacobi(h->grid.dim, h->grid.n, h->grid.kappa_dev, b, x, h->x_tmp,
+                     (double)h->opt.guess_omega, sweeps, &cur, s));
     if (cur != x) CK(cudaMemcpyAsync(x, cur, sizeof(double) * h->N, cudaMemcpyDeviceToDevice, s));
     CK(cudaStreamSynchronize(s));
     return MLGMRES_OK;

@@ -12,6 +12,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from oracle import direct
+from oracle import guess as og
 from synthetic import MovingGaussians2D, MovingGaussians3D, lognormal_kappa
 
 pytestmark = pytest.mark.gpu
@@ -55,3 +56,19 @@ def test_3d_slices_against_the_streamed_basis(n, m, prec):
         if kap is None:
             xe = direct.dst_solve_3d(n, b)
             assert np.linalg.norm(xs[0] - xe) <= 1e-7 * np.linalg.norm(xe)
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 33, 130, 321])
+def test_jacobi_tiles(n):
+    """Sweeps in tiles with halos (both tile sizes, ragged edges, launches of fewer
+    than four sweeps) against the plain formula in FP64: about ten roundings per
+    point and sweep, so 1e-13 after ten sweeps."""
+    from paper_2103_10975_gb300 import Solver
+    s = Solver(n, m=10, guess_omega=0.75)
+    rng = np.random.default_rng(n)
+    b, x0 = rng.standard_normal(n * n), rng.standard_normal(n * n)
+    for sweeps in (1, 3, 4, 6, 10):
+        xd = torch.as_tensor(x0.copy()).cuda()
+        s.smooth(torch.as_tensor(b).cuda(), xd, sweeps)
+        ref = og.jacobi(2, n, b, x0, sweeps, 0.75)
+        assert np.linalg.norm(xd.cpu().numpy() - ref) <= 1e-13 * np.linalg.norm(ref), sweeps
