@@ -258,12 +258,19 @@ __global__ void mse_grad(long long total, float scale, float ts, const float* __
   }
 }
 
-__global__ void loss_finish(const float* __restrict__ part, int nparts, float scale,
-                            float* __restrict__ loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < nparts; i++) s += part[i];
-    *loss = (float)(s * scale);
+// loss = scale * sum of the CTA partials (FP64, a fixed tree over 256 threads: one
+// thread adding them in turn took 20 us of dependent FP64 additions)
+__global__ void __launch_bounds__(256) loss_finish(const float* __restrict__ part, int nparts,
+                                                   float scale, float* __restrict__ loss) {
+  __shared__ double red[8];
+  double v = 0.0;
+  for (int i = threadIdx.x; i < nparts; i += 256) v += part[i];
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) v += red[w];
+    *loss = (float)(v * scale);
   }
 }
 
@@ -366,7 +373,8 @@ __global__ void __launch_bounds__(kW1Threads) conv_out_bwd_data(int B, int n,
 // MODE 0 (output conv):  dW[c][tap] = sum_p gy[p] t[p + off][c]
 //                                   = sum_q t[q][c] gy[q - off],  db = sum_q gy[q]
 // MODE 1 (input conv):   dW[c][tap] = sum_p g32[p][c] u[p + off], db[c] = sum_p g32[p][c],
-//                        with g32 taken as 0 where m32 <= 0 (the ReLU of a0)
+//                        with g32 taken as 0 where m32 <= 0 (the ReLU of a0), plus
+//                        2^-D of the pooled level's gradient gc (null: no such level)
 // The grid is cut into segments of R rows x W points of one (b, z) plane
 // (W = min(n, 256), R = max(1, 256 / n)).  Lane = channel: every 32-channel row
 // is read once, coalesced, U rows per warp in flight; the 1-channel field (gy
@@ -384,8 +392,8 @@ int conv1_wgrad_smem(int n) {
 template <int MODE, int D>
 __global__ void __launch_bounds__(kW1Threads, D == 3 ? 1 : 2) conv1_wgrad(
     int B, int n, const float* __restrict__ g1, const bf16* __restrict__ x32,
-    const float* __restrict__ g32, const bf16* __restrict__ m32, const float* __restrict__ u,
-    float* __restrict__ part, int stride) {
+    const float* __restrict__ g32, const float* __restrict__ gc, const bf16* __restrict__ m32,
+    const float* __restrict__ u, float* __restrict__ part, int stride) {
   constexpr int T = Geo<D>::T;
   constexpr int NW = kW1Threads / 32;
   constexpr int U = kSeg / NW;             // points per warp and segment
@@ -420,8 +428,15 @@ __global__ void __launch_bounds__(kW1Threads, D == 3 ? 1 : 2) conv1_wgrad(
           const long long p = ((long long)pl * n + y) * n + x;
           if (MODE == 0)
             v = __bfloat162float(x32[p * kC + c]);
-          else
-            v = __bfloat162float(m32[p * kC + c]) > 0.f ? g32[p * kC + c] : 0.f;
+          else if (__bfloat162float(m32[p * kC + c]) > 0.f) {
+            v = g32[p * kC + c];
+            // the pooled level's share (odd sides: the last point has none)
+            const int so = n / 2, pz = pl % n;
+            if (gc && y / 2 < so && x / 2 < so && (D == 2 || pz / 2 < so)) {
+              const int cp = D == 3 ? (pl / n) * so + pz / 2 : pl;
+              v += (1.f / (1 << D)) * gc[(((long long)cp * so + y / 2) * so + x / 2) * kC + c];
+            }
+          }
         }
         val[k] = v;
         if (++xl == W) {
@@ -542,12 +557,12 @@ __global__ void __launch_bounds__(256) reduce_wgrad(const float* __restrict__ pa
 // (built once on the host with the same arithmetic as bilin).  The
 // D-dimensional transpose is D such passes, one per axis.
 
-// With outbf (the last axis): outbf = bf16(mask > 0 ? out : 0) instead of out.
+// One axis of one level; the levels' x-axis passes where a fine row is too long
+// to stage (upsample_bwd_x_levels otherwise).
 __global__ void upsample_bwd_axis(long long outer, int n, int m, long long inner,
                                   const int* __restrict__ ptr, const int* __restrict__ idx,
                                   const float* __restrict__ wt, const float* __restrict__ in,
-                                  float* __restrict__ out, const bf16* __restrict__ mask,
-                                  bf16* __restrict__ outbf) {
+                                  float* __restrict__ out) {
   const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (id >= outer * m * inner) return;
   // element indices stay below 2^31 (network size check): 32-bit division
@@ -559,35 +574,64 @@ __global__ void upsample_bwd_axis(long long outer, int n, int m, long long inner
   float acc = 0.f;
   for (int k = ptr[j]; k < ptr[j + 1]; k++)
     acc += wt[k] * in[((long long)o * n + idx[k]) * inner + c];
-  if (outbf)
-    outbf[id] = __float2bfloat16(__bfloat162float(mask[id]) > 0.f ? acc : 0.f);
-  else
-    out[id] = acc;
+  out[id] = acc;
+}
+
+// Sum of wt[k] * src[k * stride] over k < cnt for four channels, in the order of
+// k, eight loads in flight.
+__device__ __forceinline__ float4 row_sum4(const float* __restrict__ src, long long stride,
+                                           const float* __restrict__ wt, int cnt) {
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&](float w, const float4& v) {
+    acc.x += w * v.x;
+    acc.y += w * v.y;
+    acc.z += w * v.z;
+    acc.w += w * v.w;
+  };
+  int k = 0;
+  for (; k + 8 <= cnt; k += 8) {
+    float4 v[8];
+    float w[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      v[u] = *reinterpret_cast<const float4*>(src + (k + u) * stride);
+      w[u] = wt[k + u];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; u++) add(w[u], v[u]);
+  }
+  for (; k < cnt; k++) add(wt[k], *reinterpret_cast<const float4*>(src + k * stride));
+  return acc;
 }
 
 // The x-axis pass of every coarse level's transposed upsampling at once:
 //   out_l[r][j][c] = sum_x U_l[x][j] in[r][x][c]   (levels l = 1 .. L-1)
 // for each row r of the fine grid (x is the innermost axis in 2D and 3D).  One
-// CTA per row: its n x 32 values are read from HBM once and from L1 for the
-// other levels (the per-level pass reads the whole fine gradient per level).
-// Same sums, in the same order, as upsample_bwd_axis.
-struct UpXLevels {
-  int nlev;
+// CTA per row: its n x 32 values are read from HBM once and from shared memory
+// for every level.  A thread forms four channels of one coarse point (16-byte
+// reads, a quarter of the instructions of one channel per lane; the fine points
+// of a coarse one are consecutive, so only the first index is read).  Same
+// sums, in the same order, as upsample_bwd_axis.
+struct UpLevels {
+  int nlev;                     // levels 1 .. nlev-1
   int m[kMaxLevels];
   const int* ptr[kMaxLevels];
   const int* idx[kMaxLevels];
   const float* wt[kMaxLevels];
-  long long off[kMaxLevels];  // out_l = out + off[l], rows of m_l x 32
+  long long in_off[kMaxLevels], out_off[kMaxLevels];
+  unsigned first[kMaxLevels + 1];  // first CTA of each level (axis kernel)
+  long long outer[kMaxLevels], inner[kMaxLevels];
+  const bf16* mask[kMaxLevels];    // last axis: the ReLU mask of the level's output
 };
 
 constexpr int kXLevelsMaxN = 384;  // the staged row (n x 32 floats) stays within 48 KB
 
-__global__ void __launch_bounds__(256) upsample_bwd_x_levels(int n, UpXLevels lv,
+__global__ void __launch_bounds__(256) upsample_bwd_x_levels(int n, UpLevels lv,
                                                              const float* __restrict__ in,
                                                              float* __restrict__ out) {
   extern __shared__ float row[];  // the fine row, n x 32
   const long long r = blockIdx.x;
-  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int c4 = (threadIdx.x & 7) * 4, g = threadIdx.x >> 3;
   {
     const float4* src = reinterpret_cast<const float4*>(in + r * n * kC);
     float4* dst = reinterpret_cast<float4*>(row);
@@ -596,31 +640,93 @@ __global__ void __launch_bounds__(256) upsample_bwd_x_levels(int n, UpXLevels lv
   __syncthreads();
   for (int l = 1; l < lv.nlev; l++) {
     const int m = lv.m[l];
-    const int* __restrict__ ptr = lv.ptr[l];
-    const int* __restrict__ idx = lv.idx[l];
-    const float* __restrict__ wt = lv.wt[l];
-    float* __restrict__ o = out + lv.off[l] + r * m * kC;
-    for (int j = w; j < m; j += 8) {
-      float acc = 0.f;
-      for (int k = ptr[j]; k < ptr[j + 1]; k++) acc += wt[k] * row[idx[k] * kC + c];
-      o[j * kC + c] = acc;
+    float* __restrict__ o = out + lv.out_off[l] + r * m * kC;
+    for (int j = g; j < m; j += 32) {
+      const int k0 = lv.ptr[l][j];
+      *reinterpret_cast<float4*>(o + j * kC + c4) =
+          row_sum4(row + lv.idx[l][k0] * kC + c4, kC, lv.wt[l] + k0, lv.ptr[l][j + 1] - k0);
     }
   }
 }
 
-// fine[p][c] += coarse[p / 2][c] / 2^D (fine side s, coarse side s/2)
+// One further axis of every coarse level's transposed upsampling in one launch:
+// (outer, n, inner) -> (outer, m, inner) per level, four inner elements per
+// thread.  With masks (the last axis): outbf = bf16(mask > 0 ? sum : 0), else out.
+// One launch per level left most SMs idle on the coarse ones (8 x 8 points of 64
+// sums each): 95 us in all at 256^2 x 8, 36 now.  With the pooling chain in one
+// launch and the parallel loss sum the network's forward and backward went from
+// 1464 to 1362 us.
+__global__ void __launch_bounds__(256) upsample_bwd_axis_levels(int n, UpLevels lv,
+                                                                const float* __restrict__ in,
+                                                                float* __restrict__ out,
+                                                                bf16* __restrict__ outbf) {
+  int l = 1;
+  while (l + 1 < lv.nlev && blockIdx.x >= lv.first[l + 1]) l++;
+  const unsigned i4 = (unsigned)(lv.inner[l] / 4);
+  const int m = lv.m[l];
+  const unsigned id = (blockIdx.x - lv.first[l]) * 256u + threadIdx.x;
+  if ((long long)id >= lv.outer[l] * m * i4) return;
+  // element indices stay below 2^31 (network size check): 32-bit division
+  const unsigned c = (id % i4) * 4u, p = id / i4;
+  const int j = (int)(p % (unsigned)m);
+  const unsigned o = p / (unsigned)m;
+  const int k0 = lv.ptr[l][j];
+  const float4 v = row_sum4(
+      in + lv.in_off[l] + ((long long)o * n + lv.idx[l][k0]) * lv.inner[l] + c, lv.inner[l],
+      lv.wt[l] + k0, lv.ptr[l][j + 1] - k0);
+  const long long at = lv.out_off[l] + (long long)id * 4;
+  if (!outbf) {
+    *reinterpret_cast<float4*>(out + at) = v;
+    return;
+  }
+  const uint2 mv = *reinterpret_cast<const uint2*>(lv.mask[l] + (long long)id * 4);
+  const __nv_bfloat162* mk = reinterpret_cast<const __nv_bfloat162*>(&mv);
+  const float2 m0 = __bfloat1622float2(mk[0]), m1 = __bfloat1622float2(mk[1]);
+  uint2 ov;
+  __nv_bfloat162* ob = reinterpret_cast<__nv_bfloat162*>(&ov);
+  ob[0] = __floats2bfloat162_rn(m0.x > 0.f ? v.x : 0.f, m0.y > 0.f ? v.y : 0.f);
+  ob[1] = __floats2bfloat162_rn(m1.x > 0.f ? v.z : 0.f, m1.y > 0.f ? v.w : 0.f);
+  *reinterpret_cast<uint2*>(outbf + at) = ov;
+}
+
+// The pooling chain's gradient at level 1: g_1 += 2^-D (g_2 + 2^-D (g_3 + ...))
+// over a point's ancestors (as far as they exist: odd sides drop their last
+// point), coarsest first, so each sum is the one that level-by-level passes form
+// (scaling by 2^-D is exact).  One launch instead of a read-modify-write pass
+// per level; level 0 adds its own share where its gradient is consumed
+// (conv1_wgrad), which saves its 134 MB pass at 256^2 x 8.
+struct PoolLevels {
+  int nlev;
+  int side[kMaxLevels];
+  float* g[kMaxLevels];
+};
+
 template <int D>
-__global__ void pool2_bwd_add(int B, int s, const float* __restrict__ coarse,
-                              float* __restrict__ fine) {
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= B * Geo<D>::pts(s) * kC) return;
-  const int c = (int)(idx % kC);
+__global__ void __launch_bounds__(256) pool_chain_bwd(int B, PoolLevels lv) {
+  const int s1 = lv.side[1];
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= B * Geo<D>::pts(s1) * (kC / 4)) return;
+  const int c4 = (int)(i % (kC / 4)) * 4;
   int b, z, y, x;
-  Geo<D>::decode(idx / kC, s, b, z, y, x);
-  const int so = s / 2;
-  if (y / 2 >= so || x / 2 >= so || (D == 3 && z / 2 >= so)) return;
-  const long long q = Geo<D>::nb(b, z / 2, y / 2, x / 2, 0, 0, 0, so);
-  fine[idx] += (1.f / (1 << D)) * coarse[q * kC + c];
+  Geo<D>::decode(i / (kC / 4), s1, b, z, y, x);
+  int top = 1;
+  while (top + 1 < lv.nlev) {
+    const int sh = top, so = lv.side[top + 1];  // level top + 1: coordinates >> top
+    if ((y >> sh) >= so || (x >> sh) >= so || (D == 3 && (z >> sh) >= so)) break;
+    top++;
+  }
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int l = top; l >= 1; l--) {
+    const int sh = l - 1;
+    const long long q = Geo<D>::nb(b, z >> sh, y >> sh, x >> sh, 0, 0, 0, lv.side[l]);
+    const float4 g = *reinterpret_cast<const float4*>(lv.g[l] + q * kC + c4);
+    const float f = l == top ? 0.f : 1.f / (1 << D);
+    v.x = g.x + f * v.x;
+    v.y = g.y + f * v.y;
+    v.z = g.z + f * v.z;
+    v.w = g.w + f * v.w;
+  }
+  if (top > 1) *reinterpret_cast<float4*>(lv.g[1] + i * 4) = v;
 }
 
 // Adam (Kingma & Ba): m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
@@ -846,6 +952,7 @@ cudaError_t net_create(Net& net, int n, int bmax, unsigned long long seed, int d
   NN_CK(cudaMalloc(&net.g_lvl, sizeof(float) * full));
   NN_CK(cudaMalloc(&net.g_pool, sizeof(float) * net.pyr));
   NN_CK(cudaMalloc(&net.g_bf, sizeof(bf16) * full));
+  if (L > 1) NN_CK(cudaMalloc(&net.g_bl, sizeof(bf16) * (net.pyr - net.lvl_off[1])));
   int dev = 0, nsm = 0;
   NN_CK(cudaGetDevice(&dev));
   NN_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -908,6 +1015,7 @@ void net_destroy(Net& net) {
   cudaFree(net.g_lvl);
   cudaFree(net.g_pool);
   cudaFree(net.g_bf);
+  cudaFree(net.g_bl);
   cudaFree(net.wgrad_part);
   cudaFree(net.gy);
   cudaFree(net.loss_part);
@@ -993,7 +1101,7 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
   mse_grad<<<lparts, 256, 0, s>>>(pix, 1.f / (float)pix, tscale, tscale_dev, y, target, net.gy,
                                   net.loss_part);
   note_launches(1);
-  loss_finish<<<1, 32, 0, s>>>(net.loss_part, lparts, 1.f / (float)pix, loss_dev);
+  loss_finish<<<1, 256, 0, s>>>(net.loss_part, lparts, 1.f / (float)pix, loss_dev);
   note_launches(1);
   // output conv
   const bf16* tfin = net.extra_active > 0 ? net.tt[net.extra_active - 1] : net.t;
@@ -1001,7 +1109,7 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
   const int P1 = P, stride1 = kC * (T + 1);
   const int smem1 = conv1_wgrad_smem<D>(n);
   conv1_wgrad<0, D><<<P1, kW1Threads, smem1, s>>>(B, n, net.gy, tfin, nullptr, nullptr, nullptr,
-                                                  net.wgrad_part, stride1);
+                                                  nullptr, net.wgrad_part, stride1);
   note_launches(1);
   reduce_wgrad<<<nblk(T * kC + 1, 32), 256, 0, s>>>(net.wgrad_part, P1, stride1, 2, T,
                                                      net.grad + net.off_w[L + 2],
@@ -1053,83 +1161,98 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
   // pyramid levels; first the x-axis pass of every coarse level's transposed
   // upsampling, from one read of the fine gradient (g_s) into g_t (free here:
   // the residual block's gradient is already in g_s)
-  long long xoff[kMaxLevels] = {};
   const bool fused_x = L > 1 && n <= kXLevelsMaxN;
+  UpLevels lv{};
+  lv.nlev = L;
+  const long long rows = B * Geo<D>::pts(n) / n;
+  for (int l = 1; l < L; l++) {
+    lv.m[l] = net.side[l];
+    lv.ptr[l] = net.up_ptr[l];
+    lv.idx[l] = net.up_idx[l];
+    lv.wt[l] = net.up_w[l];
+    lv.mask[l] = net.z[l];
+  }
+  // the remaining axes (y; in 3D y, then z) of levels l0 .. l1-1, from their x
+  // passes at g_t + xin[l], into their masked BF16 gradients
+  auto other_axes = [&](int l0, int l1, const long long* xin) {
+    UpLevels v = lv;
+    for (int ax = 1; ax < D; ax++) {
+      const bool last = ax == D - 1;
+      unsigned blocks = 0;
+      long long off = 0;
+      for (int l = 1; l < l1; l++) {
+        const long long m = net.side[l];
+        v.first[l] = blocks;
+        if (l < l0) continue;  // (an empty range of CTAs)
+        v.outer[l] = D == 3 && ax == 1 ? (long long)B * n : B;
+        v.inner[l] = (ax == 1 ? m : m * m) * kC;
+        v.in_off[l] = ax == 1 ? xin[l] : v.out_off[l];
+        v.out_off[l] = last ? net.lvl_off[l] - net.lvl_off[1] : off;
+        off += v.outer[l] * m * v.inner[l];
+        blocks += nblk(v.outer[l] * m * v.inner[l] / 4, 256);
+      }
+      v.nlev = l1;
+      upsample_bwd_axis_levels<<<blocks, 256, 0, s>>>(n, v, ax == 1 ? net.g_t : net.g_lvl,
+                                                      last ? nullptr : net.g_lvl,
+                                                      last ? net.g_bl : nullptr);
+      note_launches(1);
+    }
+  };
   if (fused_x) {
-    UpXLevels lv;
-    lv.nlev = L;
-    const long long rows = B * Geo<D>::pts(n) / n;
     long long off = 0;
     for (int l = 1; l < L; l++) {
-      lv.m[l] = net.side[l];
-      lv.ptr[l] = net.up_ptr[l];
-      lv.idx[l] = net.up_idx[l];
-      lv.wt[l] = net.up_w[l];
-      lv.off[l] = xoff[l] = off;
+      lv.out_off[l] = off;
       off += rows * net.side[l] * kC;
     }
     upsample_bwd_x_levels<<<(unsigned)rows, 256, sizeof(float) * n * kC, s>>>(n, lv, net.g_s,
                                                                                net.g_t);
     note_launches(1);
+    long long xin[kMaxLevels];
+    for (int l = 1; l < L; l++) xin[l] = lv.out_off[l];
+    other_axes(1, L, xin);
   }
   for (int l = 0; l < L; l++) {
     const int sd = net.side[l];
-    const long long lp = B * Geo<D>::pts(sd);
-    const float* gz = net.g_s;
+    const bf16* gz = net.g_bf;
     if (l > 0) {
-      // transposed upsampling, one axis at a time (x, y, then z); g_t and
-      // g_lvl are free here (the residual block's gradient is already in g_s)
-      const long long nn = n, m = sd;
-      const int* up = net.up_ptr[l];
-      const int* ui = net.up_idx[l];
-      const float* uw = net.up_w[l];
-      const float* gx = net.g_t + xoff[l];  // this level's x-axis pass (above)
-      if (!fused_x) {  // (rows too long to stage: the level's own x-axis pass)
-        upsample_bwd_axis<<<nblk(B * Geo<D>::pts(n) / n * m * kC, 256), 256, 0, s>>>(
-            B * Geo<D>::pts(n) / n, n, sd, kC, up, ui, uw, net.g_s, net.g_t, nullptr, nullptr);
+      if (!fused_x) {  // (rows too long to stage: the level's own passes)
+        upsample_bwd_axis<<<nblk(rows * sd * kC, 256), 256, 0, s>>>(
+            rows, n, sd, kC, net.up_ptr[l], net.up_idx[l], net.up_w[l], net.g_s, net.g_t);
         note_launches(1);
-        gx = net.g_t;
+        const long long xin[kMaxLevels] = {};
+        other_axes(l, l + 1, xin);
       }
-      if (D == 2) {
-        upsample_bwd_axis<<<nblk(B * m * m * kC, 256), 256, 0, s>>>(
-            B, n, sd, m * kC, up, ui, uw, gx, nullptr, net.z[l], net.g_bf);
-        note_launches(1);
-        gz = nullptr;  // masked BF16 gradient already in g_bf
-      } else {
-        upsample_bwd_axis<<<nblk(B * nn * m * m * kC, 256), 256, 0, s>>>(
-            B * nn, n, sd, m * kC, up, ui, uw, gx, net.g_lvl, nullptr, nullptr);
-        upsample_bwd_axis<<<nblk(B * m * m * m * kC, 256), 256, 0, s>>>(
-            B, n, sd, m * m * kC, up, ui, uw, net.g_lvl, nullptr, net.z[l], net.g_bf);
-        note_launches(2);
-        gz = nullptr;
-      }
-    }
-    if (gz) {
-      mask_to_bf16<<<nblk((lp * kC) / 8, 256), 256, 0, s>>>(lp * kC, gz, net.z[l], net.g_bf);
+      gz = net.g_bl + (net.lvl_off[l] - net.lvl_off[1]);
+    } else {
+      const long long lp = B * Geo<D>::pts(sd);
+      mask_to_bf16<<<nblk((lp * kC) / 8, 256), 256, 0, s>>>(lp * kC, net.g_s, net.z[0], net.g_bf);
       note_launches(1);
     }
     const bf16* in = l == 0 ? net.a0 : net.pool[l];
-    NN_CK(launch_wgrad_mma(D, B, sd, in, net.g_bf, 1, net.wgrad_part, stride, P, s));
+    NN_CK(launch_wgrad_mma(D, B, sd, in, gz, 1, net.wgrad_part, stride, P, s));
     reduce_wgrad<<<nblk(per + kC, 32), 256, 0, s>>>(net.wgrad_part, P, stride, 0, T,
                                                      net.grad + net.off_w[1 + l],
                                                      net.grad + net.off_b[1 + l]);
     note_launches(1);
-    NN_CK(launch_conv32_mma(D, 2, B, sd, net.g_bf, net.wq + per * l, nullptr, 1, -1, nullptr,
+    NN_CK(launch_conv32_mma(D, 2, B, sd, gz, net.wq + per * l, nullptr, 1, -1, nullptr,
                             nullptr, nullptr, net.g_pool + net.lvl_off[l], nullptr, s));
   }
   // pooling chain: the gradient of p_{l-1} collects 1/2^D of p_l's
-  for (int l = L - 1; l >= 1; l--) {
-    const int sf = net.side[l - 1];
-    const long long cnt = B * Geo<D>::pts(sf) * kC;
-    pool2_bwd_add<D><<<nblk(cnt, 256), 256, 0, s>>>(B, sf, net.g_pool + net.lvl_off[l],
-                                                    net.g_pool + net.lvl_off[l - 1]);
+  if (L > 2) {
+    PoolLevels pv{};
+    pv.nlev = L;
+    for (int l = 1; l < L; l++) {
+      pv.side[l] = net.side[l];
+      pv.g[l] = net.g_pool + net.lvl_off[l];
+    }
+    pool_chain_bwd<D><<<nblk(B * Geo<D>::pts(net.side[1]) * (kC / 4), 256), 256, 0, s>>>(B, pv);
     note_launches(1);
   }
   // input conv
   // (the ReLU mask of a0 is applied inside the weight-gradient kernel)
-  conv1_wgrad<1, D><<<P1, kW1Threads, smem1, s>>>(B, n, nullptr, nullptr,
-                                                  net.g_pool + net.lvl_off[0], net.a0, u,
-                                                  net.wgrad_part, stride1);
+  conv1_wgrad<1, D><<<P1, kW1Threads, smem1, s>>>(
+      B, n, nullptr, nullptr, net.g_pool + net.lvl_off[0],
+      L > 1 ? net.g_pool + net.lvl_off[1] : nullptr, net.a0, u, net.wgrad_part, stride1);
   note_launches(1);
   reduce_wgrad<<<nblk(T * kC + kC, 32), 256, 0, s>>>(net.wgrad_part, P1, stride1, 1, T,
                                                       net.grad + net.off_w[0],

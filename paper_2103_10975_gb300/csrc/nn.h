@@ -79,6 +79,7 @@ struct Net {
   float* g_lvl = nullptr;                    // scratch, bmax x n^2 x 32
   float* g_pool = nullptr;                   // pooled accumulation, bmax x n^2 x 32
   __nv_bfloat16* g_bf = nullptr;             // bf16 operand scratch
+  __nv_bfloat16* g_bl = nullptr;             // the coarse levels' masked gradients (levels 1 ..)
   float* wgrad_part = nullptr;               // split-K partials of weight gradients
   float* gy = nullptr;                       // bmax x n^2
   float* loss_part = nullptr;
