@@ -26,12 +26,42 @@ __global__ void sumsq_kernel(const double* __restrict__ b, int N, double* out) {
   }
 }
 
-// u = b / s with s = sqrt(sumsq / N) (s = 1 when b = 0)
-__global__ void normalise_kernel(const double* __restrict__ b, int N, const double* sumsq,
-                                 float* __restrict__ u) {
+// Partial sums of squares, one per CTA (fixed order: deterministic).
+__global__ void __launch_bounds__(256) sumsq_part_kernel(const double* __restrict__ b, int N,
+                                                         double* __restrict__ part) {
+  __shared__ double red[8];
+  double s = 0.0;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < N; i += gridDim.x * 256) s += b[i] * b[i];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) s += red[w];
+    part[blockIdx.x] = s;
+  }
+}
+
+// u = b / s with s = sqrt(sumsq / N) (s = 1 when b = 0); sumsq is the sum of the
+// nparts partials, which every CTA adds up for itself (the same tree in each) and
+// the first one stores.  (One CTA over all of b took 20 us at 256^2.)
+__global__ void __launch_bounds__(256) normalise_kernel(const double* __restrict__ b, int N,
+                                                        const double* __restrict__ part,
+                                                        int nparts, double* __restrict__ sumsq,
+                                                        float* __restrict__ u) {
+  __shared__ double sh;
+  if (threadIdx.x < 32) {
+    double v = 0.0;
+    for (int k = threadIdx.x; k < nparts; k += 32) v += part[k];
+    v = warp_sum(v);
+    if (threadIdx.x == 0) {
+      if (blockIdx.x == 0) *sumsq = v;
+      sh = sqrt(v / N);
+    }
+  }
+  __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  double s = sqrt(*sumsq / N);
+  double s = sh;
   if (!(s > 0.0)) s = 1.0;
   u[i] = (float)(b[i] / s);
 }
@@ -189,10 +219,13 @@ cudaError_t launch_sumsq(const double* b, int N, double* out, cudaStream_t s) {
   note_launches(1);
   return cudaGetLastError();
 }
-cudaError_t launch_normalise(const double* b, int N, const double* sumsq, float* u,
+cudaError_t launch_normalise(const double* b, int N, double* part, double* sumsq, float* u,
                              cudaStream_t s) {
-  normalise_kernel<<<blocks_for(N), 256, 0, s>>>(b, N, sumsq, u);
-  note_launches(1);
+  // about four elements per thread and partial
+  const int np = N < 1024 * kNormParts ? (N + 1023) / 1024 : kNormParts;
+  sumsq_part_kernel<<<np, 256, 0, s>>>(b, N, part);
+  normalise_kernel<<<blocks_for(N), 256, 0, s>>>(b, N, part, np, sumsq, u);
+  note_launches(2);
   return cudaGetLastError();
 }
 cudaError_t launch_jacobi(int dim, int n, const float* kappa, const double* b, double* x,

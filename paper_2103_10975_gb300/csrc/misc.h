@@ -5,7 +5,10 @@
 
 namespace mlg {
 cudaError_t launch_sumsq(const double* b, int N, double* out, cudaStream_t s);
-cudaError_t launch_normalise(const double* b, int N, const double* sumsq, float* u,
+// u = b / rms(b); *sumsq receives the sum of squares, part is scratch for
+// kNormParts doubles.
+constexpr int kNormParts = 152;
+cudaError_t launch_normalise(const double* b, int N, double* part, double* sumsq, float* u,
                              cudaStream_t s);
 cudaError_t launch_denormalise(const float* y, int N, const double* sumsq, double scale,
                                double* x, cudaStream_t s);

@@ -242,8 +242,8 @@ float* model_grad(mlgmres* h) { return h->linear ? h->lin.grad : h->net.grad; }
 // damped-Jacobi sweeps; returns the buffer (x_alt or x_tmp) that holds it.
 double* learned_guess(mlgmres* h, const double* b, cudaStream_t s) {
   const int N = h->N;
-  CK(launch_sumsq(b, N, h->scal, s));
-  CK(launch_normalise(b, N, h->scal, h->u_in, s));
+  // (scal: [0..7] scalars, then room for 4096 ring slots as ints, then scratch)
+  CK(launch_normalise(b, N, h->scal + 8 + 2048, h->scal, h->u_in, s));
   guess_forward(h, h->u_in, h->y_out, s);
   double* cur = h->x_alt;
   CK(launch_denormalise(h->y_out, N, h->scal, h->c_guess, cur, s));

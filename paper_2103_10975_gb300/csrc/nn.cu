@@ -16,21 +16,6 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
-__device__ __forceinline__ void load32(const bf16* p, float* v) {
-  const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    uint4 u = q[i];
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      float2 f = __bfloat1622float2(h[j]);
-      v[i * 8 + 2 * j] = f.x;
-      v[i * 8 + 2 * j + 1] = f.y;
-    }
-  }
-}
-
 __device__ __forceinline__ void store32(bf16* p, const float* v) {
   uint4* q = reinterpret_cast<uint4*>(p);
 #pragma unroll
@@ -119,43 +104,94 @@ __global__ void conv_in_fwd(int B, int n, const float* __restrict__ u,
   store32(a0 + p * kC, v);
 }
 
-// out = mean of each 2^D block of in (side s -> s/2), channels last
+// Up to kPoolDepth levels of the average-pool pyramid in one launch: out_l = mean
+// of each 2^D block of level l - 1 (side s -> s/2), channels last, BF16.  A CTA
+// owns a block of 2^kPoolDepth points per axis of the finest level, whose
+// descendants depend on nothing else: level 1 comes from global memory, the
+// others from the level before in shared memory (as rounded to BF16).
 template <int D>
-__global__ void pool2_fwd(int B, int s, const bf16* __restrict__ in, bf16* __restrict__ out) {
-  const int so = s / 2;
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= B * Geo<D>::pts(so) * kC) return;
-  const int c = (int)(i % kC);
-  int b, z, y, x;
-  Geo<D>::decode(i / kC, so, b, z, y, x);
-  float v = 0.f;
-#pragma unroll
-  for (int k = 0; k < (1 << D); k++) {
-    const long long q = Geo<D>::nb(b, 2 * z, 2 * y, 2 * x, (k >> 2) & 1, (k >> 1) & 1, k & 1, s);
-    v += __bfloat162float(in[q * kC + c]);
-  }
-  out[i] = __float2bfloat16(v * (1.f / (1 << D)));
-}
+struct PoolFwd {
+  static constexpr int kDepth = D == 3 ? 3 : 5;
+  int nlev;                 // levels written
+  int side[kDepth + 1];     // side[0]: of `in`
+  const bf16* in;
+  bf16* out[kDepth + 1];    // out[1 .. nlev]
+};
 
-// Half-pixel linear source position of output index i (m source points, n out).
-__device__ __forceinline__ void bilin(int i, int m, int n, int& i0, int& i1, float& lam) {
-  float src = ((float)i + 0.5f) * (float)m / (float)n - 0.5f;
-  if (src < 0.f) src = 0.f;
-  i0 = (int)floorf(src);
-  if (i0 > m - 1) i0 = m - 1;
-  i1 = min(i0 + 1, m - 1);
-  lam = src - (float)i0;
+template <int D>
+__global__ void __launch_bounds__(256) pool_chain_fwd(PoolFwd<D> pf) {
+  constexpr int kDepth = PoolFwd<D>::kDepth;
+  constexpr int kHalf = 1 << (kDepth - 1);  // level-1 points of a block per axis
+  constexpr int kPts1 = D == 3 ? kHalf * kHalf * kHalf : kHalf * kHalf;
+  __shared__ __align__(16) bf16 buf[2][kPts1 * kC];
+  // block coordinates (x fastest) and batch
+  const int bps = (pf.side[1] + kHalf - 1) / kHalf;
+  int r = blockIdx.x;
+  const int bx = r % bps;
+  r /= bps;
+  const int by = r % bps;
+  r /= bps;
+  const int bz = D == 3 ? r % bps : 0;
+  const int b = D == 3 ? r / bps : r;
+  for (int l = 1; l <= pf.nlev; l++) {
+    const int w = kHalf >> (l - 1);  // the block's points of level l per axis
+    const int so = pf.side[l], si = pf.side[l - 1];
+    const int pts = D == 3 ? w * w * w : w * w;
+    const bf16* __restrict__ prev = buf[(l - 1) & 1];
+    bf16* __restrict__ mine = buf[l & 1];
+    for (int i = threadIdx.x; i < pts * 4; i += 256) {
+      const int q = (i & 3) * 8, p = i >> 2;
+      const int lx = p % w, ly = (p / w) % w, lz = D == 3 ? p / (w * w) : 0;
+      const int x = bx * w + lx, y = by * w + ly, z = bz * w + lz;
+      if (x >= so || y >= so || (D == 3 && z >= so)) continue;
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < 8; e++) v[e] = 0.f;
+#pragma unroll
+      for (int k = 0; k < (1 << D); k++) {
+        const int dz = (k >> 2) & 1, dy = (k >> 1) & 1, dx = k & 1;
+        uint4 u;
+        if (l == 1) {
+          const int f = D == 3 ? ((b * si + 2 * z + dz) * si + 2 * y + dy) * si + 2 * x + dx
+                               : (b * si + 2 * y + dy) * si + 2 * x + dx;
+          u = *reinterpret_cast<const uint4*>(pf.in + (long long)f * kC + q);
+        } else {
+          const int f = ((2 * lz + dz) * 2 * w + 2 * ly + dy) * 2 * w + 2 * lx + dx;
+          u = *reinterpret_cast<const uint4*>(prev + f * kC + q);
+        }
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          const float2 t = __bfloat1622float2(h[e]);
+          v[2 * e] += t.x;
+          v[2 * e + 1] += t.y;
+        }
+      }
+      uint4 o;
+      __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&o);
+      constexpr float sc = 1.f / (1 << D);
+#pragma unroll
+      for (int e = 0; e < 4; e++)
+        h[e] = __floats2bfloat162_rn(v[2 * e] * sc, v[2 * e + 1] * sc);
+      const int f = D == 3 ? ((b * so + z) * so + y) * so + x : (b * so + y) * so + x;
+      *reinterpret_cast<uint4*>(pf.out[l] + (long long)f * kC + q) = o;
+      *reinterpret_cast<uint4*>(mine + p * kC + q) = o;
+    }
+    __syncthreads();
+  }
 }
 
 struct Levels {
   const bf16* z[kMaxLevels];
+  const float2* tab[kMaxLevels];  // half-pixel source of each fine index: (weight of i0 + 1, i0)
   int side[kMaxLevels];
   int L;
 };
 
 // s[p][c] = sum_l upsample(z_l)[p][c]  (bilinear in 2D, trilinear in 3D);
-// four threads per point, eight channels (16 bytes) each, so the
-// interpolation weights are computed once per 8 channels
+// four threads per point, eight channels (16 bytes) each; the source positions
+// come from the levels' tables (an IEEE division per axis, level and thread
+// otherwise)
 template <int D>
 __global__ void upsum_fwd(int B, int n, Levels lv, bf16* __restrict__ s) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -177,11 +213,12 @@ __global__ void upsum_fwd(int B, int n, Levels lv, bf16* __restrict__ s) {
   }
   for (int l = 1; l < lv.L; l++) {
     const int m = lv.side[l];
-    int z0 = 0, z1 = 0, y0, y1, x0, x1;
-    float lz = 0.f, ly, lx;
-    if (D == 3) bilin(z, m, n, z0, z1, lz);
-    bilin(y, m, n, y0, y1, ly);
-    bilin(x, m, n, x0, x1, lx);
+    const float2* __restrict__ tab = lv.tab[l];
+    const float2 tz = D == 3 ? __ldg(tab + z) : make_float2(0.f, 0.f);
+    const float2 ty = __ldg(tab + y), tx = __ldg(tab + x);
+    const float lz = tz.x, ly = ty.x, lx = tx.x;
+    const int z0 = __float_as_int(tz.y), y0 = __float_as_int(ty.y), x0 = __float_as_int(tx.y);
+    const int z1 = min(z0 + 1, m - 1), y1 = min(y0 + 1, m - 1), x1 = min(x0 + 1, m - 1);
 #pragma unroll
     for (int k = 0; k < (1 << D); k++) {
       const int zz = (k >> 2) & 1 ? z1 : z0, yy = (k >> 1) & 1 ? y1 : y0, xx = k & 1 ? x1 : x0;
@@ -611,16 +648,37 @@ __global__ void mask_to_bf16(long long count, const float* __restrict__ g,
 // here so the parameters keep the documented order (T taps).
 //   kind 0 (32->32): part index (tap*32 + k)*32 + o  -> param (o*32 + k)*T + tap; bias 1024 T + o
 //   kind 1/2 (1-ch): part index c*T + tap (+ 32 T + c bias) -> same order
-__global__ void __launch_bounds__(256) reduce_wgrad(const float* __restrict__ part, int nparts,
-                                                    int stride, int kind, int T,
-                                                    float* __restrict__ gw,
-                                                    float* __restrict__ gb) {
+// One launch for all convolutions of the network (one per convolution cost 5 us
+// each, mostly latency).  With the coarse levels' convolutions and the pooling
+// levels in shared launches, and the upsampling's tables: 1245 -> 1120 us at 256^2 x
+// 8, the learned guess at 256^2 272 -> 221 us: job k's outputs on the CTAs first[k] .. first[k+1]-1.
+struct ReduceJob {
+  const float* part;
+  float *gw, *gb;
+  int nparts, stride, kind;
+};
+struct ReduceJobs {
+  static constexpr int kMost = kMaxLevels + kMaxExtra + 3;
+  int n;
+  int first[kMost + 1];
+  ReduceJob job[kMost];
+};
+
+__global__ void __launch_bounds__(256) reduce_wgrad(const __grid_constant__ ReduceJobs jobs,
+                                                    int T) {
+  int jb = 0;
+  while (jb + 1 < jobs.n && (int)blockIdx.x >= jobs.first[jb + 1]) jb++;
+  const float* __restrict__ part = jobs.job[jb].part;
+  float* __restrict__ gw = jobs.job[jb].gw;
+  float* __restrict__ gb = jobs.job[jb].gb;
+  const int nparts = jobs.job[jb].nparts, stride = jobs.job[jb].stride;
+  const int kind = jobs.job[jb].kind;
   // 32 outputs per CTA (lane = output), the CTA partials split over the 8 warps
   // (coalesced rows), four independent sums per lane so that four loads are in
   // flight, all added in a fixed order (FP32: the FP64 pipe of this GPU is slow)
   __shared__ float red[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int i = blockIdx.x * 32 + lane;
+  const int i = ((int)blockIdx.x - jobs.first[jb]) * 32 + lane;
   const int nw = kind == 0 ? T * kC * kC : T * kC;
   const int nb = kind == 0 ? kC : (kind == 1 ? kC : 1);
   float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
@@ -656,7 +714,7 @@ __global__ void __launch_bounds__(256) reduce_wgrad(const float* __restrict__ pa
 // viewed as (outer, n, inner) -> (outer, m, inner):
 //   out[o][j][c] = sum_x U[x][j] in[o][x][c],  U[x][j] = the weight of coarse j
 // in fine x's half-pixel interpolation, read from the level's sparse rows
-// (built once on the host with the same arithmetic as bilin).  The
+// (built once on the host with the arithmetic of the forward tables).  The
 // D-dimensional transpose is D such passes, one per axis.
 
 // One axis of one level; the levels' x-axis passes where a fine row is too long
@@ -1008,13 +1066,17 @@ cudaError_t net_create(Net& net, int n, int bmax, unsigned long long seed, int d
   for (int l = 1; l < L; l++) {
     const int m = net.side[l];
     std::vector<std::vector<std::pair<int, float>>> rows(m);
+    std::vector<float2> tab(n);
     for (int x = 0; x < n; x++) {
-      float src = ((float)x + 0.5f) * (float)m / (float)n - 0.5f;  // as bilin
+      // half-pixel source position of fine index x (m coarse points, n fine ones)
+      float src = ((float)x + 0.5f) * (float)m / (float)n - 0.5f;
       if (src < 0.f) src = 0.f;
       int i0 = (int)floorf(src);
       if (i0 > m - 1) i0 = m - 1;
       const int i1 = i0 + 1 < m - 1 ? i0 + 1 : m - 1;
       const float lam = src - (float)i0;
+      tab[x].x = lam;
+      memcpy(&tab[x].y, &i0, sizeof(int));
       if (i0 == i1) {
         rows[i0].push_back({x, (1.f - lam) + lam});
       } else {
@@ -1034,6 +1096,8 @@ cudaError_t net_create(Net& net, int n, int bmax, unsigned long long seed, int d
     NN_CK(cudaMalloc(&net.up_ptr[l], sizeof(int) * (m + 1)));
     NN_CK(cudaMalloc(&net.up_idx[l], sizeof(int) * idx.size()));
     NN_CK(cudaMalloc(&net.up_w[l], sizeof(float) * wt.size()));
+    NN_CK(cudaMalloc(&net.up_tab[l], sizeof(float2) * n));
+    NN_CK(cudaMemcpy(net.up_tab[l], tab.data(), sizeof(float2) * n, cudaMemcpyHostToDevice));
     NN_CK(cudaMemcpy(net.up_ptr[l], ptr.data(), sizeof(int) * (m + 1), cudaMemcpyHostToDevice));
     NN_CK(cudaMemcpy(net.up_idx[l], idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice));
     NN_CK(cudaMemcpy(net.up_w[l], wt.data(), sizeof(float) * wt.size(), cudaMemcpyHostToDevice));
@@ -1072,7 +1136,9 @@ cudaError_t net_create(Net& net, int n, int bmax, unsigned long long seed, int d
     NN_CK(cudaFuncSetAttribute(conv1_wgrad<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                conv1_wgrad_smem<2>(n)));
   }
-  NN_CK(cudaMalloc(&net.wgrad_part, sizeof(float) * (long long)net.wparts * (per + kC)));
+  // one area per 32 -> 32 convolution and per 1-channel one (reduced together)
+  NN_CK(cudaMalloc(&net.wgrad_part,
+                   sizeof(float) * (nconv + 2) * (long long)net.wparts * (per + kC)));
   const long long pix = (long long)bmax * pts(n);
   NN_CK(cudaMalloc(&net.gy, sizeof(float) * pix));
   NN_CK(cudaMalloc(&net.loss_part, sizeof(float) * 1024));
@@ -1104,6 +1170,7 @@ void net_destroy(Net& net) {
     cudaFree(net.up_ptr[l]);
     cudaFree(net.up_idx[l]);
     cudaFree(net.up_w[l]);
+    cudaFree(net.up_tab[l]);
   }
   cudaFree(net.s);
   cudaFree(net.e);
@@ -1153,34 +1220,50 @@ cudaError_t forward_t(Net& net, int B, const float* u, float* y, cudaStream_t s)
   conv_in_fwd<D><<<nblk(pix, 256), 256, 0, s>>>(B, n, u, net.master + net.off_w[0],
                                                  net.master + net.off_b[0], net.a0);
   note_launches(1);
-  for (int l = 1; l < L; l++) {
-    const int sp = net.side[l - 1];
-    const bf16* src = l == 1 ? net.a0 : net.pool[l - 1];
-    const long long cnt = B * Geo<D>::pts(net.side[l]) * kC;
-    pool2_fwd<D><<<nblk(cnt, 256), 256, 0, s>>>(B, sp, src, net.pool[l]);
+  for (int l0 = 0; l0 + 1 < L; l0 += PoolFwd<D>::kDepth) {
+    PoolFwd<D> pf;
+    pf.nlev = std::min(L - 1 - l0, PoolFwd<D>::kDepth);
+    pf.in = l0 == 0 ? net.a0 : net.pool[l0];
+    pf.side[0] = net.side[l0];
+    for (int l = 1; l <= pf.nlev; l++) {
+      pf.side[l] = net.side[l0 + l];
+      pf.out[l] = net.pool[l0 + l];
+    }
+    constexpr int half = 1 << (PoolFwd<D>::kDepth - 1);
+    const int bps = (pf.side[1] + half - 1) / half;
+    pool_chain_fwd<D><<<(unsigned)(B * (D == 3 ? bps : 1) * bps * bps), 256, 0, s>>>(pf);
     note_launches(1);
   }
+  ConvJob jobs[kMaxLevels];
   for (int l = 0; l < L; l++) {
-    NN_CK(launch_conv32_mma(D, 0, B, net.side[l], l == 0 ? net.a0 : net.pool[l],
-                            net.wqT + per * l, net.master + net.off_b[1 + l], 1, 1, net.z[l],
-                            nullptr, nullptr, nullptr, nullptr, s));
+    jobs[l].H = net.side[l];
+    jobs[l].in = l == 0 ? net.a0 : net.pool[l];
+    jobs[l].wop = net.wqT + per * l;
+    jobs[l].bias = net.master + net.off_b[1 + l];
+    jobs[l].zo = net.z[l];
   }
+  NN_CK(launch_conv32(D, 0, B, L, jobs, 1, 1, s));
   Levels lv;
   lv.L = L;
   for (int l = 0; l < L; l++) {
     lv.z[l] = net.z[l];
+    lv.tab[l] = net.up_tab[l];
     lv.side[l] = net.side[l];
   }
   upsum_fwd<D><<<nblk(pix * 4, 256), 256, 0, s>>>(B, n, lv, net.s);
   note_launches(1);
-  NN_CK(launch_conv32_mma(D, 1, B, n, net.s, net.wqT + per * L, net.master + net.off_b[L + 1], 2,
-                          1, net.e, net.t, net.s, nullptr, nullptr, s));
-  const bf16* cur = net.t;
-  for (int r = 0; r < net.extra_active; r++) {  // grown residual blocks
-    NN_CK(launch_conv32_mma(D, 1, B, n, cur, net.wqT + per * (L + 1 + r),
-                            net.master + net.off_rb[r], 2, 1, net.te[r], net.tt[r], cur, nullptr,
-                            nullptr, s));
-    cur = net.tt[r];
+  // dilated residual blocks: the first, then the grown ones
+  const bf16* cur = net.s;
+  for (int r = -1; r < net.extra_active; r++) {
+    ConvJob j;
+    j.H = n;
+    j.in = j.resid = cur;
+    j.wop = net.wqT + per * (L + 1 + r);
+    j.bias = net.master + (r < 0 ? net.off_b[L + 1] : net.off_rb[r]);
+    j.zo = r < 0 ? net.e : net.te[r];
+    j.to = r < 0 ? net.t : net.tt[r];
+    NN_CK(launch_conv32(D, 1, B, 1, &j, 2, 1, s));
+    cur = j.to;
   }
   conv_out_fwd<D><<<nblk(pix, 256), 256, 0, s>>>(B, n, cur, net.master + net.off_w[L + 2],
                                                   net.master + net.off_b[L + 2], y);
@@ -1198,6 +1281,37 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
   const long long per = (long long)T * kC * kC;
   const int P = net.wparts;
   const int stride = (int)(per + kC);
+  // the partial weight gradients of every convolution, reduced together at the end
+  ReduceJobs rj;
+  rj.n = 0;
+  auto reduce_later = [&](const float* part, int nparts, int st, int kind, float* gw, float* gb) {
+    const int outs = kind == 0 ? (int)per + kC : T * kC + (kind == 1 ? kC : 1);
+    rj.job[rj.n] = ReduceJob{part, gw, gb, nparts, st, kind};
+    rj.first[rj.n + 1] = (rj.n == 0 ? 0 : rj.first[rj.n]) + (int)nblk(outs, 32);
+    if (rj.n == 0) rj.first[0] = 0;
+    rj.n++;
+  };
+  auto conv_part = [&](int c) { return net.wgrad_part + (long long)c * P * stride; };
+  const int nconv = L + 1 + net.extra_max;
+  auto data_grad = [&](int H, const bf16* gz, int c, int dil, float* fo, const float* addend) {
+    ConvJob j;
+    j.H = H;
+    j.in = gz;
+    j.wop = net.wq + per * c;
+    j.fo = fo;
+    j.addend = addend;
+    return launch_conv32(D, 2, B, 1, &j, dil, -1, s);
+  };
+  auto weight_grad = [&](const bf16* in, const bf16* gz, int c, float* gw, float* gb) {
+    WgradJob j;
+    j.H = n;
+    j.in = in;
+    j.g = gz;
+    j.part = conv_part(c);
+    const cudaError_t e = launch_wgrad(D, B, 1, &j, 2, stride, P, s);
+    if (e == cudaSuccess) reduce_later(j.part, j.nparts, stride, 0, gw, gb);
+    return e;
+  };
   // loss and dL/dy
   const int lparts = 256;
   mse_grad<<<lparts, 256, 0, s>>>(pix, 1.f / (float)pix, tscale, tscale_dev, y, target, net.gy,
@@ -1211,12 +1325,10 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
   const int P1 = P, stride1 = kC * (T + 1);
   const int smem1 = conv1_wgrad_smem<D>(n);
   conv1_wgrad<0, D><<<P1, kW1Threads, smem1, s>>>(B, n, net.gy, tfin, nullptr, nullptr, nullptr,
-                                                  nullptr, net.wgrad_part, stride1);
+                                                  nullptr, conv_part(nconv), stride1);
   note_launches(1);
-  reduce_wgrad<<<nblk(T * kC + 1, 32), 256, 0, s>>>(net.wgrad_part, P1, stride1, 2, T,
-                                                     net.grad + net.off_w[L + 2],
-                                                     net.grad + net.off_b[L + 2]);
-  note_launches(1);
+  reduce_later(conv_part(nconv), P1, stride1, 2, net.grad + net.off_w[L + 2],
+               net.grad + net.off_b[L + 2]);
   // the first masked use of g_t (the last grown block's, else the residual
   // block's) is written by the same kernel
   const bf16* mask0 = net.extra_active > 0 ? net.te[net.extra_active - 1] : net.e;
@@ -1236,13 +1348,9 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
         mask_to_bf16<<<nblk((full) / 8, 256), 256, 0, s>>>(full, gcur, net.te[r], net.g_bf);
         note_launches(1);
       }
-      NN_CK(launch_wgrad_mma(D, B, n, tin, net.g_bf, 2, net.wgrad_part, stride, P, s));
-      reduce_wgrad<<<nblk(per + kC, 32), 256, 0, s>>>(net.wgrad_part, P, stride, 0, T,
-                                                       net.grad + net.off_rw[r],
-                                                       net.grad + net.off_rb[r]);
-      note_launches(1);
-      NN_CK(launch_conv32_mma(D, 2, B, n, net.g_bf, net.wq + per * (L + 1 + r), nullptr, 2, -1,
-                              nullptr, nullptr, nullptr, gnext, gcur, s));
+      NN_CK(weight_grad(tin, net.g_bf, L + 1 + r, net.grad + net.off_rw[r],
+                        net.grad + net.off_rb[r]));
+      NN_CK(data_grad(n, net.g_bf, L + 1 + r, 2, gnext, gcur));
       std::swap(gcur, gnext);
     }
     if (gcur != net.g_t)
@@ -1253,13 +1361,8 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
     mask_to_bf16<<<nblk((full) / 8, 256), 256, 0, s>>>(full, net.g_t, net.e, net.g_bf);
     note_launches(1);
   }
-  NN_CK(launch_wgrad_mma(D, B, n, net.s, net.g_bf, 2, net.wgrad_part, stride, P, s));
-  reduce_wgrad<<<nblk(per + kC, 32), 256, 0, s>>>(net.wgrad_part, P, stride, 0, T,
-                                                   net.grad + net.off_w[L + 1],
-                                                   net.grad + net.off_b[L + 1]);
-  note_launches(1);
-  NN_CK(launch_conv32_mma(D, 2, B, n, net.g_bf, net.wq + per * L, nullptr, 2, -1, nullptr,
-                          nullptr, nullptr, net.g_s, net.g_t, s));
+  NN_CK(weight_grad(net.s, net.g_bf, L, net.grad + net.off_w[L + 1], net.grad + net.off_b[L + 1]));
+  NN_CK(data_grad(n, net.g_bf, L, 2, net.g_s, net.g_t));
   // pyramid levels; first the x-axis pass of every coarse level's transposed
   // upsampling, from one read of the fine gradient (g_s) into g_t (free here:
   // the residual block's gradient is already in g_s)
@@ -1313,31 +1416,35 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
     for (int l = 1; l < L; l++) xin[l] = lv.out_off[l];
     other_axes(1, L, xin);
   }
-  for (int l = 0; l < L; l++) {
-    const int sd = net.side[l];
-    const bf16* gz = net.g_bf;
-    if (l > 0) {
-      if (!fused_x) {  // (rows too long to stage: the level's own passes)
-        upsample_bwd_axis<<<nblk(rows * sd * kC, 256), 256, 0, s>>>(
-            rows, n, sd, kC, net.up_ptr[l], net.up_idx[l], net.up_w[l], net.g_s, net.g_t);
-        note_launches(1);
-        const long long xin[kMaxLevels] = {};
-        other_axes(l, l + 1, xin);
-      }
-      gz = net.g_bl + (net.lvl_off[l] - net.lvl_off[1]);
-    } else {
-      const long long lp = B * Geo<D>::pts(sd);
-      mask_to_bf16<<<nblk((lp * kC) / 8, 256), 256, 0, s>>>(lp * kC, net.g_s, net.z[0], net.g_bf);
+  if (!fused_x) {  // (rows too long to stage: each level's own passes)
+    for (int l = 1; l < L; l++) {
+      upsample_bwd_axis<<<nblk(rows * net.side[l] * kC, 256), 256, 0, s>>>(
+          rows, n, net.side[l], kC, net.up_ptr[l], net.up_idx[l], net.up_w[l], net.g_s, net.g_t);
       note_launches(1);
+      const long long xin[kMaxLevels] = {};
+      other_axes(l, l + 1, xin);
     }
-    const bf16* in = l == 0 ? net.a0 : net.pool[l];
-    NN_CK(launch_wgrad_mma(D, B, sd, in, gz, 1, net.wgrad_part, stride, P, s));
-    reduce_wgrad<<<nblk(per + kC, 32), 256, 0, s>>>(net.wgrad_part, P, stride, 0, T,
-                                                     net.grad + net.off_w[1 + l],
-                                                     net.grad + net.off_b[1 + l]);
-    note_launches(1);
-    NN_CK(launch_conv32_mma(D, 2, B, sd, gz, net.wq + per * l, nullptr, 1, -1, nullptr,
-                            nullptr, nullptr, net.g_pool + net.lvl_off[l], nullptr, s));
+  }
+  mask_to_bf16<<<nblk(full / 8, 256), 256, 0, s>>>(full, net.g_s, net.z[0], net.g_bf);
+  note_launches(1);
+  {
+    // every level's weight and data gradients; the coarse levels share launches
+    WgradJob wj[kMaxLevels];
+    ConvJob cj[kMaxLevels];
+    for (int l = 0; l < L; l++) {
+      const bf16* gz = l == 0 ? net.g_bf : net.g_bl + (net.lvl_off[l] - net.lvl_off[1]);
+      wj[l].H = cj[l].H = net.side[l];
+      wj[l].in = l == 0 ? net.a0 : net.pool[l];
+      wj[l].g = cj[l].in = gz;
+      wj[l].part = conv_part(l);
+      cj[l].wop = net.wq + per * l;
+      cj[l].fo = net.g_pool + net.lvl_off[l];
+    }
+    NN_CK(launch_wgrad(D, B, L, wj, 1, stride, P, s));
+    for (int l = 0; l < L; l++)
+      reduce_later(wj[l].part, wj[l].nparts, stride, 0, net.grad + net.off_w[1 + l],
+                   net.grad + net.off_b[1 + l]);
+    NN_CK(launch_conv32(D, 2, B, L, cj, 1, -1, s));
   }
   // pooling chain: the gradient of p_{l-1} collects 1/2^D of p_l's
   if (L > 2) {
@@ -1354,11 +1461,11 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
   // (the ReLU mask of a0 is applied inside the weight-gradient kernel)
   conv1_wgrad<1, D><<<P1, kW1Threads, smem1, s>>>(
       B, n, nullptr, nullptr, net.g_pool + net.lvl_off[0],
-      L > 1 ? net.g_pool + net.lvl_off[1] : nullptr, net.a0, u, net.wgrad_part, stride1);
+      L > 1 ? net.g_pool + net.lvl_off[1] : nullptr, net.a0, u, conv_part(nconv + 1), stride1);
   note_launches(1);
-  reduce_wgrad<<<nblk(T * kC + kC, 32), 256, 0, s>>>(net.wgrad_part, P1, stride1, 1, T,
-                                                      net.grad + net.off_w[0],
-                                                      net.grad + net.off_b[0]);
+  reduce_later(conv_part(nconv + 1), P1, stride1, 1, net.grad + net.off_w[0],
+               net.grad + net.off_b[0]);
+  reduce_wgrad<<<rj.first[rj.n], 256, 0, s>>>(rj, T);
   note_launches(1);
   return cudaGetLastError();
 }

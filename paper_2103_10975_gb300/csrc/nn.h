@@ -92,18 +92,29 @@ struct Net {
   int* up_ptr[kMaxLevels] = {};
   int* up_idx[kMaxLevels] = {};
   float* up_w[kMaxLevels] = {};
+  float2* up_tab[kMaxLevels] = {};           // per fine index: (weight of i0 + 1, i0 as bits)
   long long pyr = 0;                         // sum of level sizes (pixels) per sample
   int wparts = 0;                            // CTAs of the weight-gradient kernels
   TrainCtr* ctr = nullptr;                   // device state of the training phase
 };
 
-// Tensor-core 32 -> 32 convolution (dim 2: 3x3, dim 3: 3x3x3; mode 0:
+// Tensor-core 32 -> 32 convolutions (dim 2: 3x3, dim 3: 3x3x3; mode 0:
 // relu(conv + b) -> zo; 1: e = relu(conv + b) -> zo and resid + e -> to;
-// 2: conv (+ addend) -> fo in FP32).  wop is [tap][n][k].
-cudaError_t launch_conv32_mma(int dim, int mode, int B, int H, const __nv_bfloat16* in,
-                              const __nv_bfloat16* wop, const float* bias, int dil, int sign,
-                              __nv_bfloat16* zo, __nv_bfloat16* to, const __nv_bfloat16* resid,
-                              float* fo, const float* addend, cudaStream_t s);
+// 2: conv (+ addend) -> fo in FP32) on grids of side H.  wop is [tap][n][k].
+// The jobs of a call are independent; those on the mma.sync kernel share a launch.
+struct ConvJob {
+  int H = 0;
+  const __nv_bfloat16* in = nullptr;
+  const __nv_bfloat16* wop = nullptr;
+  const float* bias = nullptr;
+  __nv_bfloat16* zo = nullptr;
+  __nv_bfloat16* to = nullptr;
+  const __nv_bfloat16* resid = nullptr;
+  float* fo = nullptr;
+  const float* addend = nullptr;
+};
+cudaError_t launch_conv32(int dim, int mode, int B, int njobs, const ConvJob* jobs, int dil,
+                          int sign, cudaStream_t s);
 // The same convolution on the fifth-generation tensor cores (tcgen05.mma into
 // tensor memory, operands by TMA), for 2D and 3D grids with at least 128 points
 // per row (the environment variable MLGMRES_TC_MIN_ROW lowers the threshold).
@@ -120,13 +131,21 @@ cudaError_t conv32_tc_setup();
 cudaError_t conv32_mma_setup();
 // 1 if a tcgen05 convolution tile timed out waiting for its MMAs (0 otherwise).
 int conv32_tc_error();
-// Tensor-core weight gradient partials of a 32 -> 32 convolution (nparts CTAs):
+// Tensor-core weight gradient partials of 32 -> 32 convolutions (at most nparts
+// CTAs each; jobs[k].nparts receives how many partials job k wrote):
 // part[cta][(tap*32 + k)*32 + o] and the bias sums at 1024 T + o.  Grids whose
 // rows qualify for the tcgen05 convolution (conv32_tc_applies) take
-// launch_wgrad_tc (tcgen05.mma with the pixels as the reduction dimension).
-cudaError_t launch_wgrad_mma(int dim, int B, int H, const __nv_bfloat16* in,
-                             const __nv_bfloat16* g, int dil, float* part, int stride, int nparts,
-                             cudaStream_t s);
+// launch_wgrad_tc (tcgen05.mma with the pixels as the reduction dimension); the
+// others share a launch.
+struct WgradJob {
+  int H = 0;
+  const __nv_bfloat16* in = nullptr;
+  const __nv_bfloat16* g = nullptr;
+  float* part = nullptr;
+  int nparts = 0;
+};
+cudaError_t launch_wgrad(int dim, int B, int njobs, WgradJob* jobs, int dil, int stride,
+                         int nparts, cudaStream_t s);
 cudaError_t launch_wgrad_tc(int dim, int B, int H, const __nv_bfloat16* in,
                             const __nv_bfloat16* g, int dil, float* part, int stride, int nparts,
                             cudaStream_t s);

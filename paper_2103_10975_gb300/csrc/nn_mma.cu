@@ -91,21 +91,44 @@ __device__ __forceinline__ void decode_row(long long row, int n, int& b, int& z,
 
 enum { kRelu = 0, kResid = 1, kF32 = 2 };
 
+// The convolutions of one launch (the coarse pyramid levels share one: alone,
+// each leaves most SMs idle and costs its launch): job k runs on the CTAs
+// first[k] .. first[k+1]-1.
+struct ConvJobs {
+  int n;
+  int first[kMaxLevels + 1];
+  ConvJob job[kMaxLevels];
+};
+struct WgradJobs {
+  int n;
+  int first[3 * kMaxLevels + 1];
+  int tz[3 * kMaxLevels];
+  int job_of[3 * kMaxLevels];
+  WgradJob job[kMaxLevels];
+};
+
 template <int D>
 constexpr int conv_smem_bytes() {
   return (int)sizeof(bf16) * ((D == 3 ? 27 : 9) * kC * kPix + (D == 3 ? 9 : 3) * kTileW * kPix);
 }
 
 template <int MODE, int D>
-__global__ void __launch_bounds__(128) conv32_mma(int B, int H, const bf16* __restrict__ in,
-                                                  const bf16* __restrict__ wop,
-                                                  const float* __restrict__ bias, int dil,
-                                                  int sign, bf16* __restrict__ zo,
-                                                  bf16* __restrict__ to,
-                                                  const bf16* __restrict__ resid,
-                                                  float* __restrict__ fo,
-                                                  const float* __restrict__ addend) {
+__global__ void __launch_bounds__(128) conv32_mma(const __grid_constant__ ConvJobs jobs, int B,
+                                                  int dil, int sign) {
   constexpr int T = D == 3 ? 27 : 9;
+  int jb = 0;
+  while (jb + 1 < jobs.n && (int)blockIdx.x >= jobs.first[jb + 1]) jb++;
+  const ConvJob& J = jobs.job[jb];
+  const int H = J.H;
+  const bf16* __restrict__ in = J.in;
+  const bf16* __restrict__ wop = J.wop;
+  const float* __restrict__ bias = J.bias;
+  bf16* __restrict__ zo = J.zo;
+  bf16* __restrict__ to = J.to;
+  const bf16* __restrict__ resid = J.resid;
+  float* __restrict__ fo = J.fo;
+  const float* __restrict__ addend = J.addend;
+  const int cta = blockIdx.x - jobs.first[jb], nctas = jobs.first[jb + 1] - jobs.first[jb];
   extern __shared__ __align__(16) unsigned char nn_smem[];
   bf16* ws = reinterpret_cast<bf16*>(nn_smem);   // [tap][n][k]
   bf16* tile = ws + T * kC * kPix;               // [r][c][k]
@@ -126,7 +149,7 @@ __global__ void __launch_bounds__(128) conv32_mma(int B, int H, const bf16* __re
   long long nrows = (long long)B * H;
   if (D == 3) nrows *= H;
   const long long ntiles = nrows * tpr;
-  for (long long tIdx = blockIdx.x; tIdx < ntiles; tIdx += gridDim.x) {
+  for (long long tIdx = cta; tIdx < ntiles; tIdx += nctas) {
     const int tx = (int)(tIdx % tpr);
     int b, z, y;
     decode_row<D>(tIdx / tpr, H, b, z, y);
@@ -208,10 +231,17 @@ __global__ void __launch_bounds__(128) conv32_mma(int B, int H, const bf16* __re
 // writes them as its partial (layout (tap*32 + k)*32 + o, tap = tz*9 + local
 // tap in 3D; bias at T*1024 + o, written by the tz = 0 launch).
 template <int D>
-__global__ void __launch_bounds__(128) wgrad_mma(int B, int H, const bf16* __restrict__ in,
-                                                 const bf16* __restrict__ g, int dil, int tz,
-                                                 float* __restrict__ part, int stride) {
+__global__ void __launch_bounds__(128) wgrad_mma(const __grid_constant__ WgradJobs jobs, int B,
+                                                 int dil, int stride) {
   constexpr int T = D == 3 ? 27 : 9;
+  int jb = 0;
+  while (jb + 1 < jobs.n && (int)blockIdx.x >= jobs.first[jb + 1]) jb++;
+  const WgradJob& J = jobs.job[jobs.job_of[jb]];
+  const int H = J.H, tz = jobs.tz[jb];
+  const bf16* __restrict__ in = J.in;
+  const bf16* __restrict__ g = J.g;
+  const int cta = blockIdx.x - jobs.first[jb], nctas = jobs.first[jb + 1] - jobs.first[jb];
+  const bool biases = D == 2 || tz == 0;  // this launch range's CTAs form the bias sums
   __shared__ __align__(16) bf16 tile[3 * kTileW * kPix];
   __shared__ __align__(16) bf16 gt[kTileP * kPix];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -222,12 +252,12 @@ __global__ void __launch_bounds__(128) wgrad_mma(int B, int H, const bf16* __res
     for (int j = 0; j < 9; j++)
 #pragma unroll
       for (int e = 0; e < 4; e++) acc[mt][j][e] = 0.f;
-  float bsum = 0.f;  // thread t < 32: bias sum of channel t
+  float bsum = 0.f;  // thread t: bias sum of channel t % 32 over a quarter of the pixels
   const int tpr = (H + kTileP - 1) / kTileP;
   long long nrows = (long long)B * H;
   if (D == 3) nrows *= H;
   const long long ntiles = nrows * tpr;
-  for (long long tIdx = blockIdx.x; tIdx < ntiles; tIdx += gridDim.x) {
+  for (long long tIdx = cta; tIdx < ntiles; tIdx += nctas) {
     const int tx = (int)(tIdx % tpr);
     int b, z, y;
     decode_row<D>(tIdx / tpr, H, b, z, y);
@@ -246,8 +276,10 @@ __global__ void __launch_bounds__(128) wgrad_mma(int B, int H, const bf16* __res
       *reinterpret_cast<uint4*>(gt + p * kPix + q * 8) = v;
     }
     __syncthreads();
-    if (threadIdx.x < kC) {
-      for (int p = 0; p < kTileP; p++) bsum += __bfloat162float(gt[p * kPix + threadIdx.x]);
+    if (biases) {
+#pragma unroll
+      for (int p = 0; p < kTileP / 4; p++)
+        bsum += __bfloat162float(gt[(warp * (kTileP / 4) + p) * kPix + lane]);
     }
 #pragma unroll
     for (int ks = 0; ks < kTileP / 16; ks++) {  // 16 pixels per step
@@ -282,7 +314,7 @@ __global__ void __launch_bounds__(128) wgrad_mma(int B, int H, const bf16* __res
     }
   }
   // write the partial: c0,c1 -> (o = row, n = col, col+1), c2,c3 -> o + 8
-  float* dst = part + (long long)blockIdx.x * stride;
+  float* dst = J.part + (long long)cta * stride;
   float* dw = dst + (D == 3 ? (long long)tz * 9 * kC * kC : 0);
 #pragma unroll
   for (int mt = 0; mt < 2; mt++) {
@@ -297,34 +329,42 @@ __global__ void __launch_bounds__(128) wgrad_mma(int B, int H, const bf16* __res
       }
     }
   }
-  if (threadIdx.x < kC && (D == 2 || tz == 0)) dst[T * kC * kC + threadIdx.x] = bsum;
+  if (biases) {
+    __syncthreads();  // the last tile's readers are done with gt
+    float* bs = reinterpret_cast<float*>(gt);
+    bs[threadIdx.x] = bsum;
+    __syncthreads();
+    if (threadIdx.x < kC)
+      dst[T * kC * kC + threadIdx.x] = (bs[threadIdx.x] + bs[threadIdx.x + 32]) +
+                                       (bs[threadIdx.x + 64] + bs[threadIdx.x + 96]);
+  }
 }
 
 }  // namespace
 
-template <int D>
-static cudaError_t conv_launch(int mode, int B, int H, const __nv_bfloat16* in,
-                               const __nv_bfloat16* wop, const float* bias, int dil, int sign,
-                               __nv_bfloat16* zo, __nv_bfloat16* to, const __nv_bfloat16* resid,
-                               float* fo, const float* addend, cudaStream_t s) {
-  constexpr int smem = conv_smem_bytes<D>();
+static int sm_count() {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  long long ntiles = (long long)B * H * ((H + kTileP - 1) / kTileP);
-  if (D == 3) ntiles *= H;
-  const int grid = (int)(ntiles < 8LL * nsm ? ntiles : 8LL * nsm);
+  return nsm;
+}
+
+static long long tiles_of(int dim, int B, int H) {
+  const long long t = (long long)B * H * ((H + kTileP - 1) / kTileP);
+  return dim == 3 ? t * H : t;
+}
+
+template <int D>
+static void conv_launch(int mode, const ConvJobs& js, int B, int dil, int sign, cudaStream_t s) {
+  constexpr int smem = conv_smem_bytes<D>();
+  const int grid = js.first[js.n];
   if (mode == kRelu)
-    conv32_mma<kRelu, D><<<grid, 128, smem, s>>>(B, H, in, wop, bias, dil, sign, zo, to, resid,
-                                                  fo, addend);
+    conv32_mma<kRelu, D><<<grid, 128, smem, s>>>(js, B, dil, sign);
   else if (mode == kResid)
-    conv32_mma<kResid, D><<<grid, 128, smem, s>>>(B, H, in, wop, bias, dil, sign, zo, to, resid,
-                                                   fo, addend);
+    conv32_mma<kResid, D><<<grid, 128, smem, s>>>(js, B, dil, sign);
   else
-    conv32_mma<kF32, D><<<grid, 128, smem, s>>>(B, H, in, wop, bias, dil, sign, zo, to, resid,
-                                                 fo, addend);
+    conv32_mma<kF32, D><<<grid, 128, smem, s>>>(js, B, dil, sign);
   note_launches(1);
-  return cudaGetLastError();
 }
 
 // The 3D variants need more than the default 48 KB of dynamic shared memory;
@@ -346,34 +386,69 @@ cudaError_t conv32_mma_setup() {
   return e;
 }
 
-cudaError_t launch_conv32_mma(int dim, int mode, int B, int H, const __nv_bfloat16* in,
-                              const __nv_bfloat16* wop, const float* bias, int dil, int sign,
-                              __nv_bfloat16* zo, __nv_bfloat16* to, const __nv_bfloat16* resid,
-                              float* fo, const float* addend, cudaStream_t s) {
-  if (dil < 1 || dil > kMaxDil || (dim != 2 && dim != 3)) return cudaErrorInvalidValue;
-  // full-resolution levels go to the tcgen05 kernel (tensor memory accumulators)
-  if (conv32_tc_applies(dim, H))
-    return launch_conv32_tc(dim, mode, B, H, in, wop, bias, dil, sign, zo, to, resid, fo, addend,
-                            s);
-  return dim == 3 ? conv_launch<3>(mode, B, H, in, wop, bias, dil, sign, zo, to, resid, fo,
-                                   addend, s)
-                  : conv_launch<2>(mode, B, H, in, wop, bias, dil, sign, zo, to, resid, fo,
-                                   addend, s);
+cudaError_t launch_conv32(int dim, int mode, int B, int njobs, const ConvJob* jobs, int dil,
+                          int sign, cudaStream_t s) {
+  if (dil < 1 || dil > kMaxDil || (dim != 2 && dim != 3) || njobs < 1 || njobs > kMaxLevels)
+    return cudaErrorInvalidValue;
+  ConvJobs js;
+  js.n = 0;
+  js.first[0] = 0;
+  const long long most = 8LL * sm_count();
+  for (int k = 0; k < njobs; k++) {
+    const ConvJob& J = jobs[k];
+    // full-resolution levels go to the tcgen05 kernel (tensor memory accumulators)
+    if (conv32_tc_applies(dim, J.H)) {
+      const cudaError_t e = launch_conv32_tc(dim, mode, B, J.H, J.in, J.wop, J.bias, dil, sign,
+                                             J.zo, J.to, J.resid, J.fo, J.addend, s);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
+    const long long nt = tiles_of(dim, B, J.H);
+    js.job[js.n] = J;
+    js.first[js.n + 1] = js.first[js.n] + (int)(nt < most ? nt : most);
+    js.n++;
+  }
+  if (js.n == 0) return cudaSuccess;
+  if (dim == 3)
+    conv_launch<3>(mode, js, B, dil, sign, s);
+  else
+    conv_launch<2>(mode, js, B, dil, sign, s);
+  return cudaGetLastError();
 }
 
-cudaError_t launch_wgrad_mma(int dim, int B, int H, const __nv_bfloat16* in,
-                             const __nv_bfloat16* g, int dil, float* part, int stride, int nparts,
-                             cudaStream_t s) {
-  if (dil < 1 || dil > kMaxDil || (dim != 2 && dim != 3)) return cudaErrorInvalidValue;
-  if (conv32_tc_applies(dim, H))
-    return launch_wgrad_tc(dim, B, H, in, g, dil, part, stride, nparts, s);
-  if (dim == 2) {
-    wgrad_mma<2><<<nparts, 128, 0, s>>>(B, H, in, g, dil, 1, part, stride);
-    note_launches(1);
-  } else {
-    for (int tz = 0; tz < 3; tz++) wgrad_mma<3><<<nparts, 128, 0, s>>>(B, H, in, g, dil, tz, part, stride);
-    note_launches(3);
+cudaError_t launch_wgrad(int dim, int B, int njobs, WgradJob* jobs, int dil, int stride,
+                         int nparts, cudaStream_t s) {
+  if (dil < 1 || dil > kMaxDil || (dim != 2 && dim != 3) || njobs < 1 || njobs > kMaxLevels)
+    return cudaErrorInvalidValue;
+  WgradJobs js;
+  js.n = 0;
+  js.first[0] = 0;
+  for (int k = 0; k < njobs; k++) {
+    WgradJob& J = jobs[k];
+    J.nparts = nparts;
+    if (conv32_tc_applies(dim, J.H)) {
+      const cudaError_t e = launch_wgrad_tc(dim, B, J.H, J.in, J.g, dil, J.part, stride, nparts, s);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
+    // no more partials than tiles (a coarse level's others would be zero)
+    const long long nt = tiles_of(dim, B, J.H);
+    if (nt < nparts) J.nparts = (int)nt;
+    js.job[k] = J;
+    // in 3D one range of CTAs per plane offset tz of the taps
+    for (int tz = dim == 3 ? 0 : 1; tz < (dim == 3 ? 3 : 2); tz++) {
+      js.job_of[js.n] = k;
+      js.tz[js.n] = tz;
+      js.first[js.n + 1] = js.first[js.n] + J.nparts;
+      js.n++;
+    }
   }
+  if (js.n == 0) return cudaSuccess;
+  if (dim == 2)
+    wgrad_mma<2><<<js.first[js.n], 128, 0, s>>>(js, B, dil, stride);
+  else
+    wgrad_mma<3><<<js.first[js.n], 128, 0, s>>>(js, B, dil, stride);
+  note_launches(1);
   return cudaGetLastError();
 }
 
