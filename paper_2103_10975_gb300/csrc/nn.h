@@ -116,9 +116,10 @@ struct ConvJob {
 cudaError_t launch_conv32(int dim, int mode, int B, int njobs, const ConvJob* jobs, int dil,
                           int sign, cudaStream_t s);
 // The same convolution on the fifth-generation tensor cores (tcgen05.mma into
-// tensor memory, operands by TMA), for 2D and 3D grids with at least 128 points
-// per row (the environment variable MLGMRES_TC_MIN_ROW lowers the threshold).
-bool conv32_tc_applies(int dim, int H);
+// tensor memory, operands by TMA): rows of at least 128 points (the environment
+// variable MLGMRES_TC_MIN_ROW lowers the threshold) a tile per row, shorter ones
+// in tiles over several rows where that pays.
+bool conv32_tc_applies(int dim, int B, int H, int dil);
 cudaError_t launch_conv32_tc(int dim, int mode, int B, int H, const __nv_bfloat16* in,
                              const __nv_bfloat16* wop, const float* bias, int dil, int sign,
                              __nv_bfloat16* zo, __nv_bfloat16* to, const __nv_bfloat16* resid,
@@ -146,8 +147,9 @@ struct WgradJob {
 };
 cudaError_t launch_wgrad(int dim, int B, int njobs, WgradJob* jobs, int dil, int stride,
                          int nparts, cudaStream_t s);
+// *nparts: at most that many partials in, the number written out.
 cudaError_t launch_wgrad_tc(int dim, int B, int H, const __nv_bfloat16* in,
-                            const __nv_bfloat16* g, int dil, float* part, int stride, int nparts,
+                            const __nv_bfloat16* g, int dil, float* part, int stride, int* nparts,
                             cudaStream_t s);
 
 // infer_only: allocate what forward passes need (parameters, BF16 operand

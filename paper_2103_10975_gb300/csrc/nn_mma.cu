@@ -396,8 +396,8 @@ cudaError_t launch_conv32(int dim, int mode, int B, int njobs, const ConvJob* jo
   const long long most = 8LL * sm_count();
   for (int k = 0; k < njobs; k++) {
     const ConvJob& J = jobs[k];
-    // full-resolution levels go to the tcgen05 kernel (tensor memory accumulators)
-    if (conv32_tc_applies(dim, J.H)) {
+    // most levels go to the tcgen05 kernels (tensor memory accumulators)
+    if (conv32_tc_applies(dim, B, J.H, dil)) {
       const cudaError_t e = launch_conv32_tc(dim, mode, B, J.H, J.in, J.wop, J.bias, dil, sign,
                                              J.zo, J.to, J.resid, J.fo, J.addend, s);
       if (e != cudaSuccess) return e;
@@ -426,8 +426,8 @@ cudaError_t launch_wgrad(int dim, int B, int njobs, WgradJob* jobs, int dil, int
   for (int k = 0; k < njobs; k++) {
     WgradJob& J = jobs[k];
     J.nparts = nparts;
-    if (conv32_tc_applies(dim, J.H)) {
-      const cudaError_t e = launch_wgrad_tc(dim, B, J.H, J.in, J.g, dil, J.part, stride, nparts, s);
+    if (conv32_tc_applies(dim, B, J.H, dil)) {
+      const cudaError_t e = launch_wgrad_tc(dim, B, J.H, J.in, J.g, dil, J.part, stride, &J.nparts, s);
       if (e != cudaSuccess) return e;
       continue;
     }

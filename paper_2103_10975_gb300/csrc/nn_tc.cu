@@ -21,6 +21,18 @@
 // stages of rows in flight, an MMA warp turns each stage into one of two
 // accumulators in tensor memory, and four epilogue warps read an accumulator,
 // hand it back and store the tile while the next tiles' copies and MMAs run.
+//
+// Short rows (packed tiles).  A row of fewer than 128 points fills only part of
+// such a tile.  There a plane is taken as one line of padded rows, P = H + 2 dil
+// positions each (dil zeros on either side), and a tile is 128 consecutive
+// positions of it, starting anywhere.  One box of P pixels x RS rows per 8-channel
+// block lands as exactly that line (the zeros outside the grid by the copy's own
+// fill), so a tap is again a constant shift of the operand's start,
+// (dil + sign dil (ty - 1)) P + dil + sign dil (tx - 1) positions, for every
+// position of the tile; the results at padding positions are not stored.  H / P of
+// the tensor work is useful (96% at H = 48, dil 1) where a tile per row has H /
+// 128, and a plane takes 4 copies instead of 12 per tile.
+#include <algorithm>
 #include <cstdlib>
 #include <mutex>
 #include <cuda.h>
@@ -57,6 +69,15 @@ struct TcGeo {
 };
 static_assert(kLboA >= kBox && kLboA % 128 == 0,
               "copy destinations must be 128-byte aligned and hold a box");
+
+// Geometry of a launch with packed tiles (all zero for a tile per row).
+struct TcPack {
+  int P = 0;            // positions per padded row
+  int lbo = 0;          // bytes between 8-channel blocks of a stage (128-byte multiple)
+  int box = 0;          // bytes one copy delivers: P x RS pixels of 16 bytes
+  int stages = 0;
+  int tpp = 0;          // tiles per plane
+};
 
 __device__ __forceinline__ unsigned saddr(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
@@ -111,6 +132,19 @@ __device__ __forceinline__ void tile_coords(long long tIdx, int H, int tpr, int&
   x0 = tx * kTcM;
 }
 
+// Packed tiles: plane (b, z), first row y0 and the position c0 in it where the tile
+// starts.
+template <int D>
+__device__ __forceinline__ void pack_coords(long long tIdx, int H, const TcPack& pk, int& b,
+                                            int& z, int& y0, int& c0) {
+  const unsigned t = (unsigned)tIdx, tpp = (unsigned)pk.tpp;
+  const unsigned pos = t % tpp * kTcM, r = t / tpp;
+  y0 = (int)(pos / (unsigned)pk.P);
+  c0 = (int)(pos % (unsigned)pk.P);
+  z = D == 3 ? (int)(r % (unsigned)H) : 0;
+  b = D == 3 ? (int)(r / (unsigned)H) : (int)r;
+}
+
 // Bounded mbarrier wait (2 s); false on expiry.
 __device__ __forceinline__ bool mbar_wait_tc(unsigned bar, unsigned phase) {
   if (mbar_test_tc(bar, phase)) return true;
@@ -118,6 +152,41 @@ __device__ __forceinline__ bool mbar_wait_tc(unsigned bar, unsigned phase) {
   while (!mbar_test_tc(bar, phase))
     if (globaltimer_ns() - t0 > 2000000000ull) return false;
   return true;
+}
+
+// One box: (channel c, pixel x, row y, plane z (3D), batch b).
+template <int D>
+__device__ __forceinline__ void tma_row(const CUtensorMap* tmap, unsigned dst, int c, int x,
+                                        int y, int z, int b, unsigned bar) {
+  if (D == 3)
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
+        "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(c), "r"(x), "r"(y), "r"(z), "r"(b),
+        "r"(bar)
+        : "memory");
+  else
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+        "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(bar)
+        : "memory");
+}
+
+// A packed tile's input planes (z - sd, z, z + sd in 3D) into stage buffer `as`: one
+// copy per plane and 8-channel block, from row y0 - dil and pixel -dil.
+template <int D>
+__device__ __forceinline__ void issue_pack(const CUtensorMap* tmap, unsigned as, unsigned bar,
+                                           int b, int z, int y0, int dil, int sign,
+                                           const TcPack& pk) {
+  constexpr int kPlanes = D == 3 ? 3 : 1;
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+               "r"(kPlanes * 4 * pk.box)
+               : "memory");
+  for (int tz = 0; tz < kPlanes; tz++)
+    for (int kc = 0; kc < 4; kc++)
+      tma_row<D>(tmap, as + (unsigned)((tz * 4 + kc) * pk.lbo), 8 * kc, -dil, y0 - dil,
+                 z + (D == 3 ? sign * dil * (tz - 1) : 0), b, bar);
 }
 
 // The input rows of tile (b, z, y, x0) into stage buffer `as`: per row (3 in
@@ -176,14 +245,32 @@ __device__ __forceinline__ void issue_mmas(unsigned tmem, unsigned as, unsigned 
       : "memory");
 }
 
+// The same for a packed tile that starts at position c0 of its first staged row.
+template <int D>
+__device__ __forceinline__ void issue_mmas_pack(unsigned tmem, unsigned as, unsigned ws, int c0,
+                                                int dil, int sign, unsigned bar,
+                                                const TcPack& pk) {
+  const unsigned lbo = (unsigned)pk.lbo;
+  for (int t = 0; t < TcGeo<D>::kTaps; t++) {
+    const int tx = t % 3, ty = (t / 3) % 3, tz = t / 9;
+    const int q = c0 + (dil + sign * dil * (ty - 1)) * pk.P + dil + sign * dil * (tx - 1);
+    for (int h = 0; h < 2; h++)
+      tc_mma(tmem, mdesc(as + (unsigned)(tz * 4 + h * 2) * lbo + (unsigned)q * 16u, lbo, 128),
+             mdesc(ws + t * kWBytes + h * 256, 128, 512), (t | h) ? 1u : 0u);
+  }
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+      : "memory");
+}
+
 // Warp roles of conv32_tc (192 threads): warp 0 issues the TMA copies of the
 // input rows, warp 1 issues the MMAs, warps 2..5 run the epilogue (warp w reads
 // TMEM lanes 32 (w % 4) .. +31, the pixels of its quarter of the tile).
 constexpr int kTcThreads = 192;
 
-template <int D, int MODE>
+template <int D, int MODE, bool PACK>
 __global__ void __launch_bounds__(kTcThreads) conv32_tc(const __grid_constant__ CUtensorMap tmap,
-                                                        int B, int H, const bf16* __restrict__ wop,
+                                                        const TcPack pk, int B, int H, const bf16* __restrict__ wop,
                                                         const float* __restrict__ bias, int dil,
                                                         int sign, bf16* __restrict__ zo,
                                                         bf16* __restrict__ to,
@@ -193,8 +280,8 @@ __global__ void __launch_bounds__(kTcThreads) conv32_tc(const __grid_constant__ 
                                                         int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char tc_smem[];
   using G = TcGeo<D>;
-  constexpr int kStages = G::kStages;
-  constexpr int kStageBytes = G::kStageBytes;
+  const int kStages = PACK ? pk.stages : G::kStages;
+  const int kStageBytes = PACK ? (D == 3 ? 12 : 4) * pk.lbo : G::kStageBytes;
   unsigned char* As = tc_smem;                                  // kStages stages of input rows
   unsigned char* Ws = tc_smem + kStages * kStageBytes;          // taps x 2 KB
   unsigned long long* full = reinterpret_cast<unsigned long long*>(Ws + G::kTaps * kWBytes);
@@ -240,7 +327,8 @@ __global__ void __launch_bounds__(kTcThreads) conv32_tc(const __grid_constant__ 
   const unsigned as0 = saddr(As), ws = saddr(Ws);
 
   const int tpr = (H + kTcM - 1) / kTcM;
-  const long long ntiles = (long long)B * H * tpr * (D == 3 ? H : 1);
+  const long long ntiles = PACK ? (long long)B * pk.tpp * (D == 3 ? H : 1)
+                                : (long long)B * H * tpr * (D == 3 ? H : 1);
   // this CTA's tiles: blockIdx.x + k * gridDim.x, k < K
   const long long K = ntiles > blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
 
@@ -255,9 +343,15 @@ __global__ void __launch_bounds__(kTcThreads) conv32_tc(const __grid_constant__ 
           break;
         }
         int b, z, y, x0;
-        tile_coords<D>(blockIdx.x + k * gridDim.x, H, tpr, b, z, y, x0);
-        issue_rows<D>(&tmap, as0 + (unsigned)st * kStageBytes, saddr(full + st), b, z, y, x0,
-                      dil, sign);
+        if constexpr (PACK) {
+          pack_coords<D>(blockIdx.x + k * gridDim.x, H, pk, b, z, y, x0);
+          issue_pack<D>(&tmap, as0 + (unsigned)(st * kStageBytes), saddr(full + st), b, z, y, dil,
+                        sign, pk);
+        } else {
+          tile_coords<D>(blockIdx.x + k * gridDim.x, H, tpr, b, z, y, x0);
+          issue_rows<D>(&tmap, as0 + (unsigned)(st * kStageBytes), saddr(full + st), b, z, y, x0,
+                        dil, sign);
+        }
         prog[0] = (int)(k + 1);
       }
     }
@@ -271,8 +365,15 @@ __global__ void __launch_bounds__(kTcThreads) conv32_tc(const __grid_constant__ 
         prog[1] = (int)(k + 1);
         if (k >= 2 && !mbar_wait_tc(saddr(tempty + a), (unsigned)(((k >> 1) - 1) & 1))) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        issue_mmas<D>(tmem + 32u * a, as0 + (unsigned)st * kStageBytes, ws, dil, sign,
-                      saddr(empty + st));
+        if constexpr (PACK) {
+          int b, z, y0, c0;
+          pack_coords<D>(blockIdx.x + k * gridDim.x, H, pk, b, z, y0, c0);
+          issue_mmas_pack<D>(tmem + 32u * a, as0 + (unsigned)(st * kStageBytes), ws, c0, dil, sign,
+                             saddr(empty + st), pk);
+        } else {
+          issue_mmas<D>(tmem + 32u * a, as0 + (unsigned)(st * kStageBytes), ws, dil, sign,
+                        saddr(empty + st));
+        }
         asm volatile(
             "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                 saddr(tfull + a))
@@ -321,9 +422,17 @@ __global__ void __launch_bounds__(kTcThreads) conv32_tc(const __grid_constant__ 
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(tempty + ab))
                      : "memory");
       int b, z, y, x0;
-      tile_coords<D>(blockIdx.x + k * gridDim.x, H, tpr, b, z, y, x0);
       const int p = lq * 32 + lane;
-      const int x = x0 + p;
+      int x;
+      if constexpr (PACK) {
+        pack_coords<D>(blockIdx.x + k * gridDim.x, H, pk, b, z, y, x0);
+        const unsigned q = (unsigned)(x0 + p);
+        y += (int)(q / (unsigned)pk.P);
+        x = y < H ? (int)(q % (unsigned)pk.P) : H;  // (padding: not stored)
+      } else {
+        tile_coords<D>(blockIdx.x + k * gridDim.x, H, tpr, b, z, y, x0);
+        x = x0 + p;
+      }
       if (x < H) {
         const long long pix = D == 3 ? (((long long)b * H + z) * H + y) * H + x
                                      : ((long long)b * H + y) * H + x;
@@ -426,33 +535,18 @@ __device__ __forceinline__ void tc_mma_wg(unsigned tmem, unsigned long long a,
       : "memory");
 }
 
-// One box of a row: (channel c, pixel x, row y, plane z (3D), batch b).
-template <int D>
-__device__ __forceinline__ void tma_row(const CUtensorMap* tmap, unsigned dst, int c, int x,
-                                        int y, int z, int b, unsigned bar) {
-  if (D == 3)
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
-        "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(c), "r"(x), "r"(y), "r"(z), "r"(b),
-        "r"(bar)
-        : "memory");
-  else
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-        "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(c), "r"(x), "r"(y), "r"(b), "r"(bar)
-        : "memory");
-}
-
-template <int D>
+// Packed tiles: the three taps' rows are boxes of P pixels x RSw rows from rows y0 +
+// dil (ty - 1) and pixel -dil, g's from row y0 and pixel 0 (zero at every padding
+// position, whose products then vanish), and the K-steps run from position c0.
+template <int D, bool PACK>
 __global__ void __launch_bounds__(kTcThreads) wgrad_tc(const __grid_constant__ CUtensorMap tin,
                                                        const __grid_constant__ CUtensorMap tg,
-                                                       int B, int H, int dil, int tz,
+                                                       const TcPack pk, int B, int H, int dil, int tz,
                                                        float* __restrict__ part, int stride,
                                                        int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char wg_smem[];
-  unsigned long long* full = reinterpret_cast<unsigned long long*>(wg_smem + kWgStages * kWgStageBytes);
+  const int lbo = PACK ? pk.lbo : kLboA, rowb = 4 * lbo, stageb = kWgRows * rowb;
+  unsigned long long* full = reinterpret_cast<unsigned long long*>(wg_smem + kWgStages * stageb);
   unsigned long long* empty = full + kWgStages;  // the MMAs of a stage have completed
   unsigned long long* done = empty + kWgStages;  // every MMA of the CTA has completed
   unsigned* tmem_slot = reinterpret_cast<unsigned*>(done + 1);
@@ -460,8 +554,8 @@ __global__ void __launch_bounds__(kTcThreads) wgrad_tc(const __grid_constant__ C
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the row of ones of each stage (BF16 1.0), written once; the copies never touch it
   for (int st = 0; st < kWgStages; st++) {
-    unsigned* ones = reinterpret_cast<unsigned*>(wg_smem + st * kWgStageBytes + 3 * kRowBytes);
-    for (int i = threadIdx.x; i < kRowBytes / 4; i += blockDim.x) ones[i] = 0x3F803F80u;
+    unsigned* ones = reinterpret_cast<unsigned*>(wg_smem + st * stageb + 3 * rowb);
+    for (int i = threadIdx.x; i < rowb / 4; i += blockDim.x) ones[i] = 0x3F803F80u;
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (threadIdx.x == 0) {
@@ -485,7 +579,8 @@ __global__ void __launch_bounds__(kTcThreads) wgrad_tc(const __grid_constant__ C
   const unsigned tmem = *tmem_slot;
   const unsigned as0 = saddr(wg_smem);
   const int tpr = (H + kTcM - 1) / kTcM;
-  const long long ntiles = (long long)B * H * tpr * (D == 3 ? H : 1);
+  const long long ntiles = PACK ? (long long)B * pk.tpp * (D == 3 ? H : 1)
+                                : (long long)B * H * tpr * (D == 3 ? H : 1);
   const long long K = ntiles > blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
 
   if (warp == 0) {
@@ -499,19 +594,24 @@ __global__ void __launch_bounds__(kTcThreads) wgrad_tc(const __grid_constant__ C
           break;
         }
         int b, z, y, x0;
-        tile_coords<D>(blockIdx.x + k * gridDim.x, H, tpr, b, z, y, x0);
-        const unsigned as = as0 + (unsigned)st * kWgStageBytes;
+        if constexpr (PACK) {
+          pack_coords<D>(blockIdx.x + k * gridDim.x, H, pk, b, z, y, x0);
+          x0 = 0;
+        } else {
+          tile_coords<D>(blockIdx.x + k * gridDim.x, H, tpr, b, z, y, x0);
+        }
+        const unsigned as = as0 + (unsigned)(st * stageb);
         const unsigned bar = saddr(full + st);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                     "r"(kWgTx)
+                     "r"(PACK ? 16 * pk.box : kWgTx)
                      : "memory");
         // (3D: the input rows of plane z + dil (tz - 1), zeros outside the grid)
         for (int ty = 0; ty < 3; ty++)
           for (int kc = 0; kc < 4; kc++)
-            tma_row<D>(&tin, as + ty * kRowBytes + kc * kLboA, 8 * kc, x0 - dil,
+            tma_row<D>(&tin, as + (unsigned)(ty * rowb + kc * lbo), 8 * kc, x0 - dil,
                        y + dil * (ty - 1), z + dil * (tz - 1), b, bar);
         for (int kc = 0; kc < 4; kc++)
-          tma_row<D>(&tg, as + 4 * kRowBytes + kc * kLboA, 8 * kc, x0, y, z, b, bar);
+          tma_row<D>(&tg, as + (unsigned)(4 * rowb + kc * lbo), 8 * kc, x0, y, z, b, bar);
         prog[0] = (int)(k + 1);
       }
     }
@@ -524,12 +624,17 @@ __global__ void __launch_bounds__(kTcThreads) wgrad_tc(const __grid_constant__ C
         if (!mbar_wait_tc(saddr(full + st), (unsigned)((k / kWgStages) & 1))) break;
         prog[1] = (int)(k + 1);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const unsigned as = as0 + (unsigned)st * kWgStageBytes;
+        const unsigned as = as0 + (unsigned)(st * stageb);
+        int c0 = 0;
+        if constexpr (PACK) {
+          int b, z, y0;
+          pack_coords<D>(blockIdx.x + k * gridDim.x, H, pk, b, z, y0, c0);
+        }
         for (int ks = 0; ks < kTcM / 16; ks++) {
-          const unsigned q = (unsigned)ks * 16u * 16u;  // the K-step's first pixel, in bytes
-          const unsigned long long bdesc = mdesc(as + 4 * kRowBytes + q, 128, kLboA);
+          const unsigned q = (unsigned)(c0 + ks * 16) * 16u;  // the K-step's first pixel, in bytes
+          const unsigned long long bdesc = mdesc(as + (unsigned)(4 * rowb) + q, 128, lbo);
           for (int tx = 0; tx < 3; tx++)
-            tc_mma_wg(tmem + 32u * tx, mdesc(as + (unsigned)(dil * tx) * 16u + q, 128, kLboA),
+            tc_mma_wg(tmem + 32u * tx, mdesc(as + (unsigned)(dil * tx) * 16u + q, 128, lbo),
                       bdesc, (k | ks) ? 1u : 0u);
         }
         asm volatile(
@@ -616,7 +721,58 @@ int tc_min_row() {
 
 }  // namespace
 
-bool conv32_tc_applies(int dim, int H) { return (dim == 2 || dim == 3) && H >= tc_min_row(); }
+namespace {
+
+constexpr int kSmemMost = 227 * 1024;
+
+int rup(int v, int a) { return (v + a - 1) / a * a; }
+
+// Packed tiles of a convolution, or of a weight gradient, over rows of H points:
+// false where two stages do not fit in shared memory.
+bool pack_geometry(int dim, int H, int dil, bool wgrad, TcPack* pk, int* smem) {
+  const int P = H + 2 * dil;
+  // rows a box must hold for 128 positions from any start in its first row, with
+  // the taps' shifts (a weight gradient stages each ty on its own)
+  const int last = P - 1 + kTcM - 1 + 2 * dil + (wgrad ? 0 : 2 * dil * P);
+  const int RS = last / P + 1;
+  if (P > 256 || RS > 256) return false;
+  pk->P = P;
+  pk->box = P * RS * 16;
+  pk->lbo = rup(pk->box, 128);
+  pk->tpp = (H * P + kTcM - 1) / kTcM;
+  const int fixed = wgrad ? 128 : (dim == 3 ? 27 : 9) * kWBytes + 128;
+  const int stage = (wgrad ? 4 * kWgRows : (dim == 3 ? 12 : 4)) * pk->lbo;
+  pk->stages = wgrad ? kWgStages : (fixed + 3 * stage <= kSmemMost / 2 ? 3 : 2);
+  *smem = fixed + pk->stages * stage;
+  return *smem <= kSmemMost;
+}
+
+enum { kTcNone = 0, kTcRows = 1, kTcPacked = 2 };
+
+// Which tcgen05 tiles a job takes.  Rows of 128 points and more: a tile per row
+// segment.  Shorter ones: packed tiles where they fit shared memory (3D rows of 53
+// points and more at dilation 2 do not: a tile per row, still ahead of mma.sync when a
+// third full).  In
+// 2D, levels of little work stay on the mma.sync kernel, whose levels share one
+// launch (256^2 x 8: the 64-point level and below); a launch of their own costs
+// each of them more than the tensor cores save.  Measured at 48^3 x 2 (forward and
+// backward of the network): mma.sync 2.14 ms, a tile per row 1.54, packed 1.13.
+int tc_kind(int dim, int B, int H, int dil) {
+  if (dim != 2 && dim != 3) return kTcNone;
+  if (H >= tc_min_row()) return kTcRows;
+  TcPack pk;
+  int smem = 0;
+  if (dim == 2 && (long long)B * H * H < 40000) return kTcNone;
+  if (pack_geometry(dim, H, dil, false, &pk, &smem) && pack_geometry(dim, H, dil, true, &pk, &smem))
+    return kTcPacked;
+  return 4 * H >= kTcM ? kTcRows : kTcNone;
+}
+
+}  // namespace
+
+bool conv32_tc_applies(int dim, int B, int H, int dil) {
+  return tc_kind(dim, B, H, dil) != kTcNone;
+}
 
 namespace {
 
@@ -628,30 +784,53 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn g_encode = nullptr;
 
-template <int D>
+template <int D, bool PACK>
 void set_tc_smem() {
-  cudaFuncSetAttribute(conv32_tc<D, kRelu>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       TcGeo<D>::kSmem);
-  cudaFuncSetAttribute(conv32_tc<D, kResid>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       TcGeo<D>::kSmem);
-  cudaFuncSetAttribute(conv32_tc<D, kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       TcGeo<D>::kSmem);
+  const int most = PACK ? kSmemMost : TcGeo<D>::kSmem;
+  cudaFuncSetAttribute(conv32_tc<D, kRelu, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(conv32_tc<D, kResid, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       most);
+  cudaFuncSetAttribute(conv32_tc<D, kF32, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaFuncSetAttribute(wgrad_tc<D, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       PACK ? kSmemMost : kWgSmem);
 }
 
-template <int D>
-void launch_tc(int mode, int grid, cudaStream_t s, const CUtensorMap& tm, int B, int H,
-               const bf16* wop, const float* bias, int dil, int sign, bf16* zo, bf16* to,
-               const bf16* resid, float* fo, const float* addend) {
-  constexpr int sm = TcGeo<D>::kSmem;
+template <int D, bool PACK>
+void launch_tc(int mode, int grid, int sm, cudaStream_t s, const CUtensorMap& tm, const TcPack& pk,
+               int B, int H, const bf16* wop, const float* bias, int dil, int sign, bf16* zo,
+               bf16* to, const bf16* resid, float* fo, const float* addend) {
   if (mode == kRelu)
-    conv32_tc<D, kRelu><<<grid, kTcThreads, sm, s>>>(tm, B, H, wop, bias, dil, sign, zo, to,
-                                                     resid, fo, addend, g_tc_err);
+    conv32_tc<D, kRelu, PACK><<<grid, kTcThreads, sm, s>>>(tm, pk, B, H, wop, bias, dil, sign, zo,
+                                                           to, resid, fo, addend, g_tc_err);
   else if (mode == kResid)
-    conv32_tc<D, kResid><<<grid, kTcThreads, sm, s>>>(tm, B, H, wop, bias, dil, sign, zo, to,
-                                                      resid, fo, addend, g_tc_err);
+    conv32_tc<D, kResid, PACK><<<grid, kTcThreads, sm, s>>>(tm, pk, B, H, wop, bias, dil, sign, zo,
+                                                            to, resid, fo, addend, g_tc_err);
   else
-    conv32_tc<D, kF32><<<grid, kTcThreads, sm, s>>>(tm, B, H, wop, bias, dil, sign, zo, to,
-                                                    resid, fo, addend, g_tc_err);
+    conv32_tc<D, kF32, PACK><<<grid, kTcThreads, sm, s>>>(tm, pk, B, H, wop, bias, dil, sign, zo,
+                                                          to, resid, fo, addend, g_tc_err);
+}
+
+// A tensor map over a channels-last activation, [B][H][H][32] (2D) or
+// [B][H][H][H][32] (3D), BF16, as a tensor of rank dim + 2 (channels innermost):
+// boxes of 8 channels x bx pixels x by rows.
+bool encode_boxes(CUtensorMap* tm, const bf16* p, int dim, int B, int H, int bx, int by) {
+  const cuuint64_t row = (cuuint64_t)kC * 2;  // bytes per pixel
+  const cuuint64_t h = (cuuint64_t)H;
+  const cuuint64_t dims[5] = {(cuuint64_t)kC, h, h, dim == 3 ? h : (cuuint64_t)B, (cuuint64_t)B};
+  const cuuint64_t strides[4] = {row, row * h, row * h * h, row * h * h * h};
+  const cuuint32_t box[5] = {8, (cuuint32_t)bx, (cuuint32_t)by, 1, 1};
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)(dim + 2), (void*)p, dims,
+                  strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+         CUDA_SUCCESS;
+}
+
+int tc_sm_count() {
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return nsm;
 }
 
 }  // namespace
@@ -660,10 +839,10 @@ cudaError_t conv32_tc_setup() {
   static std::mutex mu;
   std::lock_guard<std::mutex> lk(mu);
   if (g_tc_err) return cudaSuccess;
-  set_tc_smem<2>();
-  set_tc_smem<3>();
-  cudaFuncSetAttribute(wgrad_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
-  cudaFuncSetAttribute(wgrad_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+  set_tc_smem<2, false>();
+  set_tc_smem<3, false>();
+  set_tc_smem<2, true>();
+  set_tc_smem<3, true>();
   void* fn = nullptr;
   cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
   cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
@@ -690,56 +869,34 @@ cudaError_t launch_conv32_tc(int dim, int mode, int B, int H, const __nv_bfloat1
   }
   if ((dim != 2 && dim != 3) || dil < 1 || dil > 2 || ((unsigned long long)in & 15ull))
     return cudaErrorInvalidValue;
-  // the input activation, channels last: [B]([H])[H][H][32] BF16, as a tensor of
-  // rank dim + 2 (channels innermost); a copy box is 8 channels x kRows pixels of
-  // one row
+  const bool pack = tc_kind(dim, B, H, dil) == kTcPacked;
+  TcPack pk;
+  int sm = dim == 3 ? TcGeo<3>::kSmem : TcGeo<2>::kSmem;
+  if (pack && !pack_geometry(dim, H, dil, false, &pk, &sm)) return cudaErrorInvalidValue;
   CUtensorMap tm;
-  const cuuint64_t row = (cuuint64_t)kC * 2;  // bytes per pixel
-  const cuuint64_t h = (cuuint64_t)H;
-  const cuuint64_t dims[5] = {(cuuint64_t)kC, h, h, dim == 3 ? h : (cuuint64_t)B, (cuuint64_t)B};
-  const cuuint64_t strides[4] = {row, row * h, row * h * h, row * h * h * h};
-  const cuuint32_t box[5] = {8, (cuuint32_t)kRows, 1, 1, 1};
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  if (g_encode(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)(dim + 2), (void*)in, dims,
-               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-      CUDA_SUCCESS)
+  if (!encode_boxes(&tm, in, dim, B, H, pack ? pk.P : kRows, pack ? pk.box / (pk.P * 16) : 1))
     return cudaErrorInvalidValue;
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  long long ntiles = (long long)B * H * ((H + kTcM - 1) / kTcM);
+  long long ntiles = pack ? (long long)B * pk.tpp : (long long)B * H * ((H + kTcM - 1) / kTcM);
   if (dim == 3) ntiles *= H;
-  // CTAs that fit an SM (shared memory: two in 2D, one in 3D); each runs a
-  // stream of tiles
-  const long long per_sm = dim == 3 ? 1 : 2;
-  const int grid = (int)(ntiles < per_sm * nsm ? ntiles : per_sm * nsm);
-  if (dim == 3)
-    launch_tc<3>(mode, grid, s, tm, B, H, wop, bias, dil, sign, zo, to, resid, fo, addend);
+  // CTAs that fit an SM by their shared memory; each runs a stream of tiles
+  const long long most = (long long)(2 * (sm + 1024) <= 228 * 1024 ? 2 : 1) * tc_sm_count();
+  const int grid = (int)(ntiles < most ? ntiles : most);
+  if (dim == 3 && pack)
+    launch_tc<3, true>(mode, grid, sm, s, tm, pk, B, H, wop, bias, dil, sign, zo, to, resid, fo, addend);
+  else if (dim == 3)
+    launch_tc<3, false>(mode, grid, sm, s, tm, pk, B, H, wop, bias, dil, sign, zo, to, resid, fo, addend);
+  else if (pack)
+    launch_tc<2, true>(mode, grid, sm, s, tm, pk, B, H, wop, bias, dil, sign, zo, to, resid, fo, addend);
   else
-    launch_tc<2>(mode, grid, s, tm, B, H, wop, bias, dil, sign, zo, to, resid, fo, addend);
+    launch_tc<2, false>(mode, grid, sm, s, tm, pk, B, H, wop, bias, dil, sign, zo, to, resid, fo, addend);
   note_launches(1);
   return cudaGetLastError();
 }
 
-// A tensor map over a channels-last activation, [B][H][H][32] (2D) or
-// [B][H][H][H][32] (3D), BF16: boxes of 8 channels x kRows pixels of one row.
-static bool encode_rows(CUtensorMap* tm, const __nv_bfloat16* p, int dim, int B, int H) {
-  const cuuint64_t row = (cuuint64_t)kC * 2;
-  const cuuint64_t h = (cuuint64_t)H;
-  const cuuint64_t dims[5] = {(cuuint64_t)kC, h, h, dim == 3 ? h : (cuuint64_t)B, (cuuint64_t)B};
-  const cuuint64_t strides[4] = {row, row * h, row * h * h, row * h * h * h};
-  const cuuint32_t box[5] = {8, (cuuint32_t)kRows, 1, 1, 1};
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  return g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)(dim + 2), (void*)p, dims,
-                  strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-         CUDA_SUCCESS;
-}
-
 cudaError_t launch_wgrad_tc(int dim, int B, int H, const __nv_bfloat16* in,
-                            const __nv_bfloat16* g, int dil, float* part, int stride, int nparts,
+                            const __nv_bfloat16* g, int dil, float* part, int stride, int* nparts_io,
                             cudaStream_t s) {
+  int nparts = *nparts_io;
   if (!g_tc_err) {
     const cudaError_t e = conv32_tc_setup();
     if (e != cudaSuccess) return e;
@@ -749,20 +906,34 @@ cudaError_t launch_wgrad_tc(int dim, int B, int H, const __nv_bfloat16* in,
       stride < T * kC * kC + kC || ((unsigned long long)in & 15ull) ||
       ((unsigned long long)g & 15ull) || ((unsigned long long)part & 15ull) || (stride & 3))
     return cudaErrorInvalidValue;
+  const bool pack = tc_kind(dim, B, H, dil) == kTcPacked;
+  TcPack pk;
+  int sm = kWgSmem;
+  if (pack && !pack_geometry(dim, H, dil, true, &pk, &sm)) return cudaErrorInvalidValue;
+  const int bx = pack ? pk.P : kRows, by = pack ? pk.box / (pk.P * 16) : 1;
   CUtensorMap tin, tg;
-  if (!encode_rows(&tin, in, dim, B, H) || !encode_rows(&tg, g, dim, B, H))
+  if (!encode_boxes(&tin, in, dim, B, H, bx, by) || !encode_boxes(&tg, g, dim, B, H, bx, by))
     return cudaErrorInvalidValue;
+  long long ntiles = pack ? (long long)B * pk.tpp : (long long)B * H * ((H + kTcM - 1) / kTcM);
+  if (dim == 3) ntiles *= H;
+  // packed: one wave of CTAs, and no more than tiles
+  if (pack) {
+    const int most = (2 * (sm + 1024) <= 228 * 1024 ? 2 : 1) * tc_sm_count();
+    nparts = (int)std::min<long long>(std::min(nparts, most), ntiles);
+    *nparts_io = nparts;
+  }
   // every one of the nparts CTAs writes its partial (zeros without tiles); in 3D
   // one launch per plane offset tz of the taps
-  if (dim == 2) {
-    wgrad_tc<2><<<nparts, kTcThreads, kWgSmem, s>>>(tin, tg, B, H, dil, 1, part, stride,
-                                                     g_tc_err);
+  for (int tz = dim == 3 ? 0 : 1; tz < (dim == 3 ? 3 : 2); tz++) {
+    if (dim == 3 && pack)
+      wgrad_tc<3, true><<<nparts, kTcThreads, sm, s>>>(tin, tg, pk, B, H, dil, tz, part, stride, g_tc_err);
+    else if (dim == 3)
+      wgrad_tc<3, false><<<nparts, kTcThreads, sm, s>>>(tin, tg, pk, B, H, dil, tz, part, stride, g_tc_err);
+    else if (pack)
+      wgrad_tc<2, true><<<nparts, kTcThreads, sm, s>>>(tin, tg, pk, B, H, dil, tz, part, stride, g_tc_err);
+    else
+      wgrad_tc<2, false><<<nparts, kTcThreads, sm, s>>>(tin, tg, pk, B, H, dil, tz, part, stride, g_tc_err);
     note_launches(1);
-  } else {
-    for (int tz = 0; tz < 3; tz++)
-      wgrad_tc<3><<<nparts, kTcThreads, kWgSmem, s>>>(tin, tg, B, H, dil, tz, part, stride,
-                                                       g_tc_err);
-    note_launches(3);
   }
   return cudaGetLastError();
 }

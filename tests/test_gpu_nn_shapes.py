@@ -40,3 +40,25 @@ def test_forward_and_gradients_at_odd_shapes(dim, n, B):
     lr, gr = onn.loss_and_grads(P, u, t, n, dim=dim)
     assert abs(loss - lr) <= 2e-2 * lr
     check_grads(unpack(g, n, dim=dim), gr, "%dD n=%d" % (dim, n))
+
+
+@pytest.mark.parametrize("dim,n,B", [(2, 100, 4), (2, 127, 3), (3, 8, 1), (3, 13, 2), (3, 30, 2),
+                                     (3, 52, 1)])
+def test_packed_tiles_give_the_row_tiles_bits(dim, n, B, monkeypatch):
+    """Tiles over several padded rows against a tile per row segment
+    (MLGMRES_TC_MIN_ROW = 1): the same MMAs per output in the same order, so the
+    forward pass is the same bits; the weight gradients' FP32 sums are split
+    differently (relative 1e-6 of each tensor's norm: about sqrt(tiles) roundings)."""
+    from paper_2103_10975_gb300 import Solver
+    s = Solver(n, dim=dim, m=10, batch=B)
+    rng = np.random.default_rng(n)
+    u = torch.as_tensor(rng.standard_normal((B, n ** dim)), dtype=torch.float32).cuda()
+    t = torch.as_tensor(rng.standard_normal((B, n ** dim)), dtype=torch.float32).cuda()
+    out = []
+    for rows in (None, "1"):
+        if rows:
+            monkeypatch.setenv("MLGMRES_TC_MIN_ROW", rows)
+        out.append((s.nn_forward(u).cpu().numpy(), s.nn_loss_grad(u, t)[1]))
+    assert np.array_equal(out[0][0], out[1][0])
+    d = np.linalg.norm(out[0][1] - out[1][1])
+    assert d <= 1e-6 * np.linalg.norm(out[1][1]), d
