@@ -414,58 +414,103 @@ struct Window {
   }
 };
 
+// A lane of the kernels below holds kLaneCh channels of a point (2D 4, 3D 2: what its
+// taps' weights or sums leave of the registers), 32 / kLaneCh lanes a point: a point's
+// window is read from shared memory once for all of them, and a warp's access to a
+// 32-channel field covers 4 (2) points at 16 and 8 (8 and 4) bytes per lane.  One
+// channel per lane left these kernels bound by instructions and 2- and 4-byte accesses
+// (us, one channel / now, 256^2 x 8 and 48^3 x 2; floors by bytes 19, 5, 15 and 8, 2,
+// 6): conv_out_bwd_data 68 / 42, 50 / 38; conv1_wgrad<0> 46 / 30, 37 / 29;
+// conv1_wgrad<1> 61 / 47, 45 / 36.
+template <int D>
+constexpr int kLaneCh = D == 2 ? 4 : 2;
+template <int C>
+struct LaneVec;
+template <>
+struct LaneVec<4> {
+  using B = uint2;   // bf16 values
+  using F = float4;  // float values
+};
+template <>
+struct LaneVec<2> {
+  using B = unsigned;
+  using F = float2;
+};
+template <int C>
+__device__ __forceinline__ void lane_floats(float (&v)[C], typename LaneVec<C>::B b) {
+  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&b);
+#pragma unroll
+  for (int q = 0; q < C / 2; q++) {
+    const float2 t = __bfloat1622float2(h[q]);
+    v[2 * q] = t.x;
+    v[2 * q + 1] = t.y;
+  }
+}
+template <int C>
+__device__ __forceinline__ typename LaneVec<C>::B lane_bf(const float (&v)[C]) {
+  typename LaneVec<C>::B b;
+  __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&b);
+#pragma unroll
+  for (int q = 0; q < C / 2; q++) h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+  return b;
+}
+
 // gt[p][c] = sum_tap w[c][tap] gy[p - off_tap] (transpose of the 32 -> 1 output
 // conv) and, when gbf is given, gbf[p][c] = bf16(mask[p][c] > 0 ? gt : 0) for
-// the masked consumer that follows.  Segments as above (gy staged); lane =
-// channel (coalesced 128-byte rows), each warp U points of the segment.
+// the masked consumer that follows.  Segments as above (gy staged), each group of
+// lanes U points of the segment in a row.
 template <int D>
-__global__ void __launch_bounds__(kW1Threads) conv_out_bwd_data(int B, int n,
-                                                               const float* __restrict__ gy,
-                                                               const float* __restrict__ w,
-                                                               float* __restrict__ gt,
-                                                               const bf16* __restrict__ mask,
-                                                               bf16* __restrict__ gbf) {
+__global__ void __launch_bounds__(kW1Threads, 2) conv_out_bwd_data(
+    int B, int n, const float* __restrict__ gy, const float* __restrict__ w,
+    float* __restrict__ gt, const bf16* __restrict__ mask, bf16* __restrict__ gbf) {
   constexpr int T = Geo<D>::T;
-  constexpr int NW = kW1Threads / 32;
-  constexpr int U = kSeg / NW;
+  constexpr int C = kLaneCh<D>, LP = kC / C;  // channels per lane, lanes per point
+  constexpr int U = kSeg / (kW1Threads / LP);
   constexpr int CH = 8;
+  using BV = typename LaneVec<C>::B;
+  using FV = typename LaneVec<C>::F;
   extern __shared__ float sf[];
   const int W = w1_w(n), R = w1_r(n);
   const int TW = W + 2, TP = (R + 2) * TW;
   const int xsegs = (n + W - 1) / W, ysegs = (n + R - 1) / R;
   const int nseg = B * (D == 3 ? n : 1) * ysegs * xsegs;
-  const int c = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  float wc[T];
+  const int c = threadIdx.x % LP * C, wp = threadIdx.x / LP;
+  float wc[C][T];
 #pragma unroll
-  for (int tp = 0; tp < T; tp++) wc[tp] = w[c * T + tp];
+  for (int d = 0; d < C; d++)
+#pragma unroll
+    for (int tp = 0; tp < T; tp++) wc[d][tp] = w[(c + d) * T + tp];
   const int ry0 = (wp * U) / W, xl0 = (wp * U) % W;
   const int center = D == 3 ? TP : 0;
   for (int sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
     const int xs = sg % xsegs, t2 = sg / xsegs;
     const int ys = t2 % ysegs, pl = t2 / ysegs;
     const int x0 = xs * W, y0 = ys * R;
-    __syncthreads();
-    w1_stage<D, kW1Threads>(sf, gy, n, pl, y0, x0, W, R);
-    __syncthreads();
-    int ry = ry0, xl = xl0;
-    Window<D> win;
-    bool next = false;
-#pragma unroll 1
-    for (int k0 = 0; k0 < U; k0 += CH) {
-      // CH points at a time: their masks first, in flight together (loaded one by
-      // one beside the stores, each point waited for its own)
-      bf16 mk[CH];
-      int lry = ry, lxl = xl;
+    int ry = ry0, xl = xl0, lry = ry0, lxl = xl0;  // next point to compute, to load
+    // CH points' masks in flight together, the first ones' during the staging
+    BV mk[CH];
+    auto load = [&]() {
 #pragma unroll
       for (int k = 0; k < CH; k++) {
         const int y = y0 + lry, x = x0 + lxl;
-        mk[k] = gbf && lry < R && y < n && x < n ? mask[((pl * n + y) * n + x) * kC + c]
-                                                 : __float2bfloat16(0.f);
+        mk[k] = BV{};
+        if (gbf && lry < R && y < n && x < n)
+          mk[k] = *reinterpret_cast<const BV*>(mask + ((pl * n + y) * n + x) * kC + c);
         if (++lxl == W) {
           lxl = 0;
           ++lry;
         }
       }
+    };
+    load();
+    __syncthreads();
+    w1_stage<D, kW1Threads>(sf, gy, n, pl, y0, x0, W, R);
+    __syncthreads();
+    Window<D> win;
+    bool next = false;
+#pragma unroll 1
+    for (int k0 = 0; k0 < U; k0 += CH) {
+      if (k0) load();
 #pragma unroll
       for (int k = 0; k < CH; k++) {
         const int y = y0 + ry, x = x0 + xl;
@@ -473,12 +518,24 @@ __global__ void __launch_bounds__(kW1Threads) conv_out_bwd_data(int B, int n,
           win.move(sf, center + (ry + 1) * TW + xl + 1, TP, TW, next);
           next = true;
           if (y < n && x < n) {
-            float acc = 0.f;
+            float acc[C];
 #pragma unroll
-            for (int tp = 0; tp < T; tp++) acc += wc[tp] * win.template at<-1>(tp);
+            for (int d = 0; d < C; d++) {
+              acc[d] = 0.f;
+#pragma unroll
+              for (int tp = 0; tp < T; tp++) acc[d] += wc[d][tp] * win.template at<-1>(tp);
+            }
             const int e = ((pl * n + y) * n + x) * kC + c;  // (below 2^31: network size check)
-            gt[e] = acc;
-            if (gbf) gbf[e] = __float2bfloat16(__bfloat162float(mk[k]) > 0.f ? acc : 0.f);
+            FV o;
+            memcpy(&o, acc, sizeof(o));
+            *reinterpret_cast<FV*>(gt + e) = o;
+            if (gbf) {
+              float m[C];
+              lane_floats<C>(m, mk[k]);
+#pragma unroll
+              for (int d = 0; d < C; d++) m[d] = m[d] > 0.f ? acc[d] : 0.f;
+              *reinterpret_cast<BV*>(gbf + e) = lane_bf<C>(m);
+            }
           }
         }
         if (++xl == W) {
@@ -499,11 +556,11 @@ __global__ void __launch_bounds__(kW1Threads) conv_out_bwd_data(int B, int n,
 //                        with g32 taken as 0 where m32 <= 0 (the ReLU of a0), plus
 //                        2^-D of the pooled level's gradient gc (null: no such level)
 // The grid is cut into segments of R rows x W points of one (b, z) plane
-// (W = min(n, 256), R = max(1, 256 / n)).  Lane = channel: every 32-channel row
-// is read once, coalesced, U rows per warp in flight; the 1-channel field (gy
-// or u) of the segment and its halo is staged in shared memory, zero outside
-// the grid, so each tap is one shared-memory read at a fixed offset.  The 16
-// warp sums are added in a fixed order.
+// (W = min(n, 256), R = max(1, 256 / n)).  Every 32-channel row is read once,
+// coalesced, CH rows per group of lanes in flight; the 1-channel field (gy or u) of
+// the segment and its halo is staged in shared memory, zero outside the grid, so each
+// tap is one shared-memory read at a fixed offset.  The sums of a warp's groups
+// of lanes, then of the warps, are added in a fixed order.
 template <int D>
 int conv1_wgrad_smem(int n) {
   constexpr int T = Geo<D>::T;
@@ -519,8 +576,11 @@ __global__ void __launch_bounds__(kW1Threads, 2) conv1_wgrad(
     const float* __restrict__ u, float* __restrict__ part, int stride) {
   constexpr int T = Geo<D>::T;
   constexpr int NW = kW1Threads / 32;
-  constexpr int U = kSeg / NW;             // points per warp and segment
-  constexpr int CH = 8;                    // points whose loads are in flight together
+  constexpr int C = kLaneCh<D>, LP = kC / C;      // channels per lane, lanes per point
+  constexpr int U = kSeg / (kW1Threads / LP);     // points per group of lanes and segment
+  constexpr int CH = MODE == 1 || D == 3 ? 4 : 8; // points whose loads are in flight together
+  using BV = typename LaneVec<C>::B;
+  using FV = typename LaneVec<C>::F;
   constexpr int sgn = MODE == 0 ? -1 : 1;  // MODE 0 reads gy at q - off, MODE 1 u at p + off
   extern __shared__ float sf[];
   const int W = w1_w(n), R = w1_r(n);
@@ -528,41 +588,46 @@ __global__ void __launch_bounds__(kW1Threads, 2) conv1_wgrad(
   const int xsegs = (n + W - 1) / W, ysegs = (n + R - 1) / R;
   const int nplanes = B * (D == 3 ? n : 1);  // (b, z) planes
   const int nseg = nplanes * ysegs * xsegs;
-  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int c = threadIdx.x % LP * C, gw = threadIdx.x / LP;
   const float* __restrict__ f = MODE == 0 ? g1 : u;
-  float acc[T];
+  float acc[C][T], accb[C];
 #pragma unroll
-  for (int t = 0; t < T; t++) acc[t] = 0.f;
-  float accb = 0.f;
+  for (int d = 0; d < C; d++) {
+    accb[d] = 0.f;
+#pragma unroll
+    for (int t = 0; t < T; t++) acc[d][t] = 0.f;
+  }
   for (int sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
     const int xs = sg % xsegs, t2 = sg / xsegs;
     const int ys = t2 % ysegs, pl = t2 / ysegs;  // pl = b (2D) or b n + z (3D)
     const int x0 = xs * W, y0 = ys * R;
-    // the warp's U points run along x from (ry, xl), wrapping to the next row;
+    // the group's U points run along x from (ry, xl), wrapping to the next row;
     // CH at a time, the next ones' loads in flight while these are used (the
     // first ones' during the staging).  All loads of a point are unconditional:
     // behind its mask, each would wait for the one before it.
-    int ry = (w * U) / W, xl = (w * U) % W;
+    int ry = (gw * U) / W, xl = (gw * U) % W;
     int lry = ry, lxl = xl;  // of the next point to load
     const int center = D == 3 ? TP : 0;
     const int so = n / 2, pz = pl % n;
     const int cp = D == 3 ? (pl / n) * so + pz / 2 : pl;
     const bool cok = MODE == 1 && gc && (D == 2 || pz / 2 < so);
-    bf16 rm[CH];
-    float rg[CH], rc[CH];
+    BV rm[CH];
+    FV rg[CH], rc[CH];
     auto load = [&]() {
 #pragma unroll
       for (int k = 0; k < CH; k++) {
         const int x = x0 + lxl, y = y0 + lry;
         const bool ok = lry < R && y < n && x < n;
         const int e = ((pl * n + y) * n + x) * kC + c;  // (below 2^31: network size check)
-        rm[k] = ok ? (MODE == 0 ? x32 : m32)[e] : __float2bfloat16(0.f);
+        rm[k] = BV{};
+        if (ok) rm[k] = *reinterpret_cast<const BV*>((MODE == 0 ? x32 : m32) + e);
         if constexpr (MODE == 1) {
-          rg[k] = ok ? g32[e] : 0.f;
+          rg[k] = FV{};
+          rc[k] = FV{};
+          if (ok) rg[k] = *reinterpret_cast<const FV*>(g32 + e);
           // the pooled level's share (odd sides: the last point has none)
-          rc[k] = ok && cok && y / 2 < so && x / 2 < so
-                      ? gc[((cp * so + y / 2) * so + x / 2) * kC + c]
-                      : 0.f;
+          if (ok && cok && y / 2 < so && x / 2 < so)
+            rc[k] = *reinterpret_cast<const FV*>(gc + ((cp * so + y / 2) * so + x / 2) * kC + c);
         }
         if (++lxl == W) {
           lxl = 0;
@@ -578,14 +643,18 @@ __global__ void __launch_bounds__(kW1Threads, 2) conv1_wgrad(
     bool next = false;
 #pragma unroll 1
     for (int k0 = 0; k0 < U; k0 += CH) {
-      float val[CH];
+      float val[CH][C];
 #pragma unroll
       for (int k = 0; k < CH; k++) {
-        const float m = __bfloat162float(rm[k]);
-        if constexpr (MODE == 0)
-          val[k] = m;
-        else
-          val[k] = m > 0.f ? rg[k] + (1.f / (1 << D)) * rc[k] : 0.f;
+        lane_floats<C>(val[k], rm[k]);
+        if constexpr (MODE == 1) {
+          float a[C], b[C];
+          memcpy(a, &rg[k], sizeof(a));
+          memcpy(b, &rc[k], sizeof(b));
+#pragma unroll
+          for (int d = 0; d < C; d++)
+            val[k][d] = val[k][d] > 0.f ? a[d] + (1.f / (1 << D)) * b[d] : 0.f;
+        }
       }
       if (k0 + CH < U) load();
 #pragma unroll
@@ -595,9 +664,12 @@ __global__ void __launch_bounds__(kW1Threads, 2) conv1_wgrad(
           next = true;
           // (val is 0 past the grid's edge; the staged field is finite there)
 #pragma unroll
-          for (int t = 0; t < T; t++) acc[t] += val[k] * win.template at<sgn>(t);
-          if (MODE == 1) accb += val[k];
-          else if (y0 + ry < n && x0 + xl < n) accb += win.template at<1>(T / 2);
+          for (int d = 0; d < C; d++) {
+#pragma unroll
+            for (int t = 0; t < T; t++) acc[d][t] += val[k][d] * win.template at<sgn>(t);
+            if (MODE == 1) accb[d] += val[k][d];
+          }
+          if (MODE == 0 && y0 + ry < n && x0 + xl < n) accb[0] += win.template at<1>(T / 2);
         }
         if (++xl == W) {
           xl = 0;
@@ -607,12 +679,19 @@ __global__ void __launch_bounds__(kW1Threads, 2) conv1_wgrad(
       }
     }
   }
-  // fixed-order sum of the warps' partials
+  // fixed-order sum of the groups' partials within a warp, then of the warps'
   __syncthreads();
-  float* red = sf;  // [NW][32 (T + 1)]
+  float* red = sf + (threadIdx.x >> 5) * 32 * (T + 1);  // [NW][32 (T + 1)]
 #pragma unroll
-  for (int t = 0; t < T; t++) red[w * 32 * (T + 1) + c * (T + 1) + t] = acc[t];
-  red[w * 32 * (T + 1) + c * (T + 1) + T] = accb;
+  for (int d = 0; d < C; d++)
+#pragma unroll
+    for (int t = 0; t < T + 1; t++) {
+      float v = t < T ? acc[d][t < T ? t : 0] : accb[d];
+#pragma unroll
+      for (int off = LP; off < 32; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+      if ((threadIdx.x & 31) < LP) red[(c + d) * (T + 1) + t] = v;
+    }
+  red = sf;
   __syncthreads();
   for (int t = threadIdx.x; t < kC * T + kC; t += kW1Threads) {
     // t < 32 T: weight c*T + tap; t >= 32 T: bias of channel t - 32 T (MODE 0: one bias)
@@ -771,7 +850,10 @@ __device__ __forceinline__ float4 row_sum4(const float* __restrict__ src, long l
 // for every level.  A thread forms four channels of one coarse point (16-byte
 // reads, a quarter of the instructions of one channel per lane; the fine points
 // of a coarse one are consecutive, so only the first index is read).  Same
-// sums, in the same order, as upsample_bwd_axis.
+// sums, in the same order, as upsample_bwd_axis.  The staging also writes the
+// masked BF16 gradient of the finest level, maskbf = bf16(mask > 0 ? in : 0), which
+// would read the row from HBM once more in a launch of its own (256^2 x 8: 65 + 21 us
+// in two launches, 79 in one).
 struct UpLevels {
   int nlev;                     // levels 1 .. nlev-1
   int m[kMaxLevels];
@@ -788,14 +870,27 @@ constexpr int kXLevelsMaxN = 384;  // the staged row (n x 32 floats) stays withi
 
 __global__ void __launch_bounds__(256) upsample_bwd_x_levels(int n, UpLevels lv,
                                                              const float* __restrict__ in,
-                                                             float* __restrict__ out) {
+                                                             float* __restrict__ out,
+                                                             const bf16* __restrict__ mask,
+                                                             bf16* __restrict__ maskbf) {
   extern __shared__ float row[];  // the fine row, n x 32
   const long long r = blockIdx.x;
   const int c4 = (threadIdx.x & 7) * 4, g = threadIdx.x >> 3;
   {
     const float4* src = reinterpret_cast<const float4*>(in + r * n * kC);
+    const uint2* mk = reinterpret_cast<const uint2*>(mask + r * n * kC);
+    uint2* mo = reinterpret_cast<uint2*>(maskbf + r * n * kC);
     float4* dst = reinterpret_cast<float4*>(row);
-    for (int i = threadIdx.x; i < n * kC / 4; i += 256) dst[i] = src[i];
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n * kC / 4; i += 256) {
+      const float4 v = src[i];
+      float m[4];
+      lane_floats<4>(m, mk[i]);
+      dst[i] = v;
+      const float o[4] = {m[0] > 0.f ? v.x : 0.f, m[1] > 0.f ? v.y : 0.f, m[2] > 0.f ? v.z : 0.f,
+                          m[3] > 0.f ? v.w : 0.f};
+      mo[i] = lane_bf<4>(o);
+    }
   }
   __syncthreads();
   for (int l = 1; l < lv.nlev; l++) {
@@ -1409,8 +1504,8 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
       lv.out_off[l] = off;
       off += rows * net.side[l] * kC;
     }
-    upsample_bwd_x_levels<<<(unsigned)rows, 256, sizeof(float) * n * kC, s>>>(n, lv, net.g_s,
-                                                                               net.g_t);
+    upsample_bwd_x_levels<<<(unsigned)rows, 256, sizeof(float) * n * kC, s>>>(
+        n, lv, net.g_s, net.g_t, net.z[0], net.g_bf);
     note_launches(1);
     long long xin[kMaxLevels];
     for (int l = 1; l < L; l++) xin[l] = lv.out_off[l];
@@ -1425,8 +1520,10 @@ cudaError_t backward_t(Net& net, int B, const float* u, const float* y, const fl
       other_axes(l, l + 1, xin);
     }
   }
-  mask_to_bf16<<<nblk(full / 8, 256), 256, 0, s>>>(full, net.g_s, net.z[0], net.g_bf);
-  note_launches(1);
+  if (!fused_x) {
+    mask_to_bf16<<<nblk(full / 8, 256), 256, 0, s>>>(full, net.g_s, net.z[0], net.g_bf);
+    note_launches(1);
+  }
   {
     // every level's weight and data gradients; the coarse levels share launches
     WgradJob wj[kMaxLevels];
