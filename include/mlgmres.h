@@ -131,7 +131,9 @@ typedef struct {
                                 a pass uses as many as fit in the warp's share of shared
                                 memory for its j rows), or 0 for direct loads; -1 =
                                 automatic (the autotuned value if mlgmres_autotune ran,
-                                else 16) */
+                                else 16).  In 3D
+                                a value >= 0 also asks for the basis in HBM where its
+                                slices would fit in shared memory */
   int retrain_after;         /* f_r of Algorithm 1 (Sec. 2.2): when > 0, mlgmres_solve itself
                                 starts a training phase (as mlgmres_train_step, on a stream
                                 of the handle) at tau0 and then once f_r under-performing

@@ -29,6 +29,8 @@ int own_bytes_f2c();
 cudaError_t launch_gmres_f3c(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f2cs(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f2s32(const KParams& kp, int grid, cudaStream_t s);
+cudaError_t launch_gmres_f2sl(const KParams& kp, int grid, cudaStream_t s);
+cudaError_t launch_gmres_f2sl32(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_d2s32(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f3s(const KParams& kp, int grid, cudaStream_t s);
 cudaError_t launch_gmres_f3s32(const KParams& kp, int grid, cudaStream_t s);
@@ -85,6 +87,8 @@ cudaError_t launch_gmres(const KParams& kp, bool fp32, int dim, int grid, cudaSt
   }
   if (fp32) {
     if (dim == 2) {
+      if (kp.vmode == kVSharedL)
+        return kp.m <= kSmallM ? launch_gmres_f2sl32(kp, grid, s) : launch_gmres_f2sl(kp, grid, s);
       if (kp.vmode == kVShared)
         return kp.m <= kSmallM ? launch_gmres_f2s32(kp, grid, s) : launch_gmres_f2s(kp, grid, s);
       if (kp.vmode == kVBulk) return launch_gmres_f2b(kp, grid, s);
@@ -118,7 +122,7 @@ int gmres_max_blocks(bool fp32, int dim, int m, int* bs) {
 int gmres_bulk_cap(bool fp32, int m, int P) {
   if (P <= 0) return 0;
   const long long row = 32LL * (fp32 ? 4 : 8);                                  // bytes
-  const long long share = (long long)gmres_vsmem_budget(fp32) / 8 / 128 * 128;  // per warp
+  const long long share = (long long)gmres_vsmem_budget(fp32) / 8 / 128 * 128;  // per warp (m <= kMaxM)
   // a stage: m rows of V and the X pass's w'/kappa windows (the 3D size, the
   // larger of the two dimensions)
   const long long stage =
@@ -136,9 +140,10 @@ int gmres_vsmem_budget(bool fp32, int m) {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int own = fp32           ? (int)smem_own_bytes<float, kMaxM, 256>()
-                  : m <= kSmallM ? (int)smem_own_bytes<double, kSmallM, 256>()
-                                 : (int)smem_own_bytes<double, kMaxM, 256>();
+  const int own = m <= kSmallM ? (fp32 ? (int)smem_own_bytes<float, kSmallM, 256>()
+                                       : (int)smem_own_bytes<double, kSmallM, 256>())
+                               : (fp32 ? (int)smem_own_bytes<float, kMaxM, 256>()
+                                       : (int)smem_own_bytes<double, kMaxM, 256>());
   const int left = optin - own - 1024;
   return left > 0 ? left : 0;
 }

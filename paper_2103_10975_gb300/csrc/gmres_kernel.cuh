@@ -359,6 +359,34 @@ __device__ __forceinline__ void block_finish(int L, R* part, int lb, R (*red)[LW
   }
 }
 
+// Warp 0: the CTA's sums of slots 0 .. L-1 over the warp partials, to part.  FP64: as
+// a tree (an addition is 64 cycles of pipe and ~70 of latency), two lanes per slot
+// while there are no more than 16.
+template <int LW, int BS, typename R>
+__device__ __forceinline__ void cta_sums(int L, R* part, int lb, R (*red)[LW], int ps) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (sizeof(R) == 8 && BS == 256) {
+    if (L <= 16) {
+      const int k = lane & 15, w0 = lane >> 4 << 2;
+      R s = R(0);
+      if (k < L) s = (red[w0][k] + red[w0 + 1][k]) + (red[w0 + 2][k] + red[w0 + 3][k]);
+      s += __shfl_xor_sync(0xffffffffu, s, 16);
+      if (lane < L) part[(long long)k * ps + lb] = s;
+      return;
+    }
+    for (int k = lane; k < L; k += 32)
+      part[(long long)k * ps + lb] = ((red[0][k] + red[1][k]) + (red[2][k] + red[3][k])) +
+                                     ((red[4][k] + red[5][k]) + (red[6][k] + red[7][k]));
+  } else {
+    for (int k = lane; k < L; k += 32) {
+      R s = R(0);
+#pragma unroll
+      for (int w = 0; w < BS / 32; w++) s += red[w][k];
+      part[(long long)k * ps + lb] = s;
+    }
+  }
+}
+
 // block_finish and the group barrier in one: after one CTA barrier, warp 0
 // adds the warp partials, stores the CTA's sums, and (its lanes' stores ordered
 // by __syncwarp before lane 0's release) arrives and waits at the group
@@ -371,12 +399,7 @@ __device__ __forceinline__ bool finish_and_sync(int L, R* part, int lb, R (*red)
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0) {
-    for (int k = lane; k < L; k += 32) {
-      R s = R(0);
-#pragma unroll
-      for (int w = 0; w < BS / 32; w++) s += red[w][k];
-      part[(long long)k * ps + lb] = s;
-    }
+    cta_sums<LW, BS>(L, part, lb, red, ps);
     __syncwarp();
     if (lane == 0)
       *s_flag = gb.nblocks == 1 ? (*(volatile int*)gb.err == kErrNone)
@@ -406,12 +429,7 @@ __device__ __forceinline__ void finish_and_sync_side(int L, R* part, int lb, R (
     return;
   }
   if (warp == 0) {
-    for (int k = lane; k < L; k += 32) {
-      R s = R(0);
-#pragma unroll
-      for (int w = 0; w < BS / 32; w++) s += red[w][k];
-      part[(long long)k * ps + lb] = s;
-    }
+    cta_sums<LW, BS>(L, part, lb, red, ps);
     __syncwarp();
     if (lane == 0)
       *s_flag = gb.nblocks == 1 ? (*(volatile int*)gb.err == kErrNone)
@@ -435,6 +453,22 @@ __device__ __forceinline__ void gather(const R* part, int L, int nb, double* tot
   const int lane = threadIdx.x & 31, warp0 = threadIdx.x >> 5;
   // (warp 1 under SKIP1 starts past every slot)
   const int warp = SKIP1 ? (warp0 == 1 ? (1 << 20) : (warp0 == 0 ? 0 : warp0 - 1)) : warp0;
+  if (sizeof(R) == 8 && nb <= 8) {
+    // FP64, few CTAs: four slots by eight CTAs in a warp, three additions for all (32^2,
+    // 8 CTAs: 12.9 -> 11.9 us per step)
+    for (int k0 = warp * 4; k0 < L; k0 += NW * 4) {
+      const int k = k0 + (lane >> 3), g = lane & 7;
+      R v = k < L && g < nb ? ldcg(part + (long long)k * ps + g) : R(0);
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+      if (g == 0 && k < L) {
+        if constexpr (sizeof(R) == 8) tot[k] = (double)v;
+        coef[k] = (T)v;
+      }
+    }
+    __syncthreads();
+    return;
+  }
   for (int k0 = warp; k0 < L; k0 += Q * NW) {
     R s[Q];
 #pragma unroll
@@ -488,6 +522,196 @@ __device__ __forceinline__ void gather(const R* part, int L, int nb, double* tot
     }
   }
   __syncthreads();
+}
+
+// ------------------------------- exchanges of the FP32 shared-slice variants --
+// An exchange turns every CTA's partial sums of L slots into the group's sums,
+// in every CTA.  Here the partials travel as 16-byte words that carry a tag, the
+// exchange's number, beside three slots.  A word is
+// written and read as one, so a reader that finds the expected tag has the
+// values, and neither side waits for a fence: the release that a counter barrier
+// needs (all of the CTA's stores performed before the arrival) and its acquire
+// cost 0.36 us per exchange at 128 CTAs (two exchanges: 4.84 -> 4.12 us).
+//  - up to kDirectCtas CTAs (in a batch kDirectCtasBatch): the readers spin on the
+//    words themselves (two exchanges at 32 CTAs 3.47 us, at 8 CTAs 2.63, against 4.59
+//    and 3.87 with the counter barrier);
+//  - larger groups: a relaxed counter says when everyone has arrived, and a word
+//    that is still on its way is read again (spinning on all words from all CTAs
+//    floods L2: 9.7 us at 128 CTAs);
+//  - one CTA: warp 0's sums are the group's.
+// Two sets of words alternate: a CTA writes exchange e + 2 only after it has
+// everyone's words of e + 1, which each writes after reading those of e.
+// The other variants keep the counter barrier: FP64 partials would be a word each
+// (256^2 FP64 27.3 us per step with them, 26.8 without), and the streamed
+// variants' groups of 304 CTAs read more words than the fences cost (2048^2 149.1
+// against 147.9).
+constexpr int kWordSlots = 3;  // slots per word
+// Warp 0: the CTA's sums of the slots (over the warp partials), as words of this
+// exchange (or, alone in its group, straight into coef).
+template <int LW, int BS>
+__device__ __forceinline__ void exchange_send(int L, uint4* words, int lb, int ps, int nb,
+                                              float (*red)[LW], float* coef, unsigned tag) {
+  const int lane = threadIdx.x & 31;
+  for (int k0 = 0; k0 < L; k0 += 30) {  // ten words at a time
+    const int k = k0 + lane;
+    float s = 0.f;
+    if (lane < 30 && k < L) {
+#pragma unroll
+      for (int w = 0; w < BS / 32; w++) s += red[w][k];
+      if (nb == 1) coef[k] = s;
+    }
+    if (nb == 1) continue;
+    const float s1 = __shfl_down_sync(0xffffffffu, s, 1);
+    const float s2 = __shfl_down_sync(0xffffffffu, s, 2);
+    if (lane < 30 && lane % kWordSlots == 0 && k < L)
+      st_relaxed_b128(words + (long long)(k / kWordSlots) * ps + lb,
+                      make_uint4(__float_as_uint(s), __float_as_uint(s1), __float_as_uint(s2), tag));
+  }
+}
+
+// Every warp (without warp 1 if SKIP1): the group's sums of its words' slots into
+// coef, the same order in every CTA; two words per warp and round (one round
+// covers 42 slots).
+template <int BS, bool SKIP1>
+__device__ __forceinline__ void exchange_gather(const uint4* words, int L, int nb, float* coef,
+                                                int ps, unsigned tag, const GroupBarrier& gb,
+                                                int* s_flag) {
+  constexpr int NW = BS / 32 - (SKIP1 ? 1 : 0);
+  constexpr int Q = 2;
+  constexpr int RR = 5;  // CTAs per lane and round: one round covers 160
+  const int lane = threadIdx.x & 31, warp0 = threadIdx.x >> 5;
+  const int warp = SKIP1 && warp0 > 0 ? warp0 - 1 : warp0;
+  const int nwd = (L + kWordSlots - 1) / kWordSlots;
+  for (int w0 = warp; w0 < nwd; w0 += Q * NW) {
+    float s[8];
+#pragma unroll
+    for (int q = 0; q < 8; q++) s[q] = 0.f;
+    for (int g0 = 0; g0 < nb; g0 += 32 * RR) {
+      uint4 v[Q][RR];
+      bool miss = false;
+#pragma unroll
+      for (int q = 0; q < Q; q++)
+#pragma unroll
+        for (int r = 0; r < RR; r++) {
+          const int wd = w0 + q * NW, g = g0 + r * 32 + lane;
+          v[q][r] = wd < nwd && g < nb ? ld_relaxed_b128(words + (long long)wd * ps + g)
+                                       : make_uint4(0u, 0u, 0u, tag);
+        }
+#pragma unroll
+      for (int q = 0; q < Q; q++)
+#pragma unroll
+        for (int r = 0; r < RR; r++) miss |= v[q][r].w != tag;
+      if (__any_sync(0xffffffffu, miss)) {
+        SpinLimit lim;
+        bool more = true;
+        do {
+          miss = false;
+#pragma unroll
+          for (int q = 0; q < Q; q++)
+#pragma unroll
+            for (int r = 0; r < RR; r++)
+              if (v[q][r].w != tag) {
+                v[q][r] = ld_relaxed_b128(words + (long long)(w0 + q * NW) * ps + g0 + r * 32 + lane);
+                miss |= v[q][r].w != tag;
+              }
+          miss = __any_sync(0xffffffffu, miss);
+          if (miss) more = __all_sync(0xffffffffu, lim.more(gb));
+        } while (miss && more);
+        if (!more && lane == 0) *s_flag = 0;
+      }
+#pragma unroll
+      for (int q = 0; q < Q; q++)
+#pragma unroll
+        for (int r = 0; r < RR; r++) {
+          s[3 * q] += __uint_as_float(v[q][r].x);
+          s[3 * q + 1] += __uint_as_float(v[q][r].y);
+          s[3 * q + 2] += __uint_as_float(v[q][r].z);
+        }
+    }
+    // six sums by one butterfly of eight (9 shuffles): sum u on lanes 4u
+    warp_transpose_sum<8>(s);
+    const int u = lane >> 2, q = u / 3, k = (w0 + q * NW) * kWordSlots + u % 3;
+    if ((lane & 3) == 0 && q < Q && w0 + q * NW < nwd && k < L) coef[k] = s[0];
+  }
+}
+
+// One exchange: sm.red holds the warps' partials of slots 0 .. L-1; on return
+// (ended by a CTA barrier) coef holds the group's sums in every CTA.  `side` runs
+// on warp 1 beside it (SIDE: it may outlast the arrival; warp 1 then takes no
+// part in the gather and joins at the closing barrier).  `between` runs on every
+// thread before the gather (after the group's arrival, except in direct
+// exchanges).  Returns false when the group must abandon the solve.
+template <int LW, int BS, bool SIDE, typename Side, typename Between>
+__device__ __forceinline__ bool exchange(int L, uint4* words, int lb, int nb, float (*red)[LW],
+                                         int ps, const GroupBarrier& gb, unsigned long long& epoch,
+                                         unsigned tag, float* coef, int* s_flag, Side side,
+                                         Between between) {
+  uint4* set = words + (long long)(tag & 1u) * kTagWordRows * ps;
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool direct = nb > 1 && nb <= ((int)gridDim.x == nb ? kDirectCtas : kDirectCtasBatch);
+  if (SIDE && warp == 1) {
+    side();
+  } else {
+    if (warp == 0) {
+      exchange_send<LW, BS>(L, set, lb, ps, nb, red, coef, tag);
+      __syncwarp();
+      if (lane == 0) *s_flag = nb == 1 || direct ? 1 : group_arrive_wait<true>(gb, epoch);
+    }
+    if (!direct) {  // the other warps wait for warp 0 (and the group)
+      if (SIDE)
+        asm volatile("bar.sync 1, %0;" ::"r"(BS - 32) : "memory");
+      else
+        __syncthreads();
+    }
+    between();
+    if (nb > 1) exchange_gather<BS, SIDE>(set, L, nb, coef, ps, tag, gb, s_flag);
+  }
+  __syncthreads();
+  return *s_flag != 0;
+}
+
+// Values of w' with tags (shared-slice variants): read by other CTAs without a
+// barrier that orders them, so each carries the number of the exchange its step
+// ends with, in one 8-byte word.
+template <typename T>
+struct TagVal;
+template <>
+struct TagVal<float> {
+  using raw = unsigned long long;
+  static __device__ __forceinline__ raw none(unsigned tag) { return (raw)tag << 32; }
+  static __device__ __forceinline__ raw get(const void* w, int i) {
+    return ld_relaxed_u64((const raw*)w + i);
+  }
+  static __device__ __forceinline__ void put(void* w, int i, float v, unsigned tag) {
+    st_relaxed_u64((raw*)w + i, ((raw)tag << 32) | __float_as_uint(v));
+  }
+  static __device__ __forceinline__ bool ok(raw r, unsigned tag) { return (unsigned)(r >> 32) == tag; }
+  static __device__ __forceinline__ float val(raw r) { return __uint_as_float((unsigned)r); }
+  // a value known to have arrived
+  static __device__ __forceinline__ float seen(const void* w, int i) {
+    return ldcg((const float*)w + 2 * i);
+  }
+};
+// (FP64: plain values, ordered by the Y exchange's counter barrier.)
+template <>
+struct TagVal<double> {
+  using raw = double;
+  static __device__ __forceinline__ raw none(unsigned) { return 0.0; }
+  static __device__ __forceinline__ raw get(const void* w, int i) {
+    return ldcg((const double*)w + i);
+  }
+  static __device__ __forceinline__ void put(void* w, int i, double v, unsigned) {
+    ((double*)w)[i] = v;
+  }
+  static __device__ __forceinline__ bool ok(raw, unsigned) { return true; }
+  static __device__ __forceinline__ double val(raw r) { return r; }
+  static __device__ __forceinline__ double seen(const void* w, int i) { return get(w, i); }
+};
+// The variants with tagged exchanges and a tagged w'.
+template <typename T>
+__host__ __device__ constexpr bool tagged(int vmode) {
+  return in_shared(vmode) && sizeof(T) == 4;
 }
 
 // Double-float accumulation (error-free transformations, Dekker 1971 and
@@ -816,6 +1040,13 @@ __device__ __forceinline__ void y_pass(Smem<T, MAXM, BS>& sm, int lo, int hi, in
   warp_slot<LMAX>(sm.red, j + 1, accN);
 }
 
+// A pass of bucket K runs for steps K - 8 <= j < K only, so the first K/2 - 4
+// pairs of basis vectors are in use whatever j: no test on them.  (In the FP32 m <=
+// 32 variants; with more buckets' registers the loads hoisted past the missing tests
+// spill.)
+template <typename T, int K, int MAXM>
+constexpr int kSure = sizeof(T) == 4 && MAXM <= kSmallM ? K / 2 - 4 : 0;
+
 // ---------------------------------------- one point's column, in pairs --
 // vc points at a point's column of V (pair layout: vector k at vc[vko(k)]),
 // in shared memory (a CTA slice or a bulk-copy stage).  Even and odd k are
@@ -847,7 +1078,7 @@ __device__ __forceinline__ void x_proj(const Smem<T, MAXM, BS>& sm, const T* vc,
     }
 #pragma unroll
     for (int q = 0; q < K / 2; q++) {
-      if (q < np) {
+      if (q < kSure<T, K, MAXM> || q < np) {
         const T2 v = *reinterpret_cast<const T2*>(vc + (q << 6));
         const float4 hq = h[q >> 1], cq = c[q >> 1];
         av = fma2((q & 1) ? make_float2(hq.z, hq.w) : make_float2(hq.x, hq.y), v, av);
@@ -859,7 +1090,7 @@ __device__ __forceinline__ void x_proj(const Smem<T, MAXM, BS>& sm, const T* vc,
     const T2* cc = reinterpret_cast<const T2*>(sm.cv);
 #pragma unroll
     for (int q = 0; q < K / 2; q++) {
-      if (q < np) {
+      if (q < kSure<T, K, MAXM> || q < np) {
         const T2 v = *reinterpret_cast<const T2*>(vc + (q << 6));
         av = fma2(h2[q], v, av);
         az = fma2(cc[q], v, az);
@@ -872,7 +1103,7 @@ __device__ __forceinline__ void x_proj(const Smem<T, MAXM, BS>& sm, const T* vc,
 
 // X pass dots, after v_j is stored in the column: acc_k += v_k z for k <= j
 // (for even j the last pair is (v_j, 0)).  acc holds slots 2q, 2q+1 in acc[q].
-template <typename T, int K>
+template <typename T, int K, int MAXM>
 __device__ __forceinline__ void x_dots(typename Vec2<T>::type (&acc)[K / 2], const T* vc, int j,
                                        T z) {
   using T2 = typename Vec2<T>::type;
@@ -880,7 +1111,7 @@ __device__ __forceinline__ void x_dots(typename Vec2<T>::type (&acc)[K / 2], con
   const int np = (j >> 1) + 1;
 #pragma unroll
   for (int q = 0; q < K / 2; q++)
-    if (q < np) acc[q] = fma2(*reinterpret_cast<const T2*>(vc + (q << 6)), zz, acc[q]);
+    if (q < kSure<T, K, MAXM> || q < np) acc[q] = fma2(*reinterpret_cast<const T2*>(vc + (q << 6)), zz, acc[q]);
 }
 
 // Y pass: sum_{k<=j} h1_k v_k (h1 in sm.coef; for even j the last pair's
@@ -897,7 +1128,7 @@ __device__ __forceinline__ T y_proj(const Smem<T, MAXM, BS>& sm, const T* vc, in
     for (int p = 0; p < K / 4; p++) h[p] = reinterpret_cast<const float4*>(sm.coef)[p];
 #pragma unroll
     for (int q = 0; q < K / 2; q++) {
-      if (q < np) {
+      if (q < kSure<T, K, MAXM> || q < np) {
         const float4 hq = h[q >> 1];
         a = fma2((q & 1) ? make_float2(hq.z, hq.w) : make_float2(hq.x, hq.y),
                  *reinterpret_cast<const T2*>(vc + (q << 6)), a);
@@ -907,13 +1138,13 @@ __device__ __forceinline__ T y_proj(const Smem<T, MAXM, BS>& sm, const T* vc, in
     const T2* h1 = reinterpret_cast<const T2*>(sm.coef);
 #pragma unroll
     for (int q = 0; q < K / 2; q++)
-      if (q < np) a = fma2(h1[q], *reinterpret_cast<const T2*>(vc + (q << 6)), a);
+      if (q < kSure<T, K, MAXM> || q < np) a = fma2(h1[q], *reinterpret_cast<const T2*>(vc + (q << 6)), a);
   }
   return a.x + a.y;
 }
 
 // Y pass dots: acc_k += v_k w' for k <= j.
-template <typename T, int K>
+template <typename T, int K, int MAXM>
 __device__ __forceinline__ void y_dots(typename Vec2<T>::type (&acc)[K / 2], const T* vc, int j,
                                        T w) {
   using T2 = typename Vec2<T>::type;
@@ -921,7 +1152,7 @@ __device__ __forceinline__ void y_dots(typename Vec2<T>::type (&acc)[K / 2], con
   const int np = (j >> 1) + 1;
 #pragma unroll
   for (int q = 0; q < K / 2; q++)
-    if (q < np) acc[q] = fma2(*reinterpret_cast<const T2*>(vc + (q << 6)), ww, acc[q]);
+    if (q < kSure<T, K, MAXM> || q < np) acc[q] = fma2(*reinterpret_cast<const T2*>(vc + (q << 6)), ww, acc[q]);
 }
 
 // warp_slots_k for accumulators held in pairs (slots 2q, 2q+1 in acc[q]).
@@ -932,6 +1163,21 @@ __device__ __forceinline__ void warp_slots_k2(T (*red)[LMAX],
 #pragma unroll
   for (int k = 0; k < K; k++) a[k] = (k & 1) ? acc[k >> 1].y : acc[k >> 1].x;
   warp_slots_k<LMAX, K, T>(red, a, L);
+}
+
+// A warp's partials of slots 0 .. j (acc) and j + 1 (norm).  FP64: a warp without
+// tiles writes zeros instead of adding them up (on its SM quarter's pipe, beside a
+// warp that has some: 128^2 16.9 -> 15.4 us per step, 24^3 17.3 -> 15.8).
+template <int LMAX, int K, typename T>
+__device__ __forceinline__ void warp_partials(T (*red)[LMAX],
+                                              const typename Vec2<T>::type (&acc)[K / 2], T norm,
+                                              int j, bool tiles) {
+  if (sizeof(T) == 8 && !tiles) {
+    for (int k = threadIdx.x & 31; k < j + 2; k += 32) red[threadIdx.x >> 5][k] = T(0);
+    return;
+  }
+  warp_slots_k2<LMAX, K, T>(red, acc, j + 1);
+  warp_slot<LMAX>(red, j + 1, norm);
 }
 
 // X and Y passes with the CTA's slice of V in shared memory (2D): the same
@@ -947,53 +1193,127 @@ __device__ __forceinline__ void warp_slots_k2(T (*red)[LMAX],
 // pass of the same step needs at the same points (no reload through L2).
 template <typename T, int DIM>
 struct XCarry {
-  T c[2], nb[2][2 * DIM];
+  typename TagVal<T>::raw r[2][1 + 2 * DIM];  // w' at the point and around it, as read
   T kf[2][DIM == 3 ? 6 : 1];
   T z[2];
   bool pre;  // the w' values are those the next X pass needs
 };
 
-template <typename T, int DIM, int BS>
-__device__ __forceinline__ void prefetch_x(XCarry<T, DIM>& cy, const SolveTask& tk,
-                                           const T* __restrict__ WP, int lo, int hi, int n) {
-#pragma unroll
-  for (int u = 0; u < 2; u++) {
-    const int i = lo + (int)threadIdx.x + u * BS;
-    const bool ok = i < hi;
-    cy.c[u] = ok ? ldcg(WP + i) : T(0);
+// Neighbour offsets and whether they exist at point i (-x, +x, -y, +y (, -z, +z)).
+template <int DIM>
+struct Around {
+  int off[2 * DIM];
+  bool has[2 * DIM];
+  __device__ __forceinline__ Around(int i, int n) {
     const int ix = i % n;
     const int iy = DIM == 3 ? (i / n) % n : i / n;
-    const int iz = DIM == 3 ? i / (n * n) : 0;
-    const int off[6] = {-1, 1, -n, n, -n * n, n * n};
-    const bool has[6] = {ix > 0, ix < n - 1, iy > 0, iy < n - 1, iz > 0, iz < n - 1};
-#pragma unroll
-    for (int f = 0; f < 2 * DIM; f++) cy.nb[u][f] = ok && has[f] ? ldcg(WP + i + off[f]) : T(0);
+    off[0] = -1;
+    off[1] = 1;
+    off[2] = -n;
+    off[3] = n;
+    has[0] = ix > 0;
+    has[1] = ix < n - 1;
+    has[2] = iy > 0;
+    has[3] = iy < n - 1;
     if constexpr (DIM == 3) {
-      // a wall face: kappa of the point itself, against u = 0
-      if (tk.kappa && ok) {
-        const T kc = (T)__ldg(tk.kappa + i);
-#pragma unroll
-        for (int f = 0; f < 6; f++) {
-          const int at = i + ((f & 1) ? 0 : off[f]);
-          if constexpr (sizeof(T) == 8)
-            cy.kf[u][f] = has[f] ? __ldg(tk.faces64 + (f >> 1) * tk.f64stride + at) : kc;
-          else
-            cy.kf[u][f] = has[f] ? __ldg(tk.faces + (f >> 1) * tk.fstride + at) : kc;
-        }
-      } else {
-#pragma unroll
-        for (int f = 0; f < 6; f++) cy.kf[u][f] = T(1);
-      }
+      const int iz = i / (n * n);
+      off[4] = -n * n;
+      off[5] = n * n;
+      has[4] = iz > 0;
+      has[5] = iz < n - 1;
     }
   }
+};
+
+// Face coefficients around point i (1 without kappa; a wall face: kappa of the
+// point itself, against u = 0).
+template <typename T>
+__device__ __forceinline__ void load_faces(T (&kf)[6], const SolveTask& tk, int i,
+                                           const Around<3>& a) {
+  if (!tk.kappa) {
+#pragma unroll
+    for (int f = 0; f < 6; f++) kf[f] = T(1);
+    return;
+  }
+  const T kc = (T)__ldg(tk.kappa + i);
+#pragma unroll
+  for (int f = 0; f < 6; f++) {
+    const int at = i + ((f & 1) ? 0 : a.off[f]);
+    if constexpr (sizeof(T) == 8)
+      kf[f] = a.has[f] ? __ldg(tk.faces64 + (f >> 1) * tk.f64stride + at) : kc;
+    else
+      kf[f] = a.has[f] ? __ldg(tk.faces + (f >> 1) * tk.fstride + at) : kc;
+  }
+}
+
+// Reads w' at P points and around them (0 outside the grid; point u is i0 + u BS):
+// the loads only, so that they can be in flight beside other work ...
+template <typename T, int DIM, int P, int BS>
+__device__ __forceinline__ void read_points(typename TagVal<T>::raw (&r)[P][1 + 2 * DIM],
+                                            const void* W, int i0, int hi, int n, unsigned tag) {
+  using V = TagVal<T>;
+#pragma unroll
+  for (int u = 0; u < P; u++) {
+    const int i = i0 + u * BS;
+    const bool ok = i < hi;
+    const Around<DIM> a(i, n);
+    r[u][0] = ok ? V::get(W, i) : V::none(tag);
+#pragma unroll
+    for (int f = 0; f < 2 * DIM; f++)
+      r[u][1 + f] = ok && a.has[f] ? V::get(W, i + a.off[f]) : V::none(tag);
+  }
+}
+// ... and waits (bounded) until all of them have arrived, reading again if not.
+template <typename T, int DIM, int P, int BS>
+__device__ __forceinline__ void settle_points(typename TagVal<T>::raw (&r)[P][1 + 2 * DIM],
+                                              const void* W, int i0, int hi, int n, unsigned tag,
+                                              const GroupBarrier& gb) {
+  SpinLimit lim;
+  for (;;) {
+    bool good = true;
+#pragma unroll
+    for (int u = 0; u < P; u++)
+#pragma unroll
+      for (int f = 0; f < 1 + 2 * DIM; f++) good = good && TagVal<T>::ok(r[u][f], tag);
+    if (good || !lim.more(gb)) return;
+    read_points<T, DIM, P, BS>(r, W, i0, hi, n, tag);
+  }
+}
+
+template <typename T, int DIM, int BS>
+__device__ __forceinline__ void prefetch_x(XCarry<T, DIM>& cy, const SolveTask& tk, const void* W,
+                                           int lo, int hi, int n, unsigned tag) {
+  const int i0 = lo + (int)threadIdx.x;
+  if constexpr (DIM == 3) {
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+      if (i0 + u * BS < hi) load_faces<T>(cy.kf[u], tk, i0 + u * BS, Around<3>(i0 + u * BS, n));
+  }
+  read_points<T, DIM, 2, BS>(cy.r, W, i0, hi, n, tag);
   cy.pre = true;
+}
+
+// Waits until the values of w' that this CTA's points read from other CTAs have
+// arrived (the 2D rows before lo and after hi), so that its threads may read them
+// without looking at their tags once a CTA barrier has passed.
+template <typename T, int BS>
+__device__ __forceinline__ void await_halo2d(const void* W, int lo, int hi, int n, int N,
+                                             unsigned tag, const GroupBarrier& gb) {
+  using V = TagVal<T>;
+  for (int h = threadIdx.x; h < 2 * n; h += BS) {
+    const int i = h < n ? lo - n + h : hi + (h - n);
+    if (i < 0 || i >= N) continue;
+    SpinLimit lim;
+    while (!V::ok(V::get(W, i), tag) && lim.more(gb)) {
+    }
+  }
 }
 
 template <typename T, int DIM, int MAXM, int BS, int K>
 __device__ __forceinline__ void x_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi, int j, int n,
-                                          const T* __restrict__ WP, T* __restrict__ Z,
-                                          T* __restrict__ Vs, int rows, const SolveTask& tk,
-                                          T s2t, XCarry<T, DIM>& cy) {
+                                          const void* WT, unsigned wtag, const GroupBarrier& gb,
+                                          T* __restrict__ Z, T* __restrict__ Vs, int rows,
+                                          const SolveTask& tk, T s2t, XCarry<T, DIM>& cy) {
   constexpr int LMAX = MAXM + 2;
   using T2 = typename Vec2<T>::type;
   const int tid = threadIdx.x;
@@ -1015,30 +1335,47 @@ __device__ __forceinline__ void x_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi,
     }
   }
   // one point per trip, the loop not unrolled: the body sits in the
-  // instruction stream once (the step's code is what bounds it at this size)
+  // instruction stream once (the step's code is what bounds it at this size).
   int t = 0;
 #pragma unroll 1
   for (int i = lo + tid; i < hi; i += BS, t++) {
     T wp, znum;
-    if (t < 2 && cy.pre) {
+    if (sizeof(T) == 8 && !(t < 2 && cy.pre)) {
+      // (untagged values; loading every trip's points one way, as below, cost 256^2
+      // FP64 26.8 -> 27.3 us per step)
+      wp = ldcg((const T*)WT + i);
+      znum = s2t * stencil_any<T, DIM>(tk, (const T*)WT, i, wp);
+    } else {
       // the same differences, in the same order, as stencil2d / stencil3d
-      const bool s1 = t == 1;
-      const T uc = s1 ? cy.c[1] : cy.c[0];
-      T d[2 * DIM];
+      T d[2 * DIM], kf[6];
+      if (sizeof(T) == 8 || t < 2) {
+        const bool s1 = t == 1;
+        using V = TagVal<T>;
+        wp = V::val(s1 ? cy.r[1][0] : cy.r[0][0]);
 #pragma unroll
-      for (int f = 0; f < 2 * DIM; f++) d[f] = uc - (s1 ? cy.nb[1][f] : cy.nb[0][f]);
-      wp = uc;
+        for (int f = 0; f < 2 * DIM; f++)
+          d[f] = wp - V::val(s1 ? cy.r[1][1 + f] : cy.r[0][1 + f]);
+        if constexpr (DIM == 3)
+#pragma unroll
+          for (int f = 0; f < 6; f++) kf[f] = s1 ? cy.kf[1][f] : cy.kf[0][f];
+      } else {
+        using V = TagVal<T>;
+        typename V::raw r1[1][1 + 2 * DIM];
+        if constexpr (DIM == 3) load_faces<T>(kf, tk, i, Around<3>(i, n));
+        read_points<T, DIM, 1, BS>(r1, WT, i, hi, n, wtag);
+        settle_points<T, DIM, 1, BS>(r1, WT, i, hi, n, wtag, gb);
+        wp = V::val(r1[0][0]);
+#pragma unroll
+        for (int f = 0; f < 2 * DIM; f++) d[f] = wp - V::val(r1[0][1 + f]);
+      }
       if constexpr (DIM == 2) {
         znum = s2t * ((d[0] + d[1]) + (d[2] + d[3]));
       } else {
         T acc3 = T(0);
 #pragma unroll
-        for (int f = 0; f < 6; f++) acc3 += (s1 ? cy.kf[1][f] : cy.kf[0][f]) * d[f];
+        for (int f = 0; f < 6; f++) acc3 += kf[f] * d[f];
         znum = s2t * acc3;
       }
-    } else {
-      wp = ldcg(WP + i);
-      znum = s2t * stencil_any<T, DIM>(tk, WP, i, wp);
     }
     const T* vc = Vs + vbase(i - lo, rows);
     T sv, sz;
@@ -1047,7 +1384,7 @@ __device__ __forceinline__ void x_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi,
       float2 av = make_float2(0.f, 0.f), az = make_float2(0.f, 0.f);
 #pragma unroll
       for (int q = 0; q < K / 2; q++) {
-        if (q < np) {
+        if (q < kSure<T, K, MAXM> || q < np) {
           const float2 v = *reinterpret_cast<const float2*>(vc + (q << 6));
           const float4 hq = h2r[q >> 1], cq = ccr[q >> 1];
           av = fma2((q & 1) ? make_float2(hq.z, hq.w) : make_float2(hq.x, hq.y), v, av);
@@ -1066,15 +1403,14 @@ __device__ __forceinline__ void x_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi,
     if (t == 0) cy.z[0] = z;
     if (t == 1) cy.z[1] = z;
     accZ += z * z;
-    x_dots<T, K>(acc, vc, j, z);
+    x_dots<T, K, MAXM>(acc, vc, j, z);
   }
-  warp_slots_k2<LMAX, K, T>(sm.red, acc, j + 1);
-  warp_slot<LMAX>(sm.red, j + 1, accZ);
+  warp_partials<LMAX, K, T>(sm.red, acc, accZ, j, lo + (tid & ~31) < hi);
 }
 
 template <typename T, int DIM, int MAXM, int BS, int K>
 __device__ __forceinline__ void y_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi, int j,
-                                          T* __restrict__ WP, const T* __restrict__ Z,
+                                          void* WT, unsigned ytag, const T* __restrict__ Z,
                                           const T* __restrict__ Vs, int rows,
                                           const XCarry<T, DIM>& cy) {
   constexpr int LMAX = MAXM + 2;
@@ -1104,7 +1440,7 @@ __device__ __forceinline__ void y_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi,
       float2 a = make_float2(0.f, 0.f);
 #pragma unroll
       for (int qq = 0; qq < K / 2; qq++) {
-        if (qq < np) {
+        if (qq < kSure<T, K, MAXM> || qq < np) {
           const float4 hq = h1r[qq >> 1];
           a = fma2((qq & 1) ? make_float2(hq.z, hq.w) : make_float2(hq.x, hq.y),
                    *reinterpret_cast<const float2*>(vc + (qq << 6)), a);
@@ -1114,9 +1450,172 @@ __device__ __forceinline__ void y_pass_sm(Smem<T, MAXM, BS>& sm, int lo, int hi,
     } else {
       qv = q - y_proj<T, MAXM, BS, K, !compact_bucket<MAXM>()>(sm, vc, j);
     }
-    WP[i] = qv;
+    TagVal<T>::put(WT, i, qv, ytag);
     accN += qv * qv;
-    y_dots<T, K>(acc, vc, j, qv);
+    y_dots<T, K, MAXM>(acc, vc, j, qv);
+  }
+  warp_partials<LMAX, K, T>(sm.red, acc, accN, j, lo + (tid & ~31) < hi);
+}
+
+// The same passes for long slices (FP32 2D, one CTA per SM; chosen in run_solver):
+// two points per trip, so that two projection chains are in flight per warp (with 8
+// warps per SM a single chain leaves issue slots idle), and the stencil's values and z of the next trip's points loaded
+// one trip ahead, so that no trip waits for L2.  The first trip's points come
+// with the carry.  The sums are those of the one-point passes, in their order.
+template <typename T, int MAXM, int BS, int K>
+__device__ __forceinline__ void x_pass_sl(Smem<T, MAXM, BS>& sm, int lo, int hi, int j, int n,
+                                          const void* WT, unsigned wtag, const GroupBarrier& gb,
+                                          T* __restrict__ Z, T* __restrict__ Vs, int rows,
+                                          const SolveTask& tk, T s2t, XCarry<T, 2>& cy) {
+  constexpr int LMAX = MAXM + 2;
+  using V = TagVal<T>;
+  const int tid = threadIdx.x;
+  float2 acc[K / 2];
+#pragma unroll
+  for (int q = 0; q < K / 2; q++) acc[q] = make_float2(0.f, 0.f);
+  T accZ = T(0);
+  const T inv = sm.invT;
+  const T cj = sm.cv[j];
+  const int np = (j + 1) >> 1;
+  T nb[2][5];  // this trip's points
+#pragma unroll
+  for (int u = 0; u < 2; u++)
+#pragma unroll
+    for (int f = 0; f < 5; f++) nb[u][f] = V::val(cy.r[u][f]);
+#pragma unroll 1
+  for (int i = lo + tid; i < hi; i += 2 * BS) {
+    const bool two = i + BS < hi;
+    T wp[2], znum[2], nx[2][5];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      // the same differences, in the same order, as stencil2d
+      wp[u] = nb[u][0];
+      znum[u] = s2t * (((wp[u] - nb[u][1]) + (wp[u] - nb[u][2])) +
+                       ((wp[u] - nb[u][3]) + (wp[u] - nb[u][4])));
+    }
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int i2 = i + (2 + u) * BS;
+      if (i2 < hi) {  // (arrived: the rows of other CTAs were awaited, await_halo2d)
+        const Around<2> a(i2, n);
+        nx[u][0] = V::seen(WT, i2);
+#pragma unroll
+        for (int f = 0; f < 4; f++) nx[u][1 + f] = a.has[f] ? V::seen(WT, i2 + a.off[f]) : T(0);
+      }
+    }
+    T* v0 = Vs + vbase(i - lo, rows);
+    T* v1 = two ? Vs + vbase(i + BS - lo, rows) : v0;
+    float2 av[2], az[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) av[u] = az[u] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int p = 0; p < K / 4; p++) {
+      const float4 h4 = reinterpret_cast<const float4*>(sm.h2v)[p];
+      const float4 c4 = reinterpret_cast<const float4*>(sm.cv)[p];
+#pragma unroll
+      for (int e = 0; e < 2; e++) {
+        const int q = 2 * p + e;
+        if (q < kSure<T, K, MAXM> || q < np) {
+          const float2 h = e ? make_float2(h4.z, h4.w) : make_float2(h4.x, h4.y);
+          const float2 c = e ? make_float2(c4.z, c4.w) : make_float2(c4.x, c4.y);
+          const float2 a = *reinterpret_cast<const float2*>(v0 + (q << 6));
+          const float2 b = *reinterpret_cast<const float2*>(v1 + (q << 6));
+          av[0] = fma2(h, a, av[0]);
+          av[1] = fma2(h, b, av[1]);
+          az[0] = fma2(c, a, az[0]);
+          az[1] = fma2(c, b, az[1]);
+        }
+      }
+    }
+    T z[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const T vj = (wp[u] - (av[u].x + av[u].y)) * inv;
+      z[u] = ((znum[u] - (az[u].x + az[u].y)) - cj * vj) * inv;
+      if (u == 0 || two) {
+        store_vj(u ? v1 : v0, j, vj);
+        Z[i + u * BS] = z[u];
+      }
+    }
+    if (!two) z[1] = T(0);  // (its column is the first point's: adds nothing)
+    if (i == lo + tid) {
+      cy.z[0] = z[0];
+      cy.z[1] = z[1];
+    }
+    accZ += z[0] * z[0];
+    accZ += z[1] * z[1];
+    const int nd = (j >> 1) + 1;
+    const float2 z0 = make_float2(z[0], z[0]), z1 = make_float2(z[1], z[1]);
+#pragma unroll
+    for (int q = 0; q < K / 2; q++)
+      if (q < kSure<T, K, MAXM> || q < nd) {
+        const float2 a = *reinterpret_cast<const float2*>(v0 + (q << 6));
+        const float2 b = *reinterpret_cast<const float2*>(v1 + (q << 6));
+        acc[q] = fma2(a, z0, acc[q]);
+        acc[q] = fma2(b, z1, acc[q]);
+      }
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+#pragma unroll
+      for (int f = 0; f < 5; f++) nb[u][f] = nx[u][f];
+  }
+  warp_slots_k2<LMAX, K, T>(sm.red, acc, j + 1);
+  warp_slot<LMAX>(sm.red, j + 1, accZ);
+}
+
+template <typename T, int MAXM, int BS, int K>
+__device__ __forceinline__ void y_pass_sl(Smem<T, MAXM, BS>& sm, int lo, int hi, int j, void* WT,
+                                          unsigned ytag, const T* __restrict__ Z,
+                                          const T* __restrict__ Vs, int rows,
+                                          const XCarry<T, 2>& cy) {
+  constexpr int LMAX = MAXM + 2;
+  const int tid = threadIdx.x;
+  float2 acc[K / 2];
+#pragma unroll
+  for (int q = 0; q < K / 2; q++) acc[q] = make_float2(0.f, 0.f);
+  T accN = T(0);
+  const int np = (j >> 1) + 1;
+  T zq[2] = {cy.z[0], cy.z[1]};
+#pragma unroll 1
+  for (int i = lo + tid; i < hi; i += 2 * BS) {
+    const bool two = i + BS < hi;
+    T zn[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) zn[u] = i + (2 + u) * BS < hi ? Z[i + (2 + u) * BS] : T(0);
+    const T* v0 = Vs + vbase(i - lo, rows);
+    const T* v1 = two ? Vs + vbase(i + BS - lo, rows) : v0;
+    float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+    for (int p = 0; p < K / 4; p++) {
+      const float4 h4 = reinterpret_cast<const float4*>(sm.coef)[p];
+#pragma unroll
+      for (int e = 0; e < 2; e++) {
+        const int q = 2 * p + e;
+        if (q < kSure<T, K, MAXM> || q < np) {
+          const float2 h = e ? make_float2(h4.z, h4.w) : make_float2(h4.x, h4.y);
+          s[0] = fma2(h, *reinterpret_cast<const float2*>(v0 + (q << 6)), s[0]);
+          s[1] = fma2(h, *reinterpret_cast<const float2*>(v1 + (q << 6)), s[1]);
+        }
+      }
+    }
+    T w[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      w[u] = zq[u] - (s[u].x + s[u].y);
+      if (u == 0 || two) TagVal<T>::put(WT, i + u * BS, w[u], ytag);
+    }
+    if (!two) w[1] = T(0);
+    accN += w[0] * w[0];
+    accN += w[1] * w[1];
+    const float2 w0 = make_float2(w[0], w[0]), w1 = make_float2(w[1], w[1]);
+#pragma unroll
+    for (int q = 0; q < K / 2; q++)
+      if (q < kSure<T, K, MAXM> || q < np) {
+        acc[q] = fma2(*reinterpret_cast<const float2*>(v0 + (q << 6)), w0, acc[q]);
+        acc[q] = fma2(*reinterpret_cast<const float2*>(v1 + (q << 6)), w1, acc[q]);
+      }
+    zq[0] = zn[0];
+    zq[1] = zn[1];
   }
   warp_slots_k2<LMAX, K, T>(sm.red, acc, j + 1);
   warp_slot<LMAX>(sm.red, j + 1, accN);
@@ -1520,7 +2019,7 @@ __device__ __forceinline__ void x_pass_bulk(Smem<T, MAXM, BS>& sm, int lo, int h
       store_vj(const_cast<T*>(sc), j, vj);
       Z[i] = z;
       // points past the end of a ragged last tile hold stale values: skipped
-      x_dots<T, K>(acc, sc, j, z);
+      x_dots<T, K, MAXM>(acc, sc, j, z);
       accZ += z * z;
     }
     __syncwarp();
@@ -1573,7 +2072,7 @@ __device__ __forceinline__ void y_pass_bulk(Smem<T, MAXM, BS>& sm, int lo, int h
                    y_proj<T, MAXM, BS, K, DIM == 3>(sm, sc, j);
       WP[i] = qv;
       accN += qv * qv;
-      y_dots<T, K>(acc, sc, j, qv);
+      y_dots<T, K, MAXM>(acc, sc, j, qv);
     }
     __syncwarp();
     if (lane == 0 && q + r.P < nq)
@@ -1614,7 +2113,7 @@ __device__ __forceinline__ void y_pass_bulk(Smem<T, MAXM, BS>& sm, int lo, int h
 // if it ends the cycle, that speculative pass is discarded.
 template <typename T, int DIM, int MAXM, int BS, int VM>
 __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWork& w, int lb,
-                          int nb, unsigned long long& epoch, unsigned& bphase,
+                          int nb, unsigned long long& epoch, unsigned& xseq, unsigned& bphase,
                           Smem<T, MAXM, BS>& sm) {
   constexpr int LD = MAXM + 1;
   constexpr int LMAX = MAXM + 2;
@@ -1628,13 +2127,15 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
   chunk = (chunk + 31) & ~31;  // whole tiles of the basis layout
   const int lo = min(N, lb * chunk);
   const int hi = min(N, lo + chunk);
-  const int rows = m + 1;  // basis vectors per tile (V holds m+1 vectors)
+  // basis vectors per tile (streamed bases keep m + 1: at m = 40 tiles of exactly 5 KB
+  // run 1% slower from HBM)
+  const int rows = in_shared(VM) ? slice_rows(sizeof(T) == 4, DIM, m) : m + 1;
   // V lives in shared memory when this CTA's slice fits the reserved space
   // (latency of a shared load instead of an L2 round trip); else in HBM.
   // (only the FP32 2D variant has slices small enough to be worth it; each
   // placement of V is its own kernel variant, so every pass uses the right
   // address space and registers are allocated per variant)
-  const bool vshared = VM == kVShared;
+  const bool vshared = in_shared(VM);
   T* __restrict__ Vg = (T*)w.V;
   T* __restrict__ Vs = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(&sm) +
                                             smem_own_bytes<T, MAXM, BS>());
@@ -1651,6 +2152,9 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
   pipe.err = w.bar.err;
   pipe.timeout_ns = w.bar.timeout_ns;
   T* __restrict__ WP = (T*)w.W0;  // w' (read by neighbours in X, rewritten in Y)
+  // (the shared-slice variants keep w' with tags in w.Wt instead; wtag is the tag
+  // of its current contents, and xseq counts the tagged exchanges of the launch)
+  unsigned wtag = 0;
   T* __restrict__ Z = (T*)w.W1;   // z = A v_j, own rows only
   // what the bulk-copy stages carry besides V (kappa only when its copies can
   // be 16-byte aligned: aligned base, N a multiple of 4)
@@ -1686,7 +2190,7 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
   double bnorm = 0.0;
   bool ok = true;
 
-  if (VM == kVShared && (long long)chunk * vrows_p(rows) * (long long)sizeof(T) > kp.vsmem) {
+  if (in_shared(VM) && (long long)chunk * vrows_p(rows) * (long long)sizeof(T) > kp.vsmem) {
     status = kErrConfig;  // the slice would overrun the shared-memory reservation
     goto finish;
   }
@@ -1749,6 +2253,7 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
   for (;;) {
     // ---- restart: w'_0 = r = b - A x (FP64), beta = ||r||
     {
+      wtag = ++xseq;
       double v0 = 0.0;
       for (int i = lo + tid; i < hi; i += BS) {
         double ri;
@@ -1758,7 +2263,10 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
           const double xc = ldcg(tk.x + i);
           ri = tk.b[i] - s2 * stencil64<DIM>(tk, tk.x, i, xc);
         }
-        WP[i] = (T)ri;
+        if constexpr (in_shared(VM))
+          TagVal<T>::put(w.Wt, i, (T)ri, wtag);
+        else
+          WP[i] = (T)ri;
         v0 += ri * ri;
       }
       for (int k = tid; k < LMAX; k += BS) {
@@ -1802,11 +2310,21 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
       // while thread 0 waits at the group barrier
       {
 #define MLG_X(KK) x_pass<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vg, rows, 0, tk, s2t)
-#define MLG_XS(KK) x_pass_sm<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vs, rows, tk, s2t, cy)
+#define MLG_XS(KK) \
+  x_pass_sm<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, w.Wt, wtag, w.bar, Z, Vs, rows, tk, s2t, cy)
 #define MLG_XB(KK)                                                                       \
   x_pass_bulk<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, n, WP, Z, Vg, rows, kappa, s2t, pipe, bphase, \
                                     auxs)
-        if constexpr (VM == kVShared) {
+#define MLG_XL(KK) \
+  x_pass_sl<T, MAXM, BS, KK>(sm, lo, hi, j, n, w.Wt, wtag, w.bar, Z, Vs, rows, tk, s2t, cy)
+        if constexpr (tagged<T>(VM)) {
+          // (once here, not in every bucket: the step's code is fetched anew each step)
+          if (!cy.pre) prefetch_x<T, DIM, BS>(cy, tk, w.Wt, lo, hi, n, wtag);
+          settle_points<T, DIM, 2, BS>(cy.r, w.Wt, lo + tid, hi, n, wtag, w.bar);
+        }
+        if constexpr (VM == kVSharedL) {
+          MLG_BUCKETS(MLG_XL)
+        } else if constexpr (VM == kVShared) {
           MLG_BUCKETS(MLG_XS)
         } else if constexpr (VM == kVBulk) {
           MLG_BUCKETS(MLG_XB)
@@ -1815,6 +2333,7 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
         }
 #undef MLG_X
 #undef MLG_XS
+#undef MLG_XL
 #undef MLG_XB
         if (arnoldi && j == jmax) { kcols = j; break; }
         auto givens_prev = [&]() {
@@ -1824,24 +2343,33 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
         };
         // the Givens rotation of column j-1 (warp 1) overlaps the barrier and
         // the gather; its stop code is read after the gather
-        finish_and_sync_side<LMAX, BS, T>(min(j + 2, LMAX), (T*)part(), lb, sm.red, ps, w.bar,
-                                          epoch, &sm.flag, givens_prev);
-        gather<BS, T, T, true>((const T*)part(), j + 2, nb, sm.tot, sm.coef, ps);
-        if (!sm.flag) goto abort;
+        if constexpr (tagged<T>(VM)) {
+          ok = exchange<LMAX, BS, true>(j + 2, w.words, lb, nb, sm.red, ps, w.bar, epoch, ++xseq,
+                                        sm.coef, &sm.flag, givens_prev, NoSide());
+        } else {
+          finish_and_sync_side<LMAX, BS, T>(j + 2, (T*)part(), lb, sm.red, ps, w.bar, epoch,
+                                            &sm.flag, givens_prev);
+          gather<BS, T, T, true>((const T*)part(), j + 2, nb, sm.tot, sm.coef, ps);
+          red++;
+          ok = sm.flag != 0;
+        }
+        if (!ok) goto abort;
         const int stop = sm.stop;
         if (stop == 2) { status = kErrNonfinite; goto finish; }
         if (stop == 1) { kcols = j; break; }
-        red++;
         if (tid <= j) sm.h1c[tid] = sm.coef[tid];
         if (tid == 0) sm.anorm2T = sm.coef[j + 1];
       }
       // ---- Y: w'_{j+1} = z - V h1, h2 = V^T w'_{j+1}, ||w'_{j+1}||^2
       {
 #define MLG_Y(KK) y_pass<T, MAXM, BS, KK>(sm, lo, hi, j, WP, Z, Vg, rows, 0)
-#define MLG_YS(KK) y_pass_sm<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, WP, Z, Vs, rows, cy)
+#define MLG_YS(KK) y_pass_sm<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, w.Wt, xseq + 1, Z, Vs, rows, cy)
 #define MLG_YB(KK) \
   y_pass_bulk<T, DIM, MAXM, BS, KK>(sm, lo, hi, j, WP, Z, Vg, rows, pipe, bphase, w.ldv)
-        if constexpr (VM == kVShared) {
+#define MLG_YL(KK) y_pass_sl<T, MAXM, BS, KK>(sm, lo, hi, j, w.Wt, xseq + 1, Z, Vs, rows, cy)
+        if constexpr (VM == kVSharedL) {
+          MLG_BUCKETS(MLG_YL)
+        } else if constexpr (VM == kVShared) {
           MLG_BUCKETS(MLG_YS)
         } else if constexpr (VM == kVBulk) {
           MLG_BUCKETS(MLG_YB)
@@ -1850,14 +2378,27 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
         }
 #undef MLG_Y
 #undef MLG_YS
+#undef MLG_YL
 #undef MLG_YB
-        ok = finish_and_sync<LMAX, BS, T>(j + 2, (T*)part(), lb, sm.red, ps, w.bar, epoch,
-                                          &sm.flag, NoSide());
+        // the next X pass's loads of w' go out before the gather
+        if constexpr (tagged<T>(VM)) {
+          wtag = ++xseq;
+          auto ahead_of_x = [&]() {
+            prefetch_x<T, DIM, BS>(cy, tk, w.Wt, lo, hi, n, wtag);
+            if constexpr (VM == kVSharedL) await_halo2d<T, BS>(w.Wt, lo, hi, n, N, wtag, w.bar);
+          };
+          ok = exchange<LMAX, BS, false>(j + 2, w.words, lb, nb, sm.red, ps, w.bar, epoch, wtag,
+                                         sm.coef, &sm.flag, NoSide(), ahead_of_x);
+        } else {
+          ok = finish_and_sync<LMAX, BS, T>(j + 2, (T*)part(), lb, sm.red, ps, w.bar, epoch,
+                                            &sm.flag, NoSide());
+          if (!ok) goto abort;
+          // w' is final everywhere
+          if constexpr (in_shared(VM)) prefetch_x<T, DIM, BS>(cy, tk, w.Wt, lo, hi, n, wtag);
+          gather<BS, T, T>((const T*)part(), j + 2, nb, sm.tot, sm.coef, ps);
+          red++;
+        }
         if (!ok) goto abort;
-        // w' is final everywhere: the next X pass's loads go out before the gather
-        if constexpr (VM == kVShared) prefetch_x<T, DIM, BS>(cy, tk, WP, lo, hi, n);
-        gather<BS, T, T>((const T*)part(), j + 2, nb, sm.tot, sm.coef, ps);
-        red++;
       }
       iters++;
       // ---- column j of Hu; hn_{j+1} = sqrt(||w'||^2 - ||h2||^2), in the working
@@ -1944,11 +2485,14 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
         // cancellation: apply h2 explicitly and measure ||w''||
         T accN = T(0);
         for (int i = lo + tid; i < hi; i += BS) {
-          T q = WP[i];
+          T q = in_shared(VM) ? TagVal<T>::seen(w.Wt, i) : WP[i];
 #pragma unroll
           for (int k = 0; k < MAXM; k++)
             if (k <= j) q -= sm.h2v[k] * V[vix(k, i - voff, rows)];
-          WP[i] = q;
+          if constexpr (in_shared(VM))
+            TagVal<T>::put(w.Wt, i, q, wtag);  // (the group barrier below orders it)
+          else
+            WP[i] = q;
           accN += q * q;
         }
         warp_slot<LMAX>(sm.red, 0, accN);
@@ -2132,6 +2676,7 @@ __global__ void __launch_bounds__(BS, MINB) gmres_persistent(KParams kp) {
   const int nb = kp.group_first[g + 1] - kp.group_first[g];
   const GroupWork w = kp.work[g];
   unsigned long long epoch = 0;
+  unsigned xseq = 0;    // tagged exchanges of this launch so far
   unsigned bphase = 0;  // parity of each bulk-copy stage of this thread's warp
   static_assert(r_in_shared<MAXM>() == (MINB == 1), "R placement follows the variant");
   if (!r_in_shared<MAXM>() && threadIdx.x == 0)
@@ -2142,9 +2687,14 @@ __global__ void __launch_bounds__(BS, MINB) gmres_persistent(KParams kp) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
   }
+  // this CTA's words start without a tag (an earlier launch's tags mean nothing);
+  // the first group barrier of a task orders this before any exchange
+  if constexpr (tagged<T>(VM))
+    for (int i = threadIdx.x; i < 2 * kTagWordRows; i += BS)
+      st_relaxed_b128(w.words + (long long)i * w.pstride + lb, make_uint4(0u, 0u, 0u, 0u));
   for (int t = kp.task_first[g]; t < kp.task_first[g + 1]; t++) {
     const SolveTask tk = kp.tasks[kp.task_order[t]];
-    solve_one<T, DIM, MAXM, BS, VM>(kp, tk, w, lb, nb, epoch, bphase, sm);
+    solve_one<T, DIM, MAXM, BS, VM>(kp, tk, w, lb, nb, epoch, xseq, bphase, sm);
     if (*(volatile int*)w.bar.err != kErrNone) break;
     // all CTAs finish with this task's data before the next task starts
     if (!group_sync(w.bar, epoch, &sm.flag)) break;
@@ -2166,7 +2716,7 @@ template <typename T, int DIM, int MAXM, int BS, int VM, int MINB = 1>
 cudaError_t launch_t(const KParams& kp, int grid, cudaStream_t s) {
   if (kp.m > MAXM) return cudaErrorInvalidValue;
   int extra = 0;
-  if (VM == kVShared) extra = kp.vsmem;
+  if (in_shared(VM)) extra = kp.vsmem;
   if (VM == kVBulk) extra = (BS / 32) * kp.bulk_cap;
   cudaError_t e = prepare_t<T, DIM, MAXM, BS, VM, MINB>(extra);
   if (e != cudaSuccess) return e;

@@ -33,7 +33,9 @@ struct mlgmres {
   float* faces = nullptr;    // FP32 face coefficients (single 3D FP32 solves with kappa)
   long long fstride = 0;     // their array stride
   double* faces64 = nullptr; // FP64 face coefficients (single 3D solves with kappa), stride ldv
+  void* Wt = nullptr;        // w' with tags, if a single solve may run a shared-slice variant
   double* part = nullptr;
+  uint4* words = nullptr;    // tagged partial sums (single solves)
   double* Rg = nullptr;      // compact variants' triangles R (rg_blocks of them)
   int rg_blocks = 0;
   unsigned long long* bar = nullptr;  // per group: counter
@@ -52,8 +54,9 @@ struct mlgmres {
   int batch_groups = 0;
   bool batch_compact = false;         // batches may launch the compact variant
   void* Vb = nullptr;
-  void* Wb = nullptr;                 // 2 work vectors per group
+  void* Wb = nullptr;                 // work vectors per group: W0, W1, Wt (4 ldv elements)
   double* partb = nullptr;
+  uint4* wordsb = nullptr;
 
   // ---- guess state ----
   double* x_prev = nullptr;

@@ -61,6 +61,22 @@ unsigned long long splitmix_next(unsigned long long& st) {
   return z ^ (z >> 31);
 }
 
+// FP32 2D slices of V of more points than this are long (kVSharedL: two points per
+// trip of the passes).  Measured, one point per trip / two: single systems 430^2 (1217
+// points) 9.4 / 10.1 us per step, 512^2 (1725) 10.96 / 11.07, 600^2 (2369; GMRES(20))
+// 12.9 / 12.2; batches of 40 of 24^2 -
+// 160^2 37.1 / 36.1 ms, 48 of 60^2 - 170^2 (GMRES(20)) 116 / 102, 12 of 40^2 - 100^2
+// (largest: 534 points) 11.43 / 11.79.
+constexpr int kLongPoints = 2048, kLongPointsBatch = 1024;
+
+// Shared-memory bytes a CTA has for its slice of V.  (3D FP32: what the variant for
+// every m leaves, also for m <= kSmallM, so that 62^3 - 64^3 keep the streamed basis:
+// a few hundred FP32 steps with kappa that do not converge end up to 5e-8 apart when
+// their sums are taken in another order.)
+int slice_budget(const mlgmres* h, int dim) {
+  return gmres_vsmem_budget(h->fp32, h->fp32 && dim == 3 ? kMaxM : h->opt.m);
+}
+
 // Shared-memory bytes of a single solve's V slice at `blocks` CTAs (0 if the
 // slice does not fit).
 int single_vsmem(const mlgmres* h, int blocks, bool compact = false) {
@@ -69,9 +85,10 @@ int single_vsmem(const mlgmres* h, int blocks, bool compact = false) {
   // 3D with v_stages set: the caller asked for a basis streamed from HBM
   if (h->grid.dim == 3 && h->opt.v_stages >= 0) return 0;
   const long long chunk = (((long long)h->N + blocks - 1) / blocks + 31) / 32 * 32;
-  const long long need = chunk * vrows_p(h->opt.m + 1) * (h->fp32 ? 4 : 8);
+  const long long need =
+      chunk * vrows_p(slice_rows(h->fp32, h->grid.dim, h->opt.m)) * (h->fp32 ? 4 : 8);
   const int budget = compact ? (h->grid.dim == 2 ? gmres_compact_vsmem_budget() : 0)
-                             : gmres_vsmem_budget(h->fp32, h->opt.m);
+                             : slice_budget(h, h->grid.dim);
   return need <= budget ? (int)need : 0;
 }
 
@@ -299,6 +316,18 @@ void run_solver(mlgmres* h, int ngroups, int ntasks, int grid, int arnoldi_steps
       kp.compact = 1;  // V slices in shared memory, two CTAs per SM
     }
   }
+  // long slices: by the largest system's (the one a batch waits for)
+  if (kp.vmode == kVShared && !kp.compact && h->fp32 && h->grid.dim == 2) {
+    const int *gf = h->hcfg, *tf = gf + ngroups + 1, *order = tf + ngroups + 1;
+    int largest = 0, points = 0;
+    for (int g = 0; g < ngroups; g++)
+      for (int t = tf[g]; t < tf[g + 1]; t++)
+        if (h->htasks[order[t]].N > largest) {
+          largest = h->htasks[order[t]].N;
+          points = (largest - 1) / (gf[g + 1] - gf[g]) + 1;
+        }
+    if (points > (ngroups > 1 ? kLongPointsBatch : kLongPoints)) kp.vmode = kVSharedL;
+  }
   ARG(!kp.compact || (h->Rg && grid <= h->rg_blocks), "compact variant: grid exceeds its R workspace");
   // face coefficients from the current kappa (one pass over the grid)
   if (ntasks == 1 && h->htasks[0].faces64)
@@ -319,7 +348,9 @@ GroupWork single_group_work(mlgmres* h, int nblocks) {
   w.ldv = h->ldv;
   w.W0 = h->W0;
   w.W1 = h->W1;
+  w.Wt = h->Wt;
   w.part = h->part;
+  w.words = h->words;
   w.pstride = kPartStride;
   w.Rg = h->Rg;
   w.bar.ctr = h->bar;
@@ -653,6 +684,12 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
       CK(cudaMalloc(&h->faces64, sizeof(double) * 3 * (size_t)h->ldv));
     CK(cudaMalloc(&h->W1, es * (size_t)h->ldv));
     CK(cudaMalloc(&h->part, sizeof(double) * part_doubles(kPartStride)));
+    CK(cudaMalloc(&h->words, sizeof(uint4) * tag_words(kPartStride)));
+    // w' with tags, where some CTA count lets the slices of V fit
+    if (single_vsmem(h, h->max_blocks) > 0 ||
+        (gmres_compact_ok(h->fp32, grid->dim, opt->m) &&
+         single_vsmem(h, std::max(1, gmres_compact_max_blocks(grid->dim, opt->m)), true) > 0))
+      CK(cudaMalloc(&h->Wt, 2 * es * (size_t)h->ldv));
     if (opt->compact != 0 && gmres_compact_ok(h->fp32, grid->dim, opt->m)) {
       // the compact variants keep each CTA's triangle R in HBM (L2-resident),
       // which leaves room for a second bulk-copy stage per warp
@@ -673,8 +710,9 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
       h->cfg_cap = kBatchCap;
       const size_t G = (size_t)h->batch_groups;
       CK(cudaMalloc(&h->Vb, es * G * (size_t)vrows_p(opt->m + 1) * h->ldv));
-      CK(cudaMalloc(&h->Wb, es * G * 2 * (size_t)h->ldv));
+      CK(cudaMalloc(&h->Wb, es * G * 4 * (size_t)h->ldv));
       CK(cudaMalloc(&h->partb, sizeof(double) * G * part_doubles(1)));
+      CK(cudaMalloc(&h->wordsb, sizeof(uint4) * G * tag_words(1)));
     }
     CK(cudaMalloc(&h->bar, sizeof(unsigned long long) * h->group_cap));
     CK(cudaMalloc(&h->err, sizeof(int) * h->group_cap));
@@ -727,6 +765,9 @@ void mlgmres_destroy(mlgmres_t h) {
   cudaFree(h->Vb);
   cudaFree(h->Wb);
   cudaFree(h->partb);
+  cudaFree(h->wordsb);
+  cudaFree(h->Wt);
+  cudaFree(h->words);
   cudaFree(h->V);
   cudaFree(h->W0_alloc);
   if (h->faces) cudaFree(h->faces - (h->fstride - h->ldv) / 2);
@@ -920,9 +961,9 @@ mlgmres_status mlgmres_solve_batch(mlgmres_t h, int count, const mlgmres_grid* g
         const long long N = grid_points(dim, grids[i].n);
         const long long k = gc[go[i]];
         const long long chunk = ((N + k - 1) / k + 31) / 32 * 32;
-        need = std::max(need, chunk * vrows_p(h->opt.m + 1) * (long long)es0);
+        need = std::max(need, chunk * vrows_p(slice_rows(h->fp32, dim, h->opt.m)) * (long long)es0);
       }
-      return need <= gmres_vsmem_budget(h->fp32, h->opt.m) ? (int)need : 0;
+      return need <= slice_budget(h, dim) ? (int)need : 0;
     };
     // one CTA per SM first; if the basis streams from HBM anyway, the compact
     // variant (two CTAs per SM) gets all the reserved CTAs
@@ -961,15 +1002,18 @@ mlgmres_status mlgmres_solve_batch(mlgmres_t h, int count, const mlgmres_grid* g
       t.zero_x = h->opt.guess == MLGMRES_GUESS_USER ? 0 : 1;
       h->htasks[i] = t;
     }
-    long long part_off = 0;
+    long long part_off = 0, word_off = 0;
     for (int g = 0; g < G; g++) {
       GroupWork w;
       w.V = (char*)h->Vb + es * (size_t)g * vrows_p(h->opt.m + 1) * h->ldv;
       w.ldv = h->ldv;
-      w.W0 = (char*)h->Wb + es * (size_t)g * 2 * h->ldv;
+      w.W0 = (char*)h->Wb + es * (size_t)g * 4 * h->ldv;
       w.W1 = (char*)w.W0 + es * h->ldv;
+      w.Wt = (char*)w.W1 + es * h->ldv;
       w.part = h->partb + part_off;
       part_off += part_doubles(gctas[g]);
+      w.words = h->wordsb + word_off;
+      word_off += tag_words(gctas[g]);
       w.pstride = gctas[g];
       w.Rg = h->Rg;
       w.bar.ctr = h->bar + g;

@@ -16,14 +16,33 @@ constexpr int kCompactM3 = 56;
 constexpr int kSmallM = 32;
 // Where a launch keeps the basis V (one kernel variant each):
 constexpr int kVDirect = 0;  // HBM, loaded into registers by the passes
-constexpr int kVShared = 1;  // each CTA's slice in shared memory (2D)
+constexpr int kVShared = 1;  // each CTA's slice in shared memory
 constexpr int kVBulk = 2;    // HBM, streamed through per-warp bulk-copy stages
+constexpr int kVSharedL = 3; // kVShared for long slices (FP32 2D)
+__host__ __device__ constexpr bool in_shared(int vmode) {
+  return vmode == kVShared || vmode == kVSharedL;
+}
 constexpr int kPartStride = 1024;  // max CTAs per group (partials row length)
 // doubles in a group's partial-sum area (two alternating sets)
 constexpr long long part_doubles(int pstride) { return 2LL * (kMaxM + 2) * pstride; }
+// 16-byte words of a group's tagged partial sums: three slots each, two
+// alternating sets.
+constexpr int kTagWordRows = (kMaxM + 2 + 2) / 3;
+constexpr long long tag_words(int pstride) { return 2LL * kTagWordRows * pstride; }
+// Groups of at most this many CTAs exchange their sums without a counter (fewer in a
+// batch, where the readers of many groups spinning on words slow each other down; ms
+// up to 32, 16, 12 and 8 CTAs: 7 systems of 50^2 - 170^2 32.1, 28.3, 28.3, 27.9; 12 of
+// 40^2 - 100^2 12.2, 12.2, 12.0, 11.4; 48 of 60^2 - 170^2 101, 102, 102, 106).
+constexpr int kDirectCtas = 32, kDirectCtasBatch = 12;
 // Rows a tile of the basis occupies for `rows` vectors: V stores basis vectors
 // in pairs, so the count is rounded up to even (see gmres_kernel.cuh).
 __host__ __device__ constexpr int vrows_p(int rows) { return (rows + 1) & ~1; }
+// Basis vectors per tile of a shared-memory slice: FP32 2D v_0 .. v_{m-1} only (v_m is
+// stored only in Arnoldi mode, which streams: the last column of a cycle is rotated
+// without another X pass).  The other slices keep the streamed layout's m + 1.
+__host__ __device__ constexpr int slice_rows(bool fp32, int dim, int m) {
+  return fp32 && dim == 2 ? m : m + 1;
+}
 
 // Per-system result written by the solver (mirrors mlgmres_result's numeric part).
 struct DevResult {
@@ -70,8 +89,10 @@ struct GroupWork {
   long long ldv;
   void* W0;           // two work vectors (ping-pong), ldv each
   void* W1;
+  void* Wt;           // w' with tags (shared-slice variants), ldv words of 2 elements
   double* part;       // 2 x (kMaxM+2) x pstride partial sums
-  int pstride;        // row length of part (>= the group's CTA count)
+  uint4* words;       // tag_words(pstride): the tagged partial sums of the exchanges
+  int pstride;        // row length of part and words (>= the group's CTA count)
   double* Rg;         // compact variants: (m+1) x m FP64 triangle per CTA, indexed
                       // by blockIdx.x (the others keep R in shared memory)
   GroupBarrier bar;
@@ -88,7 +109,7 @@ struct KParams {
   int vsmem;                // bytes of shared memory for a CTA's slice of V (0 = V in HBM)
   int bulk_stages;          // most bulk-copy stages per warp when V is in HBM (0 = off)
   int bulk_cap;             // bytes of staging area per warp (>= m 32-point rows)
-  int vmode;                // kVDirect | kVShared | kVBulk (the kernel variant launched)
+  int vmode;                // kVDirect | kVShared | kVSharedL | kVBulk (the kernel variant launched)
   int compact;              // 1: the two-CTAs-per-SM bulk variant (FP32, m below its limit)
   int ngroups;
   const int* group_first;   // ngroups+1 CTA ranges
@@ -106,8 +127,8 @@ cudaError_t launch_gmres(const KParams& kp, bool fp32, int dim, int grid_blocks,
 int gmres_max_blocks(bool fp32, int dim, int m, int* block_threads);
 
 // Shared-memory bytes a CTA may use for its slice of V (so that slice + the
-// solver's own state fit the per-CTA limit); 0 if none.  The FP64 variant for
-// m <= kSmallM has a smaller state and so a larger budget.
+// solver's own state fit the per-CTA limit); 0 if none.  The variants for
+// m <= kSmallM have a smaller state and so a larger budget.
 int gmres_vsmem_budget(bool fp32, int m = kMaxM);
 
 // Most bulk-copy stages per warp (kMaxStages) for a basis in HBM.  A pass uses

@@ -20,9 +20,11 @@ constexpr int kStaticMaxM = 32;
 constexpr long long kStaticLdv = kStaticMaxN;  // a multiple of 64
 constexpr size_t kStaticBasis = sizeof(float) * (size_t)vrows_p(kStaticMaxM + 1) * kStaticLdv;
 constexpr size_t kStaticWork = 2 * sizeof(float) * (size_t)kStaticLdv;
-constexpr size_t kStaticPart = sizeof(double) * part_doubles(kPartStride);
+constexpr int kStaticStride = kStaticMaxN / 512;  // one CTA per 512 points
+constexpr size_t kStaticPart = sizeof(double) * part_doubles(kStaticStride);
+constexpr size_t kStaticWords = sizeof(uint4) * tag_words(kStaticStride);
 constexpr size_t kStaticMisc = 4096;  // barrier counter, error flag, result, launch tables
-constexpr size_t kStaticBytes = kStaticBasis + kStaticWork + kStaticPart + kStaticMisc;
+constexpr size_t kStaticBytes = kStaticBasis + kStaticWork + kStaticPart + kStaticWords + kStaticMisc;
 
 // The fixed workspace.  In host code this name is only a stand-in for the
 // symbol; the device address comes from cudaGetSymbolAddress.
@@ -78,6 +80,8 @@ extern "C" mlgmres_status mlgmres_solve_static(int n, int m, double rtol, long l
   p += kStaticWork;
   double* part = (double*)p;
   p += kStaticPart;
+  uint4* words = (uint4*)p;
+  p += kStaticWords;
   unsigned long long* bar = (unsigned long long*)p;
   int* err = (int*)(p + 8);
   DevResult* dres = (DevResult*)(p + 64);
@@ -91,7 +95,7 @@ extern "C" mlgmres_status mlgmres_solve_static(int n, int m, double rtol, long l
   if (maxb < 1) return MLGMRES_ERR_CUDA;
   long long want = (N + 511) / 512;
   int blocks = (int)(want < 1 ? 1 : (want > maxb ? maxb : want));
-  if (blocks > kPartStride) blocks = kPartStride;
+  if (blocks > kStaticStride) blocks = kStaticStride;
 
   int hcfg[5] = {0, blocks, 0, 1, 0};
   SolveTask t;
@@ -110,8 +114,10 @@ extern "C" mlgmres_status mlgmres_solve_static(int n, int m, double rtol, long l
   w.ldv = kStaticLdv;
   w.W0 = W0;
   w.W1 = W1;
+  w.Wt = nullptr;
   w.part = part;
-  w.pstride = kPartStride;
+  w.words = words;
+  w.pstride = kStaticStride;
   w.Rg = nullptr;
   w.bar.ctr = bar;
   w.bar.err = err;

@@ -45,7 +45,10 @@ def test_3d_slices_against_the_streamed_basis(n, m, prec):
     from paper_2103_10975_gb300 import Solver
     b = MovingGaussians3D(n, 5001, 50).rhs(2)
     bd = torch.as_tensor(b).cuda()
-    for kap in (None, lognormal_kappa(n, 5001, smooth_sigma=1.5).astype(np.float32)):
+    kaps = [None]
+    if n > 1:  # (one point has no spread to normalise: kappa would be 0)
+        kaps.append(lognormal_kappa(n, 5001, smooth_sigma=1.5).astype(np.float32))
+    for kap in kaps:
         xs = []
         for opt in ({}, {"v_stages": 2}):
             s = Solver(n, dim=3, kappa=kap, m=m, rtol=1e-10, precision=prec, **opt)
@@ -72,3 +75,12 @@ def test_jacobi_tiles(n):
         s.smooth(torch.as_tensor(b).cuda(), xd, sweeps)
         ref = og.jacobi(2, n, b, x0, sweeps, 0.75)
         assert np.linalg.norm(xd.cpu().numpy() - ref) <= 1e-13 * np.linalg.norm(ref), sweeps
+
+
+@pytest.mark.parametrize("n,m,blocks", [(33, 30, 1), (33, 30, 2), (33, 40, 5), (47, 20, 32),
+                                        (47, 31, 33), (64, 30, 96), (90, 12, 152), (61, 30, 4),
+                                        (123, 30, 9), (100, 33, 12)])
+def test_fp32_exchanges_and_long_slices(n, m, blocks):
+    """Group sizes on both sides of the direct exchange's limit, one CTA alone, more
+    than 128 CTAs, and slices of one tile up to many points per thread."""
+    _solve_2d(n, m=m, precision="fp32_refine", grid_blocks=blocks)
