@@ -131,7 +131,7 @@ typedef struct {
                                 a pass uses as many as fit in the warp's share of shared
                                 memory for its j rows), or 0 for direct loads; -1 =
                                 automatic (the autotuned value if mlgmres_autotune ran,
-                                else 16).  In 3D
+                                else as many as fit, 2 for large compact solves).  In 3D
                                 a value >= 0 also asks for the basis in HBM where its
                                 slices would fit in shared memory */
   int retrain_after;         /* f_r of Algorithm 1 (Sec. 2.2): when > 0, mlgmres_solve itself
@@ -150,8 +150,10 @@ typedef struct {
   int compact;               /* the two-CTAs-per-SM variants (at most 128 registers, smaller
                                 shared state) for FP32 grids: 2D with m <= 47 (V slices in
                                 shared memory when they fit, else streamed), 3D with m <= 55
-                                (streamed): -1 = if the autotuner chose it, 0 = never, 1 =
-                                always (where it applies) */
+                                (streamed): -1 = if the autotuner chose it, or untuned by
+                                size (a 2D streamed basis of 400 000 points and more, with
+                                grid_blocks and v_stages automatic), 0 = never, 1 = always
+                                (where it applies) */
   int model;                 /* MLGMRES_MODEL_CONV: the multi-scale network of Sec. 2.1;
                                 MLGMRES_MODEL_LINEAR: one dense layer x0 = c s T (b/s) =
                                 c T b (the simplified model of Sec. 3.1, for studying the

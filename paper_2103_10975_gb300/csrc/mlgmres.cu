@@ -107,6 +107,14 @@ int auto_blocks(const mlgmres* h, int N) {
       if (single_vsmem(h, nb) > 0) return nb;  // V in shared memory
     }
   }
+  if (h->fp32) {
+    // FP32 with V in shared memory: a tile per warp where the co-resident CTAs allow
+    // (us per step, GMRES(30), 16 tiles per CTA against 8: 64^2 6.66 / 6.48, 101^2
+    // 7.00 / 6.77, 160^2 7.19 / 6.81), as the passes of two cost more than the
+    // larger group's exchange
+    const int tiles = (N + 31) / 32, nb = (tiles + 7) / 8;
+    if (nb <= h->max_blocks && single_vsmem(h, nb) > 0) return nb;
+  }
   // about 512 grid points per CTA (two per thread): measured on GB300 at 256^2,
   // 128 CTAs take 18 us per Arnoldi step against 26 us with 64 and 43 us with 32;
   // never more CTAs than can be co-resident
@@ -660,6 +668,19 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
     h->ldv = ((long long)h->N + 63) / 64 * 64;
     // V slice in shared memory when it fits (the compact variant streams V)
     h->vsmem = single_vsmem(h, h->blocks, force_compact);
+    // Untuned default for a streamed FP32 basis: the compact variant (two CTAs per
+    // SM) from kCompactPoints on (measured, us per step, one CTA per SM against
+    // two: 520^2 m = 30 17.6 / 17.3, 640^2 22.3 / 20.7, 1024^2 46.0 / 37.5, 1500^2
+    // 91.4 / 73.3); two stages per warp where its passes are longest.  (In 3D it is
+    // left to the tuner: the other number of CTAs is another order of the sums, on
+    // which an unconverged FP32 solve with kappa depends, see slice_budget.)
+    constexpr int kCompactPoints = 400000;
+    if (grid->dim == 2 && opt->compact == -1 && opt->grid_blocks == 0 && opt->v_stages == -1 &&
+        h->vsmem == 0 && h->N >= kCompactPoints && gmres_compact_ok(h->fp32, grid->dim, opt->m)) {
+      h->blocks = std::min(gmres_compact_max_blocks(grid->dim, opt->m), kPartStride);
+      h->tuned_compact = 1;
+      if (h->N >= 1 << 20) h->default_stages = 2;
+    }
     const size_t es = h->fp32 ? sizeof(float) : sizeof(double);
     CK(cudaMalloc(&h->V, es * (size_t)vrows_p(opt->m + 1) * h->ldv));
     if (grid->dim == 3 && grid->kappa_dev && h->fp32) {
@@ -858,7 +879,8 @@ mlgmres_status mlgmres_solve(mlgmres_t h, const double* b, double* x, void* stre
       t.hist_cap = 0;
       t.zero_x = 0;
       stage_single(h, t, h->blocks);
-      run_solver(h, 1, 1, h->blocks, 0, s, h->vsmem, maxit, -1, use_compact(h));
+      const int stages = h->opt.v_stages < 0 && h->tuned_stages < 0 ? h->default_stages : -1;
+      run_solver(h, 1, 1, h->blocks, 0, s, h->vsmem, maxit, stages, use_compact(h));
       CK(cudaMemcpyAsync(h->hres, h->dres, sizeof(DevResult), cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
       return h->hres[0];
@@ -1252,8 +1274,10 @@ mlgmres_status mlgmres_arnoldi(mlgmres_t h, const double* v0, int steps, double*
     t.hist = Hd;
     t.hist_cap = (long long)(steps + 1) * steps;
     t.zero_x = 0;
-    stage_single(h, t, h->blocks);
-    run_solver(h, 1, 1, h->blocks, steps, s);
+    // (this mode runs one CTA per SM, also where solves run the compact variant)
+    const int nb = std::min(h->blocks, h->max_blocks);
+    stage_single(h, t, nb);
+    run_solver(h, 1, 1, nb, steps, s);
     CK(cudaMemcpyAsync(h->hres, h->dres, sizeof(DevResult), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(H_host, Hd, sizeof(double) * (steps + 1) * steps, cudaMemcpyDeviceToHost,
                        s));
