@@ -218,7 +218,9 @@ mlgmres_status mlgmres_solve(mlgmres_t h, const double* b_dev, double* x_dev, vo
  * into groups by mlgmres_batch_plan: a system whose n^(dim+2) cost estimate
  * exceeds the ideal per-CTA share gets a group of several CTAs, the rest of
  * the CTAs form one-CTA groups, and every group works through its list of
- * systems largest first.  b_dev[i], x_dev[i]: device
+ * systems largest first.  (2D FP32 batches whose bases fit in the shared memory of
+ * groups of CTAs are scheduled for that instead, where it is estimated to end
+ * earlier.)  b_dev[i], x_dev[i]: device
  * arrays of grids[i].n^dim doubles; b_dev and x_dev themselves are HOST arrays
  * of device pointers.  Guesses are ZERO (USER when the handle's mode is USER);
  * no pair is collected.  out: `count` results (host); tos_ms of each is the
@@ -395,7 +397,8 @@ typedef struct {
 mlgmres_status mlgmres_autotune(mlgmres_t h, const double* b_dev, int steps, int retune,
                                 void* stream, mlgmres_tuning* out);
 
-/* The batch schedule mlgmres_solve_batch uses, computed on the host only (no
+/* The batch schedule mlgmres_solve_batch uses for a basis streamed from HBM,
+ * computed on the host only (no
  * device work; the paper has no counterpart: it solves one system at a time).
  * Splits `ctas` CTAs into groups and assigns each of the `count` systems of
  * sides n[0..count-1] (dim 2 or 3) to one group.  Cost of a system: N n^2

@@ -989,11 +989,32 @@ mlgmres_status mlgmres_solve_batch(mlgmres_t h, int count, const mlgmres_grid* g
     };
     // one CTA per SM first; if the basis streams from HBM anyway, the compact
     // variant (two CTAs per SM) gets all the reserved CTAs
-    int G = plan_batch(dim, count, sides.data(), std::min(h->batch_groups, h->max_blocks), gctas,
-                       gof, order);
-    const int vsmem = slice_need(gctas, gof);
-    const bool compact = vsmem == 0 && h->batch_compact && h->batch_groups > h->max_blocks;
-    if (compact) G = plan_batch(dim, count, sides.data(), h->batch_groups, gctas, gof, order);
+    const int ctas = std::min(h->batch_groups, h->max_blocks);
+    int G = plan_batch(dim, count, sides.data(), ctas, gctas, gof, order);
+    int vsmem = slice_need(gctas, gof);
+    const bool can_compact = h->batch_compact && h->batch_groups > h->max_blocks;
+    if (vsmem == 0 && can_compact)
+      G = plan_batch(dim, count, sides.data(), h->batch_groups, gctas, gof, order);
+    // FP32 2D: groups large enough to keep every basis in shared memory, where
+    // that is estimated to end earlier (large systems: a step of a streamed basis
+    // waits for its bulk copies on top of the exchanges)
+    if (h->fp32 && dim == 2 && vsmem == 0) {
+      const int max_tiles = gmres_vsmem_budget(true, h->opt.m) / (32 * vrows_p(h->opt.m) * 4);
+      std::vector<int> gc2, gof2, order2;
+      double span = 0.0;
+      const int G2 = max_tiles > 0 ? plan_batch_slices(count, sides.data(), ctas, max_tiles, gc2,
+                                                       gof2, order2, &span)
+                                   : 0;
+      if (G2 > 0 && span < stream_makespan(count, sides.data(), gctas, gof) &&
+          slice_need(gc2, gof2) > 0) {
+        G = G2;
+        gctas = gc2;
+        gof = gof2;
+        order = order2;
+        vsmem = slice_need(gctas, gof);
+      }
+    }
+    const bool compact = vsmem == 0 && can_compact;
     ARG(G >= 1 && G <= h->batch_groups, "batch schedule failed");
     int* gf = h->hcfg;
     int* tf = h->hcfg + (G + 1);

@@ -89,6 +89,127 @@ int plan_batch(int dim, int count, const int* n, int ctas, std::vector<int>& gro
   return (int)group_ctas.size();
 }
 
+// ------------------------------------------------- V slices in shared memory --
+// FP32 2D batches may keep every system's basis in the shared memory of its
+// group's CTAs.  A group then needs at least tiles / max_tiles CTAs for each of its
+// systems, and a step costs (GB300, GMRES(30); us, measured on single systems)
+namespace {
+double slice_step_us(int ctas, int tiles) {
+  const double base = ctas == 1 ? 5.0 : (ctas <= 32 ? 5.5 : 6.0);
+  return base + 0.08 * tiles;
+}
+// ... where a streamed basis costs about (two CTAs per SM)
+double stream_step_us(int ctas, int tiles) {
+  return (ctas == 1 ? 5.0 : 7.0) + 0.25 * tiles;
+}
+int tiles_per_cta(int n, int ctas) {
+  const int tiles = (n * n + 31) / 32;
+  return (tiles + ctas - 1) / ctas;
+}
+}  // namespace
+
+double stream_makespan(int count, const int* n, const std::vector<int>& group_ctas,
+                       const std::vector<int>& group_of) {
+  std::vector<double> load(group_ctas.size(), 0.0);
+  for (int i = 0; i < count; i++) {
+    const int c = group_ctas[group_of[i]];
+    load[group_of[i]] += (double)n[i] * n[i] * stream_step_us(c, tiles_per_cta(n[i], c));
+  }
+  return *std::max_element(load.begin(), load.end());
+}
+
+// For a target makespan every system has a least CTA count (its slices fit, and
+// alone it ends in time); systems in decreasing order of size go to the group of
+// at least that many CTAs where they end earliest within the target, else open a
+// group of exactly that many.  The smallest target that places everything, by
+// bisection; CTAs left over then go to the groups that end last.
+int plan_batch_slices(int count, const int* n, int ctas, int max_tiles,
+                      std::vector<int>& group_ctas, std::vector<int>& group_of,
+                      std::vector<int>& order, double* makespan) {
+  order.resize(count);
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] > n[b]; });
+  auto time = [&](int i, int c) {
+    return (double)n[i] * n[i] * slice_step_us(c, tiles_per_cta(n[i], c));
+  };
+  std::vector<double> load;
+  auto place = [&](double target) {
+    group_ctas.clear();
+    load.clear();
+    group_of.assign(count, -1);
+    int left = ctas;
+    for (int i : order) {
+      const int tiles = (n[i] * n[i] + 31) / 32;
+      int need = (tiles + max_tiles - 1) / max_tiles;
+      while (need <= ctas && time(i, need) > target) need++;
+      if (need > ctas) return false;
+      int best = -1;
+      double best_t = target;
+      for (int g = 0; g < (int)group_ctas.size(); g++) {
+        if (group_ctas[g] < need) continue;
+        const double t = load[g] + time(i, group_ctas[g]);
+        if (t <= best_t) {
+          best_t = t;
+          best = g;
+        }
+      }
+      if (best < 0) {
+        if (need > left) return false;
+        left -= need;
+        group_ctas.push_back(need);
+        load.push_back(0.0);
+        best = (int)group_ctas.size() - 1;
+        best_t = time(i, need);
+      }
+      load[best] = best_t;
+      group_of[i] = best;
+    }
+    return true;
+  };
+  // all systems one after the other on all CTAs always fits (if any plan does)
+  double hi = 0.0, lo = 0.0;
+  for (int i = 0; i < count; i++) {
+    if (tiles_per_cta(n[i], ctas) > max_tiles) return 0;
+    hi += time(i, ctas);
+    lo = std::max(lo, (double)n[i] * n[i] * slice_step_us(2, 1));
+  }
+  hi *= 1.000001;
+  for (int it = 0; it < 24 && hi > 1.002 * lo; it++) {
+    const double mid = 0.5 * (lo + hi);
+    (place(mid) ? hi : lo) = mid;
+  }
+  if (!place(hi)) {  // the whole launch as one group
+    group_ctas.assign(1, ctas);
+    group_of.assign(count, 0);
+  }
+  // the CTAs left over, one at a time, to the group that ends last (as long as
+  // they shorten it)
+  const int G = (int)group_ctas.size();
+  auto group_time = [&](int g, int c) {
+    double t = 0.0;
+    for (int i = 0; i < count; i++)
+      if (group_of[i] == g) t += time(i, c);
+    return t;
+  };
+  load.assign(G, 0.0);
+  int left = ctas;
+  for (int g = 0; g < G; g++) {
+    load[g] = group_time(g, group_ctas[g]);
+    left -= group_ctas[g];
+  }
+  while (left > 0) {
+    const int g = (int)(std::max_element(load.begin(), load.end()) - load.begin());
+    int add = 1;
+    while (add <= left && group_time(g, group_ctas[g] + add) >= load[g]) add++;
+    if (add > left) break;
+    group_ctas[g] += add;
+    left -= add;
+    load[g] = group_time(g, group_ctas[g]);
+  }
+  *makespan = *std::max_element(load.begin(), load.end());
+  return G;
+}
+
 }  // namespace mlg
 
 extern "C" mlgmres_status mlgmres_batch_plan(int dim, int count, const int* n, int ctas,

@@ -14,4 +14,14 @@ double system_cost(int dim, int n);
 int plan_batch(int dim, int count, const int* n, int ctas, std::vector<int>& group_ctas,
                std::vector<int>& group_of, std::vector<int>& order);
 
+// The schedule of a 2D FP32 batch whose bases stay in shared memory: group_ctas[g]
+// CTAs hold slices of at most max_tiles tiles of each of their systems.  Returns
+// the number of groups, 0 if some system does not fit; *makespan in the unit of
+// stream_makespan, which estimates a streamed schedule.
+int plan_batch_slices(int count, const int* n, int ctas, int max_tiles,
+                      std::vector<int>& group_ctas, std::vector<int>& group_of,
+                      std::vector<int>& order, double* makespan);
+double stream_makespan(int count, const int* n, const std::vector<int>& group_ctas,
+                       const std::vector<int>& group_of);
+
 }  // namespace mlg

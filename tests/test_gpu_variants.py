@@ -84,3 +84,18 @@ def test_fp32_exchanges_and_long_slices(n, m, blocks):
     """Group sizes on both sides of the direct exchange's limit, one CTA alone, more
     than 128 CTAs, and slices of one tile up to many points per thread."""
     _solve_2d(n, m=m, precision="fp32_refine", grid_blocks=blocks)
+
+
+@pytest.mark.parametrize("m", [20, 30, 33])
+def test_batch_of_uneven_systems_in_slices(m):
+    """Systems from one tile to 170^2 in one launch (several groups, several systems
+    per group, slices of different lengths), each against the DST solution."""
+    from paper_2103_10975_gb300 import Solver
+    ns = [170, 5, 64, 33, 128, 97, 12, 150, 40, 81, 1, 111]
+    bs = [MovingGaussians2D(n, 900 + i, 50).rhs(i) for i, n in enumerate(ns)]
+    s = Solver(max(ns), m=m, rtol=1e-10, precision="fp32_refine", batch_slots=4096)
+    xs, res = s.solve_batch(ns, [torch.as_tensor(b).cuda() for b in bs])
+    for n, b, x, r in zip(ns, bs, xs, res):
+        assert r["status"] == 0 and r["relres_true"] <= 1e-10, (n, r)
+        xe = direct.dst_solve_2d(n, b)
+        assert np.linalg.norm(x.cpu().numpy() - xe) <= 1e-7 * np.linalg.norm(xe), n
