@@ -34,9 +34,9 @@ struct mlgmres {
   float* faces = nullptr;    // FP32 face coefficients (single 3D FP32 solves with kappa)
   long long fstride = 0;     // their array stride
   double* faces64 = nullptr; // FP64 face coefficients (single 3D solves with kappa), stride ldv
-  void* Wt = nullptr;        // w' with tags, if a single solve may run a shared-slice variant
+  void* Wt = nullptr;        // w' with tags, if a single solve may run a shared-slice variant (in W1's allocation)
   double* part = nullptr;
-  uint4* words = nullptr;    // tagged partial sums (single solves)
+  uint4* words = nullptr;    // tagged partial sums (single solves; in part's allocation)
   double* Rg = nullptr;      // compact variants' triangles R (rg_blocks of them)
   int rg_blocks = 0;
   unsigned long long* bar = nullptr;  // per group: counter

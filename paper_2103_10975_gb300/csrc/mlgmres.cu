@@ -64,9 +64,8 @@ unsigned long long splitmix_next(unsigned long long& st) {
 // FP32 2D slices of V of more points than this are long (kVSharedL: two points per
 // trip of the passes).  Measured, one point per trip / two: single systems 430^2 (1217
 // points) 9.4 / 10.1 us per step, 512^2 (1725) 10.96 / 11.07, 600^2 (2369; GMRES(20))
-// 12.9 / 12.2; batches of 40 of 24^2 -
-// 160^2 37.1 / 36.1 ms, 48 of 60^2 - 170^2 (GMRES(20)) 116 / 102, 12 of 40^2 - 100^2
-// (largest: 534 points) 11.43 / 11.79.
+// 12.9 / 12.2; batches of 40 of 24^2 - 160^2 37.1 / 36.1 ms, 48 of 60^2 - 170^2
+// (GMRES(20)) 116 / 102, 12 of 40^2 - 100^2 (largest: 534 points) 11.43 / 11.79.
 constexpr int kLongPoints = 2048, kLongPointsBatch = 1024;
 
 // Shared-memory bytes a CTA has for its slice of V.  (3D FP32: what the variant for
@@ -703,14 +702,17 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
     }
     if (grid->dim == 3 && grid->kappa_dev)
       CK(cudaMalloc(&h->faces64, sizeof(double) * 3 * (size_t)h->ldv));
-    CK(cudaMalloc(&h->W1, es * (size_t)h->ldv));
-    CK(cudaMalloc(&h->part, sizeof(double) * part_doubles(kPartStride)));
-    CK(cudaMalloc(&h->words, sizeof(uint4) * tag_words(kPartStride)));
-    // w' with tags, where some CTA count lets the slices of V fit
-    if (single_vsmem(h, h->max_blocks) > 0 ||
+    // (two areas per allocation: one costs about 0.1 ms)
+    // z, and w' with tags where some CTA count lets the slices of V fit
+    const bool slices =
+        single_vsmem(h, h->max_blocks) > 0 ||
         (gmres_compact_ok(h->fp32, grid->dim, opt->m) &&
-         single_vsmem(h, std::max(1, gmres_compact_max_blocks(grid->dim, opt->m)), true) > 0))
-      CK(cudaMalloc(&h->Wt, 2 * es * (size_t)h->ldv));
+         single_vsmem(h, std::max(1, gmres_compact_max_blocks(grid->dim, opt->m)), true) > 0);
+    CK(cudaMalloc(&h->W1, (slices ? 3 : 1) * es * (size_t)h->ldv));
+    if (slices) h->Wt = (char*)h->W1 + es * (size_t)h->ldv;
+    CK(cudaMalloc(&h->part, sizeof(double) * part_doubles(kPartStride) +
+                                sizeof(uint4) * tag_words(kPartStride)));
+    h->words = (uint4*)(h->part + part_doubles(kPartStride));
     if (opt->compact != 0 && gmres_compact_ok(h->fp32, grid->dim, opt->m)) {
       // the compact variants keep each CTA's triangle R in HBM (L2-resident),
       // which leaves room for a second bulk-copy stage per warp
@@ -732,8 +734,9 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
       const size_t G = (size_t)h->batch_groups;
       CK(cudaMalloc(&h->Vb, es * G * (size_t)vrows_p(opt->m + 1) * h->ldv));
       CK(cudaMalloc(&h->Wb, es * G * 4 * (size_t)h->ldv));
-      CK(cudaMalloc(&h->partb, sizeof(double) * G * part_doubles(1)));
-      CK(cudaMalloc(&h->wordsb, sizeof(uint4) * G * tag_words(1)));
+      CK(cudaMalloc(&h->partb,
+                    G * (sizeof(double) * part_doubles(1) + sizeof(uint4) * tag_words(1))));
+      h->wordsb = (uint4*)(h->partb + G * part_doubles(1));
     }
     CK(cudaMalloc(&h->bar, sizeof(unsigned long long) * h->group_cap));
     CK(cudaMalloc(&h->err, sizeof(int) * h->group_cap));
@@ -786,9 +789,6 @@ void mlgmres_destroy(mlgmres_t h) {
   cudaFree(h->Vb);
   cudaFree(h->Wb);
   cudaFree(h->partb);
-  cudaFree(h->wordsb);
-  cudaFree(h->Wt);
-  cudaFree(h->words);
   cudaFree(h->V);
   cudaFree(h->W0_alloc);
   if (h->faces) cudaFree(h->faces - (h->fstride - h->ldv) / 2);

@@ -99,3 +99,10 @@ def test_batch_of_uneven_systems_in_slices(m):
         assert r["status"] == 0 and r["relres_true"] <= 1e-10, (n, r)
         xe = direct.dst_solve_2d(n, b)
         assert np.linalg.norm(x.cpu().numpy() - xe) <= 1e-7 * np.linalg.norm(xe), n
+
+
+@pytest.mark.parametrize("n,m", [(632, 20), (633, 30), (700, 47), (640, 48)])
+def test_untuned_large_bases(n, m):
+    """The untuned default for streamed 2D FP32 bases on both sides of its size and m
+    limits."""
+    _solve_2d(n, m=m, precision="fp32_refine")
