@@ -389,8 +389,10 @@ typedef struct {
  * basis held in HBM, 0/2/4/8/16 bulk-copy stages, and for FP32 grids the compact
  * variants at one and two CTAs per SM -- and keeps the fastest per
  * step for this handle's later solves (options grid_blocks and v_stages set
- * explicitly at create still win).  Results are cached per process by
- * (device, dim, n, m, precision); a cached shape is reused without timing
+ * explicitly at create still win).  A handle whose learned guesses train beside the
+ * solves (overlap_train) prefers shapes that leave an eighth of the SMs free unless
+ * another is 3% faster.  Results are cached per process by
+ * (device, dim, n, m, precision, that preference); a cached shape is reused without timing
  * unless `retune` is 1.  Writes into an internal scratch vector (allocated
  * here and freed before returning), records no (b, x) pair, synchronises
  * `stream`.  out may be NULL.  ERR_ARG on a NULL handle or b_dev, steps < 0. */
