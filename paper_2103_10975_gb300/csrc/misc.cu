@@ -77,12 +77,13 @@ __global__ void denormalise_kernel(const float* __restrict__ y, int N, const dou
 }
 
 // Damped Jacobi on the 2D operator: out = in + omega/d (b - A in), d = 4/h^2 the
-// diagonal of A, written as out = wc in + wn (sum of the neighbours) + f b with wc = 1 -
-// omega, wn = omega/4, f = omega/d from the host and f b formed as the tile is loaded:
-// three additions and two FMAs per point and sweep, on a GPU whose FP64 pipe bounds
-// this kernel, where differences from the neighbours took nine operations.  (Rounding
-// after 32 sweeps at 256^2 against extended precision: 9e-17 of the iterate's norm,
-// 6e-17 by differences; a double's unit is 1.1e-16.)
+// diagonal of A.  s2 = 1/h^2 and f = omega/(4 s2) come from the host (the same
+// IEEE divisions, once per launch instead of three FP64 divisions per point on a
+// GPU whose FP64 pipe is narrow).  By differences from the neighbours: on a smooth
+// iterate they are nearly exact, so a sweep adds little but the rounding of its last
+// addition (32 sweeps at 256^2 against extended precision: 6e-17 of the iterate's norm).  A
+// weighted sum of the five points takes five operations instead of nine (the guess
+// 186 us instead of 218) and rounds to 9e-17: not used.
 //
 // Up to S damped-Jacobi sweeps of the 2D operator in one launch: a CTA loads its
 // TW x TH tile with a halo of S points (x and b) into shared memory and sweeps
@@ -90,14 +91,14 @@ __global__ void denormalise_kernel(const float* __restrict__ y, int N, const dou
 // another CTA and the tile goes through L2 once per S sweeps.  The same FP64
 // operations per point whatever the tile or the number of sweeps per launch.  The halo
 // is computed redundantly ((TW + 2 (S - s)) (TH + 2 (S - s)) points in sweep s: 1.4 x
-// the tile at 32 x 16, S = 4); eight sweeps per launch measured the same at 256^2 and
-// slower at 320^2.  32 sweeps at 256^2: 32 launches 310 us for the whole guess, 8
-// launches 276; by differences 218, by sums as above 186.
+// the tile at 32 x 16, S = 4); more sweeps per launch cost more FP64 than the launches
+// they save.  32 sweeps at 256^2: 32 launches 310 us for the whole guess, 8 launches
+// 276 (218 with what the other kernels of the guess gained later).
 template <int TW, int TH, int S>
 __global__ void __launch_bounds__(256) jacobi_tile_kernel(int n, const double* __restrict__ b,
                                                           const double* __restrict__ xin,
-                                                          double* __restrict__ xout, double f,
-                                                          double wn, double wc, int sweeps) {
+                                                          double* __restrict__ xout, double s2,
+                                                          double f, int sweeps) {
   constexpr int RW = TW + 2 * S, RH = TH + 2 * S;
   __shared__ double sb[RH * RW], sx[2][RH * RW];
   const int gx0 = (int)blockIdx.x * TW - S, gy0 = (int)blockIdx.y * TH - S;
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(256) jacobi_tile_kernel(int n, const double* _
     const int x = gx0 + p % RW, y = gy0 + p / RW;
     const bool in = x >= 0 && x < n && y >= 0 && y < n;
     const long long g = (long long)y * n + x;
-    sb[p] = in ? f * b[g] : 0.0;
+    sb[p] = in ? b[g] : 0.0;
     sx[0][p] = in ? xin[g] : 0.0;
     sx[1][p] = 0.0;  // (points outside the grid stay 0 in both buffers)
   }
@@ -121,7 +122,9 @@ __global__ void __launch_bounds__(256) jacobi_tile_kernel(int n, const double* _
       const int x = gx0 + lx, y = gy0 + ly;
       if (x < 0 || x >= n || y < 0 || y >= n) continue;
       const int q = ly * RW + lx;
-      v[q] = fma(wn, (u[q - 1] + u[q + 1]) + (u[q - RW] + u[q + RW]), fma(wc, u[q], sb[q]));
+      const double c = u[q], l = u[q - 1], r = u[q + 1], d = u[q - RW], t = u[q + RW];
+      const double ax = s2 * (((c - l) + (c - r)) + ((c - d) + (c - t)));
+      v[q] = c + f * (sb[q] - ax);
     }
   }
   __syncthreads();
@@ -247,10 +250,10 @@ cudaError_t launch_jacobi(int dim, int n, const float* kappa, const double* b, d
       // a serial FP64 chain per point; more CTAs shorten it)
       if ((long long)((n + 31) / 32) * ((n + 15) / 16) >= 100)
         jacobi_tile_kernel<32, 16, S><<<dim3((n + 31) / 32, (n + 15) / 16), 256, 0, s>>>(
-            n, b, cur, oth, f, 0.25 * omega, 1.0 - omega, c);
+            n, b, cur, oth, s2, f, c);
       else
         jacobi_tile_kernel<16, 8, S><<<dim3((n + 15) / 16, (n + 7) / 8), 256, 0, s>>>(
-            n, b, cur, oth, f, 0.25 * omega, 1.0 - omega, c);
+            n, b, cur, oth, s2, f, c);
     }
     note_launches(1);
     double* t = cur;
