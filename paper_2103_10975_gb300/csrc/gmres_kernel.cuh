@@ -2418,17 +2418,10 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
       // c_{j+1} = Hu(j+1,j) h2_j, the new vector's own coefficient
       auto set_norm = [&]() {
         const T h2v = sm.hn2T > T(0) ? sm.hn2T : T(0);
-        T hnT;
-        if (sizeof(T) == 8 && h2v > T(1e-290) && h2v < T(1e290)) {
-          // FP64: one reciprocal square root instead of a square root and a
-          // division (dependent chains of ~680 and ~430 cycles on this GPU)
-          const T inv = rsqrt(h2v);
-          hnT = h2v * inv;
-          sm.invT = inv;
-        } else {
-          hnT = sqrt(h2v);
-          sm.invT = T(1) / hnT;
-        }
+        // (correctly rounded in FP64 too: h2 rsqrt(h2) saves a dependent chain of ~500
+        // cycles but is off by a unit in the last place on a quarter of the values)
+        const T hnT = sqrt(h2v);
+        sm.invT = T(1) / hnT;
         sm.HuT[j + 1 + j * LD] = hnT;  // (the Givens warp reads it in FP64)
         sm.cv[j + 1] = hnT * sm.coef[j];
       };
@@ -2463,8 +2456,8 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
         if constexpr (sizeof(T) == 8) {
           // FP64: only the products that exist (a warp FMA occupies its SM
           // quarter's pipe for 64 cycles), column j's by the row's first lane.
-          // With the gather's tests, the norm's rsqrt and the m <= 32 variant:
-          // 28.5 -> 26.8 us per step at 256^2, GMRES(30)
+          // With the gather's tests and the m <= 32 variant: 28.5 -> 26.8 us per
+          // step at 256^2, GMRES(30) (with a reciprocal square root in the norm)
           if (i <= j) {
             if (sub == 0) c = (sm.h1c[i] + sm.coef[i]) * sm.coef[j];
             for (int k = k0; k < j; k += 8) c = fma(sm.HuT[i + k * LD], sm.coef[k], c);

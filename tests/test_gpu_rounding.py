@@ -47,3 +47,19 @@ def test_smooth_rounds_no_worse_than_differences(n, sweeps):
         return np.linalg.norm((v - ref).astype(np.float64)) / np.linalg.norm(ref.astype(np.float64))
 
     assert err(xd.cpu().numpy()) <= 1.15 * err(plain), (err(xd.cpu().numpy()), err(plain))
+
+
+@pytest.mark.parametrize("at", ["corner", "edge"])
+def test_fp64_norm_is_the_rounded_root(at):
+    """The first subdiagonal entry of the Hessenberg matrix from a unit vector at a corner
+    (or edge) point: A e leaves -1/h^2 at its 2 (3) neighbours, every sum on the way is
+    exact or rounded once, so ||w|| is the correctly rounded root of 2 (3) / h^4."""
+    from paper_2103_10975_gb300 import Solver
+    for n in range(3, 17):
+        h = 2.0 / (n + 1)
+        s2 = 1.0 / (h * h)
+        a = s2 * s2
+        e = torch.zeros(n * n, dtype=torch.float64)
+        e[0 if at == "corner" else 1] = 1.0
+        _, H, _ = Solver(n, m=4).arnoldi(e.cuda(), 2)
+        assert H[1, 0] == np.sqrt(2.0 * a if at == "corner" else 2.0 * a + a), n
