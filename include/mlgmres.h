@@ -392,8 +392,9 @@ typedef struct {
  * explicitly at create still win).  A handle whose learned guesses train beside the
  * solves (overlap_train) prefers shapes that leave an eighth of the SMs free unless
  * another is 3% faster.  Results are cached per process by
- * (device, dim, n, m, precision, that preference); a cached shape is reused without timing
- * unless `retune` is 1.  Writes into an internal scratch vector (allocated
+ * (device, dim, n, m, precision, whether there is a kappa, options grid_blocks, v_stages
+ * and compact, that preference); a cached shape is reused without timing unless `retune`
+ * is 1.  Writes into an internal scratch vector (allocated
  * here and freed before returning), records no (b, x) pair, synchronises
  * `stream`.  out may be NULL.  ERR_ARG on a NULL handle or b_dev, steps < 0. */
 mlgmres_status mlgmres_autotune(mlgmres_t h, const double* b_dev, int steps, int retune,

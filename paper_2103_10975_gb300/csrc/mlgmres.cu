@@ -1115,11 +1115,14 @@ mlgmres_status mlgmres_train_step(mlgmres_t h, void* side_stream, float* loss_ho
 }
 
 namespace {
+// Everything the candidates depend on: a shape found under other options (two CTAs per
+// SM, say) may be one that this handle cannot launch.
 struct TuneKey {
-  int dev, dim, n, m, fp32, beside;
+  int dev, dim, n, m, fp32, kappa, grid_blocks, v_stages, compact, beside;
   bool operator<(const TuneKey& o) const {
-    return std::tie(dev, dim, n, m, fp32, beside) <
-           std::tie(o.dev, o.dim, o.n, o.m, o.fp32, o.beside);
+    return std::tie(dev, dim, n, m, fp32, kappa, grid_blocks, v_stages, compact, beside) <
+           std::tie(o.dev, o.dim, o.n, o.m, o.fp32, o.kappa, o.grid_blocks, o.v_stages,
+                    o.compact, o.beside);
   }
 };
 struct TuneVal {
@@ -1141,7 +1144,8 @@ mlgmres_status mlgmres_autotune(mlgmres_t h, const double* b, int steps, int ret
     cudaStream_t s = (cudaStream_t)stream;
     if (steps == 0) steps = 2 * h->opt.m;
     const TuneKey key{h->dev, h->grid.dim, h->grid.n, h->opt.m, h->fp32 ? 1 : 0,
-                      trains_beside(h) ? 1 : 0};
+                      h->grid.kappa_dev ? 1 : 0, h->opt.grid_blocks, h->opt.v_stages,
+                      h->opt.compact, trains_beside(h) ? 1 : 0};
     mlgmres_tuning t;
     memset(&t, 0, sizeof(t));
     auto apply = [&](int blocks, int stages, int compact) {
