@@ -22,9 +22,8 @@ constexpr size_t kStaticBasis = sizeof(float) * (size_t)vrows_p(kStaticMaxM + 1)
 constexpr size_t kStaticWork = 2 * sizeof(float) * (size_t)kStaticLdv;
 constexpr int kStaticStride = kStaticMaxN / 512;  // one CTA per 512 points
 constexpr size_t kStaticPart = sizeof(double) * part_doubles(kStaticStride);
-constexpr size_t kStaticWords = sizeof(uint4) * tag_words(kStaticStride);
 constexpr size_t kStaticMisc = 4096;  // barrier counter, error flag, result, launch tables
-constexpr size_t kStaticBytes = kStaticBasis + kStaticWork + kStaticPart + kStaticWords + kStaticMisc;
+constexpr size_t kStaticBytes = kStaticBasis + kStaticWork + kStaticPart + kStaticMisc;
 
 // The fixed workspace.  In host code this name is only a stand-in for the
 // symbol; the device address comes from cudaGetSymbolAddress.
@@ -80,8 +79,6 @@ extern "C" mlgmres_status mlgmres_solve_static(int n, int m, double rtol, long l
   p += kStaticWork;
   double* part = (double*)p;
   p += kStaticPart;
-  uint4* words = (uint4*)p;
-  p += kStaticWords;
   unsigned long long* bar = (unsigned long long*)p;
   int* err = (int*)(p + 8);
   DevResult* dres = (DevResult*)(p + 64);
@@ -114,9 +111,9 @@ extern "C" mlgmres_status mlgmres_solve_static(int n, int m, double rtol, long l
   w.ldv = kStaticLdv;
   w.W0 = W0;
   w.W1 = W1;
-  w.Wt = nullptr;
+  w.Wt = nullptr;     // (w' with tags and tagged sums: shared-slice variants only)
   w.part = part;
-  w.words = words;
+  w.words = nullptr;
   w.pstride = kStaticStride;
   w.Rg = nullptr;
   w.bar.ctr = bar;
