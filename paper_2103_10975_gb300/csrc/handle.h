@@ -55,7 +55,8 @@ struct mlgmres {
   int batch_groups = 0;
   bool batch_compact = false;         // batches may launch the compact variant
   void* Vb = nullptr;
-  void* Wb = nullptr;                 // work vectors per group: W0, W1, Wt (4 ldv elements)
+  void* Wb = nullptr;                 // work vectors per group: W1, then W0 and Wt in one place
+  int batch_wvecs = 0;                // elements per point of Wb and group
   double* partb = nullptr;
   uint4* wordsb = nullptr;
 

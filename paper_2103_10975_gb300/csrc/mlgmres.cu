@@ -742,7 +742,10 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
       h->cfg_cap = kBatchCap;
       const size_t G = (size_t)h->batch_groups;
       CK(cudaMalloc(&h->Vb, es * G * (size_t)vrows_p(opt->m + 1) * h->ldv));
-      CK(cudaMalloc(&h->Wb, es * G * 4 * (size_t)h->ldv));
+      // w' and z; in the FP32 2D variants w' with tags takes two elements a point (the
+      // streamed variants' w' is the first half of the same area)
+      h->batch_wvecs = h->fp32 && grid->dim == 2 ? 3 : 2;
+      CK(cudaMalloc(&h->Wb, es * G * h->batch_wvecs * (size_t)h->ldv));
       CK(cudaMalloc(&h->partb,
                     G * (sizeof(double) * part_doubles(1) + sizeof(uint4) * tag_words(1))));
       h->wordsb = (uint4*)(h->partb + G * part_doubles(1));
@@ -1059,9 +1062,8 @@ mlgmres_status mlgmres_solve_batch(mlgmres_t h, int count, const mlgmres_grid* g
       GroupWork w;
       w.V = (char*)h->Vb + es * (size_t)g * vrows_p(h->opt.m + 1) * h->ldv;
       w.ldv = h->ldv;
-      w.W0 = (char*)h->Wb + es * (size_t)g * 4 * h->ldv;
-      w.W1 = (char*)w.W0 + es * h->ldv;
-      w.Wt = (char*)w.W1 + es * h->ldv;
+      w.W1 = (char*)h->Wb + es * (size_t)g * h->batch_wvecs * h->ldv;
+      w.W0 = w.Wt = (char*)w.W1 + es * h->ldv;  // (a launch uses one of the two)
       w.part = h->partb + part_off;
       part_off += part_doubles(gctas[g]);
       w.words = h->wordsb + word_off;

@@ -89,7 +89,8 @@ struct GroupWork {
   long long ldv;
   void* W0;           // two work vectors (ping-pong), ldv each
   void* W1;
-  void* Wt;           // w' with tags (shared-slice variants), ldv words of 2 elements
+  void* Wt;           // w' of the shared-slice variants: FP32 with tags (2 ldv elements), FP64
+                      // plain (ldv); they do not use W0, which may be the same place
   double* part;       // 2 x (kMaxM+2) x pstride partial sums
   uint4* words;       // tag_words(pstride): the tagged partial sums of the exchanges
   int pstride;        // row length of part and words (>= the group's CTA count)
