@@ -263,7 +263,7 @@ __host__ __device__ constexpr size_t smem_own_bytes() {
 }
 
 // Warp partial of slot k (lane 0 stores it); block_finish then adds the warp
-// partials of slots 0..L-1 and writes the CTA's sums to part[k*kPartStride + lb].
+// partials of slots 0..L-1 and writes the CTA's sums to part[k * ps + lb].
 // All of it runs in the element type R (FP32 for the FP32 variant: the FP64
 // pipe of this GPU is ~1/64 of FP32 and would otherwise dominate).
 template <int LW, typename R, typename V>

@@ -36,6 +36,7 @@ struct mlgmres {
   double* faces64 = nullptr; // FP64 face coefficients (single 3D solves with kappa), stride ldv
   void* Wt = nullptr;        // w' with tags, if a single solve may run a shared-slice variant (in W1's allocation)
   double* part = nullptr;
+  int pstride = 0;           // row length of part and words
   uint4* words = nullptr;    // tagged partial sums (single solves; in part's allocation)
   double* Rg = nullptr;      // compact variants' triangles R (rg_blocks of them)
   int rg_blocks = 0;

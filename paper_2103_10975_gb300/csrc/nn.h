@@ -89,6 +89,7 @@ struct Net {
   long long lvl_off[kMaxLevels];             // offsets of level l inside g_pool (per sample)
   // transposed linear upsampling n -> side[l], per axis, as sparse rows:
   // coarse j takes sum over k in [up_ptr[j], up_ptr[j+1]) of up_w[k] * fine[up_idx[k]]
+  void* up_mem = nullptr;                    // holds these tables, for every level
   int* up_ptr[kMaxLevels] = {};
   int* up_idx[kMaxLevels] = {};
   float* up_w[kMaxLevels] = {};

@@ -22,7 +22,7 @@ constexpr int kVSharedL = 3; // kVShared for long slices (FP32 2D)
 __host__ __device__ constexpr bool in_shared(int vmode) {
   return vmode == kVShared || vmode == kVSharedL;
 }
-constexpr int kPartStride = 1024;  // max CTAs per group (partials row length)
+constexpr int kPartStride = 1024;  // max CTAs per group
 // doubles in a group's partial-sum area (two alternating sets)
 constexpr long long part_doubles(int pstride) { return 2LL * (kMaxM + 2) * pstride; }
 // 16-byte words of a group's tagged partial sums: three slots each, two
