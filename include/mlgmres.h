@@ -400,9 +400,9 @@ typedef struct {
 mlgmres_status mlgmres_autotune(mlgmres_t h, const double* b_dev, int steps, int retune,
                                 void* stream, mlgmres_tuning* out);
 
-/* The batch schedule mlgmres_solve_batch uses for a basis streamed from HBM,
- * computed on the host only (no
- * device work; the paper has no counterpart: it solves one system at a time).
+/* The batch schedule mlgmres_solve_batch uses (2D FP32 batches may prefer the one of
+ * mlgmres_batch_plan_slices), computed on the host only (no device work; the paper has
+ * no counterpart: it solves one system at a time).
  * Splits `ctas` CTAs into groups and assigns each of the `count` systems of
  * sides n[0..count-1] (dim 2 or 3) to one group.  Cost of a system: N n^2
  * (Arnoldi steps grow like n^2, each moves O(N) values).  Systems whose cost
@@ -416,6 +416,20 @@ mlgmres_status mlgmres_autotune(mlgmres_t h, const double* b_dev, int steps, int
  * a side < 1 or a NULL pointer. */
 mlgmres_status mlgmres_batch_plan(int dim, int count, const int* n, int ctas, int* groups,
                                   int* group_ctas, int* group_of);
+
+/* The other schedule mlgmres_solve_batch has for 2D FP32 batches, likewise on the host:
+ * groups of CTAs large enough to keep the GMRES(m) basis of each of their systems in
+ * shared memory, at most max_tiles tiles of 32 points per CTA (what the shared memory
+ * left by the kernel holds: 213 KB / (128 m), m rounded up to even, for m <= 32).  It is
+ * used where mlgmres_batch_plan's schedule on `ctas` CTAs does not fit in shared memory
+ * and this one is estimated (from m, rtol and max_iters) to end at least 5% before
+ * mlgmres_batch_plan's on `stream_ctas` CTAs with streamed bases: *preferred = 1.  *groups = 0 if some system
+ * does not fit at all.  Outputs and errors otherwise as mlgmres_batch_plan; sides are at
+ * most 32768. */
+mlgmres_status mlgmres_batch_plan_slices(int count, const int* n, int m, double rtol,
+                                         long long max_iters, int ctas, int stream_ctas,
+                                         int max_tiles, int* groups, int* group_ctas,
+                                         int* group_of, int* preferred);
 
 #ifdef __cplusplus
 }

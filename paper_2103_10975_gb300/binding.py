@@ -153,6 +153,10 @@ _SIGS = {
                                           ctypes.c_int, ctypes.POINTER(ctypes.c_int),
                                           ctypes.POINTER(ctypes.c_int),
                                           ctypes.POINTER(ctypes.c_int)]),
+    "mlgmres_batch_plan_slices": (ctypes.c_int, [ctypes.c_int, ctypes.POINTER(ctypes.c_int),
+                                                 ctypes.c_int, ctypes.c_double,
+                                                 ctypes.c_longlong] +
+                                  [ctypes.c_int] * 3 + [ctypes.POINTER(ctypes.c_int)] * 4),
 }
 
 _lib = None
@@ -210,8 +214,9 @@ def solve_static(n, b, x, m=30, rtol=1e-10, max_iters=10 ** 7, stream=None):
 
 
 def batch_plan(dim, sides, ctas):
-    """mlgmres_batch_plan: the CTA groups a batched launch would use (host
-    only).  Returns (group_ctas list, group_of list)."""
+    """mlgmres_batch_plan: the CTA groups of a batched launch with streamed bases, or whose
+    slices of the bases fit in shared memory with these groups as well (host only).
+    Returns (group_ctas list, group_of list)."""
     count = len(sides)
     n = (ctypes.c_int * count)(*[int(v) for v in sides])
     G = ctypes.c_int(0)
@@ -221,6 +226,23 @@ def batch_plan(dim, sides, ctas):
     if st != MLGMRES_OK:
         raise MLGMRESError(st, "batch_plan: invalid arguments")
     return list(gc[:G.value]), list(go)
+
+
+def batch_plan_slices(sides, m, ctas, stream_ctas, max_tiles, rtol=1e-10, max_iters=10 ** 7):
+    """mlgmres_batch_plan_slices: the CTA groups of a 2D FP32 batch whose bases stay in
+    shared memory (host only).  Returns (group_ctas list, group_of list, preferred); empty
+    lists if some system does not fit."""
+    count = len(sides)
+    n = (ctypes.c_int * count)(*[int(v) for v in sides])
+    G, use = ctypes.c_int(0), ctypes.c_int(0)
+    gc = (ctypes.c_int * max(1, int(ctas)))()
+    go = (ctypes.c_int * count)()
+    st = load_library().mlgmres_batch_plan_slices(count, n, int(m), float(rtol), int(max_iters),
+                                                  int(ctas), int(stream_ctas), int(max_tiles),
+                                                  ctypes.byref(G), gc, go, ctypes.byref(use))
+    if st != MLGMRES_OK:
+        raise MLGMRESError(st, "batch_plan_slices: invalid arguments")
+    return list(gc[:G.value]), list(go) if G.value else [], bool(use.value)
 
 
 class MLGMRESError(RuntimeError):

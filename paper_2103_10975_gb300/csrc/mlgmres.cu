@@ -1020,10 +1020,12 @@ mlgmres_status mlgmres_solve_batch(mlgmres_t h, int count, const mlgmres_grid* g
       const int max_tiles = gmres_vsmem_budget(true, h->opt.m) / (32 * vrows_p(h->opt.m) * 4);
       std::vector<int> gc2, gof2, order2;
       double span = 0.0;
-      const int G2 = max_tiles > 0 ? plan_batch_slices(count, sides.data(), ctas, max_tiles, gc2,
-                                                       gof2, order2, &span)
+      const SolveKind kind{h->opt.m, h->opt.rtol, h->opt.max_iters};
+      const int G2 = max_tiles > 0 ? plan_batch_slices(count, sides.data(), kind, ctas, max_tiles,
+                                                       gc2, gof2, order2, &span)
                                    : 0;
-      if (G2 > 0 && span < stream_makespan(count, sides.data(), gctas, gof) &&
+      if (G2 > 0 &&
+          slices_pay(span, stream_makespan(count, sides.data(), kind, ctas, gctas, gof)) &&
           slice_need(gc2, gof2) > 0) {
         G = G2;
         gctas = gc2;

@@ -92,15 +92,30 @@ int plan_batch(int dim, int count, const int* n, int ctas, std::vector<int>& gro
 // ------------------------------------------------- V slices in shared memory --
 // FP32 2D batches may keep every system's basis in the shared memory of its
 // group's CTAs.  A group then needs at least tiles / max_tiles CTAs for each of its
-// systems, and a step costs (GB300, GMRES(30); us, measured on single systems)
+// systems.  Whether that ends earlier than streaming the bases is estimated from a
+// system's steps and from what a step takes; measured on GB300 (batches of equal
+// systems, m = 5 .. 64, groups of 1 to 152 CTAs, 2 to 320 tiles per CTA): the formulas
+// are within 5% rms of 1 131 and 1 590 timings, 23% at worst.  (Formulas of m = 30 alone,
+// with n^2 for the steps, chose slices for batches of many small systems, or of m >= 40,
+// that took up to twice as long with them.)
 namespace {
-double slice_step_us(int ctas, int tiles) {
-  const double base = ctas == 1 ? 5.0 : (ctas <= 32 ? 5.5 : 6.0);
-  return base + 0.08 * tiles;
+// Arnoldi steps of GMRES(m) from x0 = 0: about n until the basis is full, then as n^2
+// (3 200 solves of n = 5 .. 320, m = 3 .. 64, rtol 1e-4 .. 1e-12: 6-11% rms at one rtol).
+double system_steps(int n, const SolveKind& k) {
+  const double digits = std::max(2.0, -log10(k.rtol));
+  return std::min((double)k.max_iters, (0.44 * digits - 0.35) * n * (1.0 + (double)n / k.m));
 }
-// ... where a streamed basis costs about (two CTAs per SM)
-double stream_step_us(int ctas, int tiles) {
-  return (ctas == 1 ? 5.0 : 7.0) + 0.25 * tiles;
+// us per step with slices: exchanges (few CTAs exchange directly), scalar work by m,
+// the passes, and the restart's share
+double slice_step_us(int m, int ctas, int tiles) {
+  return 2.2 + (ctas > 1 ? 0.9 : 0.0) + (ctas > 12 ? 0.6 : 0.0) + 0.066 * m +
+         (0.071 + 0.0004 * m) * tiles + 23.0 / m;
+}
+// ... and with a streamed basis, all SMs' CTAs sharing L2 and HBM; two_per_sm: more than
+// one CTA per SM at work
+double stream_step_us(int m, int ctas, int tiles, bool two_per_sm) {
+  return 6.2 + (ctas > 1 ? 1.4 : 0.0) +
+         (two_per_sm ? 0.16 + 0.0024 * m : 0.11 + 0.0018 * m) * tiles + 17.0 / m;
 }
 int tiles_per_cta(int n, int ctas) {
   const int tiles = (n * n + 31) / 32;
@@ -108,29 +123,37 @@ int tiles_per_cta(int n, int ctas) {
 }
 }  // namespace
 
-double stream_makespan(int count, const int* n, const std::vector<int>& group_ctas,
-                       const std::vector<int>& group_of) {
+double stream_makespan(int count, const int* n, const SolveKind& k, int sms,
+                       const std::vector<int>& group_ctas, const std::vector<int>& group_of) {
   std::vector<double> load(group_ctas.size(), 0.0);
+  const bool two = std::accumulate(group_ctas.begin(), group_ctas.end(), 0) > sms;
   for (int i = 0; i < count; i++) {
     const int c = group_ctas[group_of[i]];
-    load[group_of[i]] += (double)n[i] * n[i] * stream_step_us(c, tiles_per_cta(n[i], c));
+    load[group_of[i]] +=
+        system_steps(n[i], k) * stream_step_us(k.m, c, tiles_per_cta(n[i], c), two);
   }
   return *std::max_element(load.begin(), load.end());
 }
+
+// (Timed on 150 mixed batches of 2 to 400 systems, sides 8 to 251, m = 3 to 64: where the
+// ratio of the estimates lay between 0.9 and 1.05, that of the times was within 6% of it.)
+bool slices_pay(double slices, double stream) { return slices < 0.95 * stream; }
 
 // For a target makespan every system has a least CTA count (its slices fit, and
 // alone it ends in time); systems in decreasing order of size go to the group of
 // at least that many CTAs where they end earliest within the target, else open a
 // group of exactly that many.  The smallest target that places everything, by
 // bisection; CTAs left over then go to the groups that end last.
-int plan_batch_slices(int count, const int* n, int ctas, int max_tiles,
+int plan_batch_slices(int count, const int* n, const SolveKind& k, int ctas, int max_tiles,
                       std::vector<int>& group_ctas, std::vector<int>& group_of,
                       std::vector<int>& order, double* makespan) {
   order.resize(count);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] > n[b]; });
+  std::vector<double> steps(count);
+  for (int i = 0; i < count; i++) steps[i] = system_steps(n[i], k);
   auto time = [&](int i, int c) {
-    return (double)n[i] * n[i] * slice_step_us(c, tiles_per_cta(n[i], c));
+    return steps[i] * slice_step_us(k.m, c, tiles_per_cta(n[i], c));
   };
   std::vector<double> load;
   auto place = [&](double target) {
@@ -171,7 +194,7 @@ int plan_batch_slices(int count, const int* n, int ctas, int max_tiles,
   for (int i = 0; i < count; i++) {
     if (tiles_per_cta(n[i], ctas) > max_tiles) return 0;
     hi += time(i, ctas);
-    lo = std::max(lo, (double)n[i] * n[i] * slice_step_us(2, 1));
+    lo = std::max(lo, steps[i] * slice_step_us(k.m, 2, 1));
   }
   hi *= 1.000001;
   for (int it = 0; it < 24 && hi > 1.002 * lo; it++) {
@@ -211,6 +234,29 @@ int plan_batch_slices(int count, const int* n, int ctas, int max_tiles,
 }
 
 }  // namespace mlg
+
+extern "C" mlgmres_status mlgmres_batch_plan_slices(int count, const int* n, int m, double rtol,
+                                                    long long max_iters, int ctas,
+                                                    int stream_ctas, int max_tiles, int* groups,
+                                                    int* group_ctas, int* group_of,
+                                                    int* preferred) {
+  if (count < 1 || m < 1 || !(rtol > 0.0 && rtol < 1.0) || max_iters < 1 || ctas < 1 ||
+      stream_ctas < 1 || max_tiles < 1 || !n || !groups || !group_ctas || !group_of || !preferred)
+    return MLGMRES_ERR_ARG;
+  for (int i = 0; i < count; i++)
+    if (n[i] < 1 || n[i] > 32768) return MLGMRES_ERR_ARG;
+  const mlg::SolveKind k{m, rtol, max_iters};
+  std::vector<int> gc, gof, order, sgc, sgof;
+  double span = 0.0;
+  mlg::plan_batch(2, count, n, stream_ctas, sgc, sgof, order);
+  const int G = mlg::plan_batch_slices(count, n, k, ctas, max_tiles, gc, gof, order, &span);
+  *groups = G;
+  *preferred =
+      G > 0 && mlg::slices_pay(span, mlg::stream_makespan(count, n, k, ctas, sgc, sgof)) ? 1 : 0;
+  for (int g = 0; g < G; g++) group_ctas[g] = gc[g];
+  for (int i = 0; i < count && G > 0; i++) group_of[i] = gof[i];
+  return MLGMRES_OK;
+}
 
 extern "C" mlgmres_status mlgmres_batch_plan(int dim, int count, const int* n, int ctas,
                                              int* groups, int* group_ctas, int* group_of) {

@@ -14,14 +14,23 @@ double system_cost(int dim, int n);
 int plan_batch(int dim, int count, const int* n, int ctas, std::vector<int>& group_ctas,
                std::vector<int>& group_of, std::vector<int>& order);
 
+// What the solves of a batch have in common.
+struct SolveKind {
+  int m;
+  double rtol;
+  long long max_iters;
+};
+
 // The schedule of a 2D FP32 batch whose bases stay in shared memory: group_ctas[g]
 // CTAs hold slices of at most max_tiles tiles of each of their systems.  Returns
 // the number of groups, 0 if some system does not fit; *makespan in the unit of
-// stream_makespan, which estimates a streamed schedule.
-int plan_batch_slices(int count, const int* n, int ctas, int max_tiles,
+// stream_makespan, which estimates a streamed schedule on a GPU of `sms` SMs.
+int plan_batch_slices(int count, const int* n, const SolveKind& k, int ctas, int max_tiles,
                       std::vector<int>& group_ctas, std::vector<int>& group_of,
                       std::vector<int>& order, double* makespan);
-double stream_makespan(int count, const int* n, const std::vector<int>& group_ctas,
-                       const std::vector<int>& group_of);
+double stream_makespan(int count, const int* n, const SolveKind& k, int sms,
+                       const std::vector<int>& group_ctas, const std::vector<int>& group_of);
+// Whether the slices' estimate is enough below the streamed one's.
+bool slices_pay(double slices, double stream);
 
 }  // namespace mlg
