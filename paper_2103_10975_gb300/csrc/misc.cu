@@ -85,15 +85,29 @@ __global__ void denormalise_kernel(const float* __restrict__ y, int N, const dou
 // weighted sum of the five points takes five operations instead of nine (the guess
 // 186 us instead of 218) and rounds to 9e-17: not used.
 //
+// One sweep, a thread per point.
+__global__ void jacobi_kernel(int n, const double* __restrict__ b, const double* __restrict__ xin,
+                              double* __restrict__ xout, double s2, double f) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n * n) return;
+  const int ix = i % n, iy = i / n;
+  const double c = xin[i];
+  const double l = ix > 0 ? xin[i - 1] : 0.0;
+  const double r = ix < n - 1 ? xin[i + 1] : 0.0;
+  const double d = iy > 0 ? xin[i - n] : 0.0;
+  const double t = iy < n - 1 ? xin[i + n] : 0.0;
+  const double ax = s2 * (((c - l) + (c - r)) + ((c - d) + (c - t)));
+  xout[i] = c + f * (b[i] - ax);
+}
+
 // Up to S damped-Jacobi sweeps of the 2D operator in one launch: a CTA loads its
 // TW x TH tile with a halo of S points (x and b) into shared memory and sweeps
 // there, the valid region shrinking by one point per sweep, so no sweep waits for
 // another CTA and the tile goes through L2 once per S sweeps.  The same FP64
 // operations per point whatever the tile or the number of sweeps per launch.  The halo
 // is computed redundantly ((TW + 2 (S - s)) (TH + 2 (S - s)) points in sweep s: 1.4 x
-// the tile at 32 x 16, S = 4); more sweeps per launch cost more FP64 than the launches
-// they save.  32 sweeps at 256^2: 32 launches 310 us for the whole guess, 8 launches
-// 276 (218 with what the other kernels of the guess gained later).
+// the tile at 32 x 16, S = 4).  32 sweeps at 256^2: 32 launches of one sweep 147 us, 8
+// of four 112 (the whole guess 310 -> 276, and 218 with what its other kernels gained).
 template <int TW, int TH, int S>
 __global__ void __launch_bounds__(256) jacobi_tile_kernel(int n, const double* __restrict__ b,
                                                           const double* __restrict__ xin,
@@ -238,22 +252,33 @@ cudaError_t launch_jacobi(int dim, int n, const float* kappa, const double* b, d
                           cudaStream_t s) {
   const double h = 2.0 / (n + 1);
   const double s2 = 1.0 / (h * h);
-  constexpr int S = 4;
+  // Four sweeps per launch where that saves more than the halos' FP64 work costs: up to
+  // two tiles per SM (32 sweeps, us, one per launch / four: 128^2 145 / 65, 256^2 147 /
+  // 112, 384^2 212 / 163; past that 416^2 213 / 227, 512^2 278 / 279, 1024^2 727 / 854),
+  // and not for one or two sweeps (256^2 21 / 24 and 23 / 25).
+  constexpr int S = 4, kMostTiles = 2 * 152;
+  const long long tiles = (long long)((n + 31) / 32) * ((n + 15) / 16);
+  const double f = omega / (4.0 * s2);
   double *cur = x, *oth = tmp;
-  for (int k = 0; k < sweeps; k += dim == 3 ? 1 : S) {
+  for (int k = 0; k < sweeps;) {
+    const int left = sweeps - k;
     if (dim == 3) {
       jacobi3d_kernel<<<blocks_for(n * n * n), 256, 0, s>>>(n, kappa, b, cur, oth, omega, s2);
+      k++;
+    } else if (left < 3 || tiles > kMostTiles) {
+      jacobi_kernel<<<blocks_for(n * n), 256, 0, s>>>(n, b, cur, oth, s2, f);
+      k++;
     } else {
-      const double f = omega / (4.0 * s2);
-      const int c = sweeps - k < S ? sweeps - k : S;
+      const int c = left < S ? left : S;
       // 32 x 16 tiles where they fill the GPU, else 16 x 8 (a sweep of a tile is
       // a serial FP64 chain per point; more CTAs shorten it)
-      if ((long long)((n + 31) / 32) * ((n + 15) / 16) >= 100)
+      if (tiles >= 100)
         jacobi_tile_kernel<32, 16, S><<<dim3((n + 31) / 32, (n + 15) / 16), 256, 0, s>>>(
             n, b, cur, oth, s2, f, c);
       else
         jacobi_tile_kernel<16, 8, S><<<dim3((n + 15) / 16, (n + 7) / 8), 256, 0, s>>>(
             n, b, cur, oth, s2, f, c);
+      k += c;
     }
     note_launches(1);
     double* t = cur;

@@ -63,3 +63,20 @@ def test_fp64_norm_is_the_rounded_root(at):
         e[0 if at == "corner" else 1] = 1.0
         _, H, _ = Solver(n, m=4).arnoldi(e.cuda(), 2)
         assert H[1, 0] == np.sqrt(2.0 * a if at == "corner" else 2.0 * a + a), n
+
+
+@pytest.mark.parametrize("n", [5, 33, 130, 321, 384, 390, 450])
+def test_sweeps_in_one_call_or_one_by_one(n):
+    """Several sweeps per launch (small grids), one per launch (large ones) and the
+    remainders of one or two sweeps: the same operations per point, so at most a rounding
+    or two per sweep apart if a compiler contracts them differently."""
+    from paper_2103_10975_gb300 import Solver
+    s = Solver(n, m=5, guess_omega=0.75)
+    rng = np.random.default_rng(n)
+    b = torch.as_tensor(rng.standard_normal(n * n)).cuda()
+    x0 = torch.as_tensor(rng.standard_normal(n * n)).cuda()
+    one = x0.clone()
+    for k in range(1, 12):
+        s.smooth(b, one, 1)
+        many = s.smooth(b, x0.clone(), k)
+        assert float((many - one).norm()) <= k * 2.3e-16 * float(one.norm()), k
