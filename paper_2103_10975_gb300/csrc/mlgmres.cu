@@ -91,8 +91,8 @@ int single_vsmem(const mlgmres* h, int blocks, bool compact = false) {
   return need <= budget ? (int)need : 0;
 }
 
-// Most CTAs a solve takes without leaving SMs free: a CTA holds an SM's registers, and
-// training phases run on the others beside the solves (with none free they wait for
+// The CTAs of a solve that leaves an eighth of the SMs free: a CTA holds an SM's registers,
+// and training phases run on the others beside the solves (with none free they wait for
 // the gaps between solves: at 256^2 no learned guess was taken any more).
 int beside_limit(int ctas) { return ctas - ctas / 8; }
 bool trains_beside(const mlgmres* h) {
@@ -130,6 +130,12 @@ int auto_blocks(const mlgmres* h, int N) {
   if (want < 1) want = 1;
   if (want > h->max_blocks) want = h->max_blocks;
   if (want > kPartStride) want = kPartStride;
+  // Training beside the solves: SMs are left free as long as the slices of V still fit
+  // in shared memory then (learned series from x0 = 0, ms per time step with training,
+  // all SMs / 133 CTAs: 300^2 110.6 / 108.1, 400^2 226.7 / 222.9; but 512^2, whose slices
+  // no longer fit, 353 / 546, and streamed bases 600^2 642 / 674, 700^2 939 / 994 with 266
+  // of its 304 CTAs).
+  if (want > most && single_vsmem(h, most) > 0) want = most;
   return (int)want;
 }
 
@@ -679,7 +685,8 @@ mlgmres_status mlgmres_create(const mlgmres_grid* grid, const mlgmres_options* o
     // Untuned default for a streamed FP32 basis: the compact variant (two CTAs per
     // SM) from kCompactPoints on (measured, us per step, one CTA per SM against
     // two: 520^2 m = 30 17.6 / 17.3, 640^2 22.3 / 20.7, 1024^2 46.0 / 37.5, 1500^2
-    // 91.4 / 73.3); two stages per warp where its passes are longest.  (In 3D it is
+    // 91.4 / 73.3); two stages per warp where its passes are longest.  With training
+    // beside the solves too (see auto_blocks).  (In 3D it is
     // left to the tuner: the other number of CTAs is another order of the sums, on
     // which an unconverged FP32 solve with kappa depends, see slice_budget.)
     constexpr int kCompactPoints = 400000;
