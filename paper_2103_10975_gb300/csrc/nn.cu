@@ -688,14 +688,17 @@ __global__ void __launch_bounds__(kW1Threads, 2) conv1_wgrad(
         if (ry < R) {
           win.move(sf, center + (ry + 1) * TW + xl + 1, TP, TW, next);
           next = true;
-          // (val is 0 past the grid's edge; the staged field is finite there)
+          // (a ragged segment's points past the grid's edge are no terms of the sums: 0
+          // times a neighbour that is not finite would be one)
+          if (y0 + ry < n && x0 + xl < n) {
 #pragma unroll
-          for (int d = 0; d < C; d++) {
+            for (int d = 0; d < C; d++) {
 #pragma unroll
-            for (int t = 0; t < T; t++) acc[d][t] += val[k][d] * win.template at<sgn>(t);
-            if (MODE == 1) accb[d] += val[k][d];
+              for (int t = 0; t < T; t++) acc[d][t] += val[k][d] * win.template at<sgn>(t);
+              if (MODE == 1) accb[d] += val[k][d];
+            }
+            if (MODE == 0) accb[0] += win.template at<1>(T / 2);
           }
-          if (MODE == 0 && y0 + ry < n && x0 + xl < n) accb[0] += win.template at<1>(T / 2);
         }
         if (++xl == W) {
           xl = 0;
