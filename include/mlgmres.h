@@ -76,8 +76,8 @@ enum {
 /* Problem geometry.  dim = 2 or 3; n = interior points per axis (square / cubic
  * grids); kappa_dev = n^3 cell coefficients (3D only; NULL = constant 1).  The
  * kappa array must stay valid for the handle's lifetime; it is read at the start
- * of every solve (the FP32 cycles of a single solve use face coefficients formed
- * from it then, the harmonic means in FP64 rounded once to FP32), so it may
+ * of every solve (a single solve uses face coefficients formed from it then, the
+ * harmonic means in FP64; the FP32 cycles have them rounded once to FP32), so it may
  * change between solves. */
 typedef struct {
   int dim;

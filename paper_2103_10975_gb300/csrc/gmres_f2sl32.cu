@@ -1,5 +1,5 @@
-// The FP32 2D shared-slice variant for long slices (more than two points per
-// thread), m <= 32.  Compiled on its own so the variants build in parallel.
+// The FP32 2D shared-slice variant for long slices (more than eight points per thread, in
+// batches four), m <= 32.  Compiled on its own so the variants build in parallel.
 #include "gmres_kernel.cuh"
 
 namespace mlg {

@@ -531,10 +531,10 @@ __device__ __forceinline__ void gather(const R* part, int L, int nb, double* tot
 // written and read as one, so a reader that finds the expected tag has the
 // values, and neither side waits for a fence: the release that a counter barrier
 // needs (all of the CTA's stores performed before the arrival) and its acquire
-// cost 0.36 us per exchange at 128 CTAs (two exchanges: 4.84 -> 4.12 us).
+// cost 0.4 us per exchange at 128 CTAs (two exchanges: 4.57 -> 3.77 us).
 //  - up to kDirectCtas CTAs (in a batch kDirectCtasBatch): the readers spin on the
-//    words themselves (two exchanges at 32 CTAs 3.47 us, at 8 CTAs 2.63, against 4.59
-//    and 3.87 with the counter barrier);
+//    words themselves (two exchanges at 32 CTAs 3.15 us, at 8 CTAs 2.3 to 2.8, against
+//    4.25 and 4.16 with the counter barrier);
 //  - larger groups: a relaxed counter says when everyone has arrived, and a word
 //    that is still on its way is read again (spinning on all words from all CTAs
 //    floods L2: 9.7 us at 128 CTAs);
@@ -1180,11 +1180,10 @@ __device__ __forceinline__ void warp_partials(T (*red)[LMAX],
   warp_slot<LMAX>(red, j + 1, norm);
 }
 
-// X and Y passes with the CTA's slice of V in shared memory (2D): the same
-// arithmetic as x_pass / y_pass, but a point's V column is read from shared
-// memory twice (update, then dots) instead of being held in registers, so
-// registers only carry the accumulators; U points per trip keep the
-// stencil's global loads in flight together.
+// X and Y passes with the CTA's slice of V in shared memory (2D and 3D, both
+// precisions): the same arithmetic as x_pass / y_pass, but a point's V column is
+// read from shared memory twice (update, then dots) instead of being held in
+// registers, so registers only carry the accumulators.
 // What a thread carries between the passes of the shared-slice variants for
 // its first U = 2 points: w' at each point and its 2 DIM neighbours (0 outside
 // the grid), loaded right after the Y barrier so that the loads are in flight
@@ -2136,10 +2135,9 @@ __device__ void solve_one(const KParams& kp, const SolveTask& tk, const GroupWor
   // run 1% slower from HBM)
   const int rows = in_shared(VM) ? slice_rows(sizeof(T) == 4, DIM, m) : m + 1;
   // V lives in shared memory when this CTA's slice fits the reserved space
-  // (latency of a shared load instead of an L2 round trip); else in HBM.
-  // (only the FP32 2D variant has slices small enough to be worth it; each
-  // placement of V is its own kernel variant, so every pass uses the right
-  // address space and registers are allocated per variant)
+  // (latency of a shared load instead of an L2 round trip); else in HBM.  (Each
+  // placement of V is its own kernel variant, in both precisions and dimensions, so
+  // every pass uses the right address space and registers are allocated per variant)
   const bool vshared = in_shared(VM);
   T* __restrict__ Vg = (T*)w.V;
   T* __restrict__ Vs = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(&sm) +

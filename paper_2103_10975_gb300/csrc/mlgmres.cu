@@ -69,9 +69,10 @@ unsigned long long splitmix_next(unsigned long long& st) {
 constexpr int kLongPoints = 2048, kLongPointsBatch = 1024;
 
 // Shared-memory bytes a CTA has for its slice of V.  (3D FP32: what the variant for
-// every m leaves, also for m <= kSmallM, so that 62^3 - 64^3 keep the streamed basis:
-// a few hundred FP32 steps with kappa that do not converge end up to 5e-8 apart when
-// their sums are taken in another order.)
+// every m leaves, also for m <= kSmallM.  The larger budget would change the placement,
+// and with it the order of the sums, of cubes that stream now; a few hundred FP32 steps
+// with kappa that do not converge end up to 5e-8 apart then.  Converged solves agree on
+// either side of the line.)
 int slice_budget(const mlgmres* h, int dim) {
   return gmres_vsmem_budget(h->fp32, h->fp32 && dim == 3 ? kMaxM : h->opt.m);
 }

@@ -364,7 +364,6 @@ __global__ void __launch_bounds__(256) loss_finish(const float* __restrict__ par
   }
 }
 
-// g_t[p][c] = sum_tap w[c][tap] gy[p - off_tap]
 // Segments of the 1-channel <-> 32-channel kernels: R rows x W points of one
 // (b, z) plane (W = min(n, 256), R = max(1, 256 / n)), with the 1-channel field
 // of the segment and its one-point halo staged in shared memory, zero outside
@@ -756,10 +755,11 @@ __global__ void mask_to_bf16(long long count, const float* __restrict__ g,
 // here so the parameters keep the documented order (T taps).
 //   kind 0 (32->32): part index (tap*32 + k)*32 + o  -> param (o*32 + k)*T + tap; bias 1024 T + o
 //   kind 1/2 (1-ch): part index c*T + tap (+ 32 T + c bias) -> same order
-// One launch for all convolutions of the network (one per convolution cost 5 us
-// each, mostly latency).  With the coarse levels' convolutions and the pooling
-// levels in shared launches, and the upsampling's tables: 1245 -> 1120 us at 256^2 x
-// 8, the learned guess at 256^2 272 -> 221 us: job k's outputs on the CTAs first[k] .. first[k+1]-1.
+// One launch for all convolutions of the network: job k's outputs on the CTAs
+// first[k] .. first[k+1]-1 (one launch per convolution cost 5 us each, mostly
+// latency; with the coarse levels' convolutions and the pooling levels in shared
+// launches, and the upsampling's tables: 1245 -> 1120 us at 256^2 x 8, the learned
+// guess at 256^2 272 -> 221 us).
 struct ReduceJob {
   const float* part;
   float *gw, *gb;
@@ -1261,8 +1261,8 @@ cudaError_t net_create(Net& net, int n, int bmax, unsigned long long seed, int d
   NN_CK(cudaGetDevice(&dev));
   NN_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   net.wparts = 2 * nsm;
-  // the 1-channel weight gradients take more than the default 48 KB of
-  // dynamic shared memory in 3D (their fixed-order reduction buffer)
+  // the output convolution's tile takes more than the default 48 KB of dynamic shared
+  // memory in 3D (here only: the inference copy of a network is made after it)
   if (dim == 3) {
     NN_CK(cudaFuncSetAttribute(conv_out_fwd<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                OutTile<3>::kSmem));

@@ -750,13 +750,15 @@ bool pack_geometry(int dim, int H, int dil, bool wgrad, TcPack* pk, int* smem) {
 enum { kTcNone = 0, kTcRows = 1, kTcPacked = 2 };
 
 // Which tcgen05 tiles a job takes.  Rows of 128 points and more: a tile per row
-// segment.  Shorter ones: packed tiles where they fit shared memory (3D rows of 53
-// points and more at dilation 2 do not: a tile per row, still ahead of mma.sync when a
-// third full).  In
-// 2D, levels of little work stay on the mma.sync kernel, whose levels share one
-// launch (256^2 x 8: the 64-point level and below); a launch of their own costs
-// each of them more than the tensor cores save.  Measured at 48^3 x 2 (forward and
-// backward of the network): mma.sync 2.14 ms, a tile per row 1.54, packed 1.13.
+// segment.  Shorter ones: packed tiles where both the convolution and its weight
+// gradient fit shared memory -- in 3D rows up to 89 points (dilation 1) and 53 (dilation
+// 2), in 2D up to 118 and 116 -- else a tile per row, still ahead of mma.sync when a
+// third full.  Measured at 48^3 x 2 (forward and backward of the network): mma.sync 2.14
+// ms, a tile per row 1.54, packed 1.13.  In 2D, levels of little work stay on the
+// mma.sync kernel, whose levels share one launch; a launch of their own costs each of
+// them more than the tensor cores save (gradients at 256^2 x 8, us: 1 012 with this line,
+// 1 074 with every level packed, 1 022 with none; learned guess at 256^2 115, 136, 116, at
+// 110^2 82, 102, 82).
 int tc_kind(int dim, int B, int H, int dil) {
   if (dim != 2 && dim != 3) return kTcNone;
   if (H >= tc_min_row()) return kTcRows;
